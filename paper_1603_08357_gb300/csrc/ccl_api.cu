@@ -27,7 +27,7 @@ namespace {
 struct TuneChoice {
     int threads = 256;
     int ctas_per_sm = 0;
-    int pre_analysis = 1;
+    int pre_analysis = -1;  // step (ii): 1 run, 0 skip; -1 (never set) the library's choice: skip
     int link_mode = 0;
     int refill = 1;         // step (iii): 1 static per-lane pairs, 0 in-order hand-out
     int ana_seq = 1;        // steps (ii)/(iv): 1 contiguous ranges per warp, 0 interleaved
@@ -378,9 +378,19 @@ bool resolve_park(const ccl_context *ctx, const TuneChoice &tc, const Params &P)
     return tc.ana_park >= 0 ? tc.ana_park != 0 : labels_fit_l2(ctx, P);
 }
 
+// Whether step (ii) runs as a pass of its own: as set, else not. Steps (i) and
+// (iii) do without it (the band shortcut and the in-window jump of step (i)
+// leave short chains, and step (iii)'s search is bounded by the window's
+// slowest pair, not by the mean chain), and step (iv) repeats its work: on one
+// GB300 a call with / without it took 356 / 313 us (triangle 4096^2 at p_c),
+// 1105 / 910 us (Bethe lattice, 24 shells, random numbering), 5.73 / 5.05 ms
+// (triangle 16384^2), 11.3 / 9.9 ms (1024 mixed instances) and 30.2 / 30.6 us
+// (honeycomb 64^2).
+bool resolve_pre(const TuneChoice &tc) { return tc.pre_analysis > 0; }
+
 // Records in the context's statistics the settings a call runs with.
 void note_settings(ccl_context *ctx, const TuneChoice &tc, const Params &P) {
-    ctx->last.pre_analysis = tc.pre_analysis;
+    ctx->last.pre_analysis = resolve_pre(tc) ? 1 : 0;
     ctx->last.link_mode = tc.link_mode;
     ctx->last.refill = tc.refill;
     ctx->last.analysis_order = tc.ana_seq;
@@ -422,7 +432,7 @@ ccl_status enqueue_tail(ccl_context *ctx, const Params &P0, bool batched, const 
             else k_analysis<false, false><<<g, T, 0, s>>>(P);
         }
     };
-    if (tc.pre_analysis) {
+    if (resolve_pre(tc)) {
         analysis();
         CCL_CUDA(cudaGetLastError());
     }
@@ -854,7 +864,7 @@ ccl_status ccl_context_create(ccl_context **out, int device) {
                 const int nf = sscanf(line, "%lld %d %d %d %d %d %d %d %d %d", &cls, &a, &b, &c, &d, &r, &q, &w, &g, &k);
                 if (nf != 7 && nf != 10) continue;
                 TuneChoice t;
-                t.threads = a; t.ctas_per_sm = b < 0 ? 0 : b; t.pre_analysis = c ? 1 : 0;
+                t.threads = a; t.ctas_per_sm = b < 0 ? 0 : b; t.pre_analysis = c > 0 ? 1 : 0;
                 t.link_mode = d ? 1 : 0; t.refill = r ? 1 : 0; t.ana_seq = q ? 1 : 0;
                 t.red_window = (w >= 64 && w <= 65536) ? w : 0;
                 t.ana_group = g >= 0 ? g : -1;
@@ -949,7 +959,7 @@ ccl_status ccl_set_option(ccl_context *ctx, int option, int64_t value) {
 ccl_status ccl_get_option(ccl_context *ctx, int option, int64_t *value) {
     if (!ctx || !value) return CCL_ERR_INVALID_ARGUMENT;
     switch (option) {
-        case CCL_OPT_PRE_ANALYSIS: *value = ctx->opt.pre_analysis; break;
+        case CCL_OPT_PRE_ANALYSIS: *value = ctx->opt.pre_analysis != 0; break;
         case CCL_OPT_BLOCK_THREADS: *value = ctx->opt.threads; break;
         case CCL_OPT_USE_GRAPHS: *value = ctx->use_graphs; break;
         case CCL_OPT_PROFILE: *value = ctx->profile; break;

@@ -148,7 +148,6 @@ extern "C" ccl_status ccl_label_noalloc(int32_t n, int64_t nnz, const int32_t *r
     cudaError_t e = cudaMemsetAsync(d->scratch, 0, kOffBand + sizeof(BandRec) * (size_t)g_init, s);
     if (e == cudaSuccess) {
         k_init<false><<<(unsigned)g_init, kInitThreads, kInitSmem, s>>>(P);
-        k_analysis<false, true><<<(unsigned)g_ana, 256, 0, s>>>(P);
         k_reduce<false, true><<<(unsigned)g_red, 256, 0, s>>>(P);
         k_analysis<false, true><<<(unsigned)g_ana, 256, 0, s>>>(P);
         e = cudaGetLastError();
