@@ -459,8 +459,9 @@ ccl_status enqueue_steps(ccl_context *ctx, const Params &P0, bool batched, const
     Params P = P0;
     const int64_t g_init = init_grid(ctx, P, batched, kMaxBands);
     P.n_bands = (int32_t)g_init;
+#ifdef CCL_DEVICE_STATS
     CCL_CUDA(cudaMemsetAsync(P.counters, 0, 4 * sizeof(unsigned long long), s));
-    CCL_CUDA(cudaMemsetAsync(P.band, 0, (size_t)g_init * sizeof(BandRec), s));
+#endif
     if (profile) CCL_CUDA(cudaEventRecord(ctx->ev[0], s));
     ccl_status st = launch_init(P, batched, g_init, s);
     if (st != CCL_OK) return st;
@@ -1308,7 +1309,6 @@ ccl_status label_host_parts(ccl_context *ctx, int32_t n, int64_t nnz, const int3
     ctx->last.n_inst = 1;
     ctx->last.used_graph = 0;
     CCL_CUDA(cudaMemsetAsync(P.counters, 0, 4 * sizeof(unsigned long long), s));
-    CCL_CUDA(cudaMemsetAsync(P.band, 0, (size_t)kMaxBands * sizeof(BandRec), s));
     // the uploads may not overwrite the buffers before earlier work on s is done
     CCL_CUDA(cudaEventRecord(ctx->part_ev[kHostParts], s));
     CCL_CUDA(cudaStreamWaitEvent(ctx->copy_stream, ctx->part_ev[kHostParts], 0));
@@ -1514,9 +1514,8 @@ ccl_status ccl_label_batched_host(ccl_context *ctx, int32_t K, const int64_t *si
         } else {
             P.one = tg[0];
         }
-        if (cudaMemsetAsync(P.band, 0, (size_t)kMaxBands * sizeof(BandRec), s) != cudaSuccess ||
-            cudaStreamWaitEvent(s, ctx->bh_up[part], 0) != cudaSuccess)
-            return fail(CCL_ERR_CUDA);
+        P.more_pairs = 1;
+        if (cudaStreamWaitEvent(s, ctx->bh_up[part], 0) != cudaSuccess) return fail(CCL_ERR_CUDA);
         P.tile_off = 0;
         P.n_tiles = t1 - t0;
         P.band_off = 0;

@@ -54,14 +54,13 @@ __device__ __forceinline__ int32_t dense_label(const Params &P, int32_t i, int32
 // Appends the warp's residual pairs (r of them at this lane) to the band's
 // part of the queue: returns this lane's first slot.
 __device__ __forceinline__ int64_t dense_emit_slot(int64_t qband, unsigned long long *band_cnt, int lane,
-                                                   int r, unsigned long long &my_pairs) {
+                                                   int r) {
     const int incl = warp_incl_scan(r, lane);
     const int total = __shfl_sync(kFull, incl, 31);
     unsigned long long base = 0;
     if (total) {
         if (lane == 0) base = atomicAdd(band_cnt, (unsigned long long)total);
         base = __shfl_sync(kFull, base, 0);
-        if (lane == 0) my_pairs += (unsigned long long)total;
     }
     return qband + (int64_t)base + (incl - r);
 }
@@ -83,7 +82,6 @@ __global__ void __launch_bounds__(kDenseThreads) k_init_dense(Params P) {
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
-    unsigned long long my_pairs = 0;
     bool bad = false;
     for (int64_t t0 = s_lo; t0 < s_hi; t0 += kDenseSpan) {
         if (W <= kRowRegs) {
@@ -137,7 +135,7 @@ __global__ void __launch_bounds__(kDenseThreads) k_init_dense(Params P) {
                 const int cnt = __popc(lowmask);
                 if (i64 < s_hi) P.one.labels[i] = dense_label(P, i, m, cnt, s_lo, t0);
                 const int r = cnt > 1 ? cnt - 1 : 0;
-                int64_t slot = dense_emit_slot(qband, &band_cnt, lane, r, my_pairs);
+                int64_t slot = dense_emit_slot(qband, &band_cnt, lane, r);
                 if (r > 0) {
                     const uint32_t rm = lowmask & ~(1u << mk);
 #pragma unroll
@@ -166,7 +164,7 @@ __global__ void __launch_bounds__(kDenseThreads) k_init_dense(Params P) {
                     P.one.labels[i] = dense_label(P, i, m, cnt, s_lo, t0);
                 }
                 const int r = cnt > 1 ? cnt - 1 : 0;
-                int64_t slot = dense_emit_slot(qband, &band_cnt, lane, r, my_pairs);
+                int64_t slot = dense_emit_slot(qband, &band_cnt, lane, r);
                 if (r > 0) {
                     for (int k = 0; k < W; ++k) {
                         const int64_t e = i64 + (int64_t)k * n;
@@ -179,10 +177,7 @@ __global__ void __launch_bounds__(kDenseThreads) k_init_dense(Params P) {
         __syncthreads();        // this step's labels become visible to the CTA's next steps
     }
     if (bad) raise_err(P.err, kErrIndex);
-    if (lane == 0 && my_pairs) {
-        atomicAdd(P.counters, my_pairs);
-        atomicAdd(&P.band[P.band_off + blockIdx.x].cnt, my_pairs);
-    }
+    if (threadIdx.x == 0) P.band[P.band_off + blockIdx.x].cnt = band_cnt;      // (after the last step's barrier)
 }
 
 // ---------------------------------------------------------------------------
@@ -457,7 +452,6 @@ __global__ void __launch_bounds__(kInitThreads, 2) k_init_dense_tma(Params P) {
         if (lane == 0) dense_produce<kGen>(P, st, full, empty);
         return;
     }
-    unsigned long long my_pairs = 0;
     int64_t band_lo, band_hi;
     cta_band(P, band_lo, band_hi);
     int64_t t_local = 0;
@@ -494,7 +488,6 @@ __global__ void __launch_bounds__(kInitThreads, 2) k_init_dense_tma(Params P) {
             unsigned long long base = 0;
             if (lane == 0) base = atomicAdd(&band_cnt, (unsigned long long)total);
             base = __shfl_sync(kFull, base, 0);
-            if (lane == 0) my_pairs += (unsigned long long)total;
             const int64_t slot = S.h.qband + (int64_t)base + (incl - rr);
             if (c0.r > 0) dense_emit_chunk<kGen>(P, S, c0, tc.staged, slot);
             if (c1.r > 0) dense_emit_chunk<kGen>(P, S, c1, tc.staged, slot + c0.r);
@@ -502,10 +495,8 @@ __global__ void __launch_bounds__(kInitThreads, 2) k_init_dense_tma(Params P) {
         __syncwarp();
         if (lane == 0) mbar_arrive(&empty[s]);
     }
-    if (lane == 0 && my_pairs) {
-        atomicAdd(P.counters, my_pairs);
-        atomicAdd(&P.band[P.band_off + blockIdx.x].cnt, my_pairs);
-    }
+    consumers_sync<32 * kInitConsumers>();
+    if (threadIdx.x == 0) P.band[P.band_off + blockIdx.x].cnt = band_cnt;
 }
 
 }  // namespace ccl

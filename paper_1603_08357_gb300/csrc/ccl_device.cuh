@@ -135,6 +135,12 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
     return ok != 0;
 }
 
+// barrier of the first kThreads threads of the CTA
+template <int kThreads>
+__device__ __forceinline__ void consumers_sync() {
+    asm volatile("bar.sync 1, %0;" ::"n"(kThreads) : "memory");
+}
+
 // Waits for the phase of `parity` to complete; gives up after a bounded
 // number of polls (each poll itself suspends for a hardware-bounded time).
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity) {
@@ -599,7 +605,6 @@ __global__ void __launch_bounds__(kInitThreads, 2) k_init(Params P) {
         if (lane == 0) init_produce<kBatched, kGen>(P, st, full, empty);
         return;
     }
-    unsigned long long my_pairs = 0;
     int64_t band_lo, band_hi;
     cta_band(P, band_lo, band_hi);
     // stage s = tl % kStages and phase parity (tl / kStages) & 1 of local tile
@@ -645,7 +650,6 @@ __global__ void __launch_bounds__(kInitThreads, 2) k_init(Params P) {
             if (has0 && c0.i < I.n) I.labels[c0.i] = c0.lab;
             if (has1 && c1.i < I.n) I.labels[c1.i] = c1.lab;
             if (total > 0) {
-                if (lane == 0) my_pairs += (unsigned long long)total;
                 const int64_t slot = S.h.qband + (int64_t)base + (incl - rr);
                 if (c0.fast && c1.fast) {
                     init_emit_pair<kBatched>(P, S, th, c0, c1, slot, rr);
@@ -658,10 +662,10 @@ __global__ void __launch_bounds__(kInitThreads, 2) k_init(Params P) {
         __syncwarp();
         if (lane == 0) mbar_arrive(&empty[s]);
     }
-    if (lane == 0 && my_pairs) {
-        atomicAdd(P.counters, my_pairs);
-        atomicAdd(&P.band[P.band_off + blockIdx.x].cnt, my_pairs);
-    }
+    // the band's pair count, once every consumer warp has added its own (the
+    // producer warp may have returned)
+    consumers_sync<32 * kInitConsumers>();
+    if (threadIdx.x == 0) P.band[P.band_off + blockIdx.x].cnt = band_cnt;
 }
 
 // ---------------------------------------------------------------------------
@@ -934,6 +938,11 @@ __global__ void __launch_bounds__(256) k_reduce(Params P) {
     }
     __syncthreads();
     const long long total = s_pref[P.n_bands];
+    // the call's statistics (a call in parts adds its later parts' pairs)
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (P.more_pairs) P.counters[0] += (unsigned long long)total;
+        else P.counters[0] = (unsigned long long)total;
+    }
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
     const long long nwarps = (long long)gridDim.x * (blockDim.x >> 5);

@@ -143,9 +143,9 @@ extern "C" ccl_status ccl_label_noalloc(int32_t n, int64_t nnz, const int32_t *r
     const int64_t g_ana = std::max<int64_t>(1, std::min<int64_t>((int64_t)d->num_sms * d->ana_per_sm, (ana_warps + 7) / 8));
     const int64_t g_red = (int64_t)d->num_sms * d->red_per_sm;
 
-    // the array keeps the previous call's contents: clear the error word, the
-    // counters and the band records that must start at zero
-    cudaError_t e = cudaMemsetAsync(d->scratch, 0, kOffBand + sizeof(BandRec) * (size_t)g_init, s);
+    // the array keeps the previous call's contents: clear the error word (step
+    // (i) writes every band record, step (iii) the pair count)
+    cudaError_t e = cudaMemsetAsync(d->scratch + kOffErr, 0, sizeof(unsigned), s);
     if (e == cudaSuccess) {
         k_init<false><<<(unsigned)g_init, kInitThreads, kInitSmem, s>>>(P);
         k_reduce<false, true><<<(unsigned)g_red, 256, 0, s>>>(P);

@@ -92,6 +92,7 @@ struct Params {
     int64_t nn_width;          // slots per site of the dense list
     int64_t tile_off;          // step (i) on part of the tiles: its first tile ...
     int32_t band_off;          // ... and its first band record
+    int32_t more_pairs;        // 1: the pairs of this step (iii) add to counters[0], 0: they replace it
     int32_t iter_cap;          // > 0: steps (ii)-(iv) give up after this many iterations (test option)
     int32_t red_window;        // step (iii): most pairs per warp window (0: kRedWindowMax)
     int32_t ana_group;         // steps (ii)/(iv), contiguous order: > 0 visit the sites in super-chunks
