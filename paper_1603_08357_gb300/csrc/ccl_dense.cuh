@@ -431,7 +431,7 @@ __device__ __forceinline__ void dense_emit_chunk(const Params &P, const DenseSta
 }
 
 template <bool kGen>
-__global__ void __launch_bounds__(kInitThreads, 2) k_init_dense_tma(Params P) {
+__global__ void __launch_bounds__(kDenseTmaThreads, 2) k_init_dense_tma(Params P) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     uint64_t *full = reinterpret_cast<uint64_t *>(smem_raw);
     uint64_t *empty = full + kStages;
@@ -441,14 +441,14 @@ __global__ void __launch_bounds__(kInitThreads, 2) k_init_dense_tma(Params P) {
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
             mbar_init(&full[s], 1);
-            mbar_init(&empty[s], kInitConsumers);
+            mbar_init(&empty[s], kDenseConsumers);
         }
         mbar_fence_init();
     }
     __shared__ unsigned long long band_cnt;
     if (threadIdx.x == 0) band_cnt = 0;
     __syncthreads();
-    if (warp == kInitConsumers) {
+    if (warp == kDenseConsumers) {
         if (lane == 0) dense_produce<kGen>(P, st, full, empty);
         return;
     }
@@ -495,7 +495,7 @@ __global__ void __launch_bounds__(kInitThreads, 2) k_init_dense_tma(Params P) {
         __syncwarp();
         if (lane == 0) mbar_arrive(&empty[s]);
     }
-    consumers_sync<32 * kInitConsumers>();
+    consumers_sync<32 * kDenseConsumers>();
     if (threadIdx.x == 0) P.band[P.band_off + blockIdx.x].cnt = band_cnt;
 }
 

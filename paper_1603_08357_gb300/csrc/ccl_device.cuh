@@ -7,10 +7,10 @@
 //  * Step (i) streams the CSR input: per CTA one producer warp moves each
 //    tile's row pointers, column indices and bit words into shared memory with
 //    bulk asynchronous copies (cp.async.bulk, completion on mbarriers, a ring
-//    of kStages stages); kInitConsumers consumer warps scan the rows (two
-//    chunks per warp and tile, interleaved), write the labels and append the
-//    residual pairs to their CTA's part of the queue through one prefix sum
-//    per warp and tile. Each CTA owns a contiguous band of tiles; a site whose
+//    of kStages stages); kInitConsumers consumer warps scan the rows (four
+//    chunks per warp and tile, one row of each per lane, interleaved), write
+//    the labels and append the residual pairs to their CTA's part of the
+//    queue through one prefix sum per warp and tile. Each CTA owns a contiguous band of tiles; a site whose
 //    smallest lower neighbour lies in a band tile finished kStages tiles
 //    earlier takes that neighbour's label (most of step (ii) on lattices).
 //  * Step (iii) runs Algorithm 1 over the queue: each warp drains a window of
@@ -416,8 +416,8 @@ __device__ __forceinline__ void init_scan_chunk(const Params &P, const Stage &S,
         scan_row_general<kGen>(P, S, I, a, a_next, i, m, mk, cnt, bad);
     }
     if (bad) raise_err(P.err, kErrIndex);
-    // the label; the caller stores it after scanning its other chunk, so the
-    // shortcut's load below has that scan's time to arrive
+    // the label; the caller stores it after scanning its other chunks, so the
+    // shortcut's load below has their scans' time to arrive
     int32_t lab = cnt ? m : i;
     if (cnt) {
         const int32_t mt = (int32_t)((uint32_t)m / kTileSites);
@@ -433,92 +433,174 @@ __device__ __forceinline__ void init_scan_chunk(const Params &P, const Stage &S,
     cr.r = cnt > 1 ? cnt - 1 : 0;
 }
 
-// Both chunks of a consumer warp at once, when every row of both is short and
-// staged (the common case): the two rows of a lane are scanned in one loop,
-// so their shared-memory loads and dependent arithmetic interleave. Returns
-// false (having done nothing) otherwise.
-template <bool kBatched, bool kGen = false>
-__device__ __forceinline__ bool init_scan_pair(const Params &P, const Stage &S, const Inst &I, int cc0,
-                                               int lane, const TileCtx &tc, const TileHdr &h, ChunkRes &c0,
-                                               ChunkRes &c1) {
-    const int32_t n = I.n;
-    const int32_t s00 = h.s0 + cc0 * kChunk;
-    if (!tc.staged || s00 + 2 * kChunk > n || s00 < h.rp_lo || s00 + 2 * kChunk >= h.rp_hi) return false;
-    const int32_t i0 = s00 + lane, i1 = i0 + kChunk;
-    const int32_t *rp = S.rp + (s00 - h.rp_lo);
-    int32_t a0 = rp[lane], b0 = rp[lane + 1], a1 = rp[lane + kChunk], b1 = rp[lane + kChunk + 1];
-    const bool ok0 = a0 >= h.e0 && a0 <= b0 && b0 <= h.e1, ok1 = a1 >= h.e0 && a1 <= b1 && b1 <= h.e1;
-    const int32_t d0 = b0 - a0, d1 = b1 - a1;
-    const int32_t dmax = __reduce_max_sync(kFull, (uint32_t)max(ok0 ? d0 : 0, ok1 ? d1 : 0));
-    if (!__all_sync(kFull, ok0 && ok1) || dmax > kRowRegs) return false;
-    const int32_t *col0 = S.ci + (a0 - h.ci_lo), *col1 = S.ci + (a1 - h.ci_lo);
-    uint32_t w0 = 0, w1 = 0;
-    if (!kGen) {
-        const int32_t r0 = tc.rb0 + a0, r1 = tc.rb0 + a1;
-        if (d0 > 0) w0 = __funnelshift_r(S.bw[r0 >> 5], S.bw[(r0 + d0 - 1) >> 5], (uint32_t)r0 & 31u);
-        if (d1 > 0) w1 = __funnelshift_r(S.bw[r1 >> 5], S.bw[(r1 + d1 - 1) >> 5], (uint32_t)r1 & 31u);
-    }
-    int32_t m0 = INT32_MAX, m1 = INT32_MAX, k0 = -1, k1 = -1;
-    uint32_t l0 = 0, l1 = 0, jmax = 0;
+// The four rows of a lane on the register path.
+struct RowsRes {
+    int32_t lab[kRows];     // labels to store (may be loads still in flight)
+    int32_t off[kRows];     // stage index of each row's first column
+    uint32_t res;           // residual entries: entry t of row k at bit 8 k + last - t
+    int32_t last;
+};
+
+// Scans four rows per lane, rows s00 + 32 k + lane. kD > 0: every row has kD
+// entries; kD = 0: row k has d[k] <= kRowRegs entries, dmax the longest of the
+// warp. The rows are interleaved, so their loads and dependent arithmetic
+// overlap.
+//
+// Step (i) is bound by the instructions of this scan (the integer pipe), not
+// by memory, until rows are cheap. Four rows a lane with eight warps a CTA
+// against two rows with sixteen: the tile's header, the prefix sum and the
+// queue bookkeeping are paid once for 128 sites instead of 64; rows of one
+// degree need no row ends, no per-entry tests of the row's length and half
+// the loads (the rows of a lane lie 32 apart, so 8-byte loads of degree 4 and
+// 6 and 4-byte loads of degree 3 spread over the banks); keys find the
+// smallest neighbour and its place with one minimum. Warp instructions per 64
+// sites on triangle 3000^2: 537 -> 308. Times of step (i), before -> after:
+// triangle 4096^2 160 -> 118 us (4.6 TB/s; streaming alone takes 88),
+// triangle 16384^2 2.44 -> 1.83 ms, honeycomb 2048^2 71 -> 55 us, Bethe
+// lattice of 24 shells 390 -> 364 us, 1024 mixed instances 4.98 -> 4.80 ms.
+// (Two rows a lane and sixteen warps with the same scan: 140 us on triangle
+// 4096^2; two stages and three CTAs per SM: 124 us there, 347 us on the Bethe
+// lattice.) A call of few tiles pays for the longer lanes: honeycomb 64^2
+// 8.4 -> 9.5 us.
+template <bool kGen, int kD, bool kWide = false>
+__device__ __forceinline__ void scan_rows(const Params &P, const Stage &S, const TileCtx &tc, const TileHdr &h,
+                                          int32_t n, int32_t s00, int lane, const int32_t (&a)[kRows],
+                                          const int32_t (&d)[kRows], int32_t dmax, RowsRes &q, bool &bad) {
+    const int32_t *col[kRows];
+    uint32_t w[kRows], low[kRows];
+    int32_t m[kRows];
+    uint32_t jmax = 0;
 #pragma unroll
-    for (int t = 0; t < kRowRegs; ++t) {
-        if (t >= dmax) break;
-        if (t < d0) {
-            const int32_t j = col0[t];
-            jmax = max(jmax, (uint32_t)j);
-            const bool open = kGen ? ((uint32_t)j < (uint32_t)i0 &&
-                                      gen_bond_open(P.gen_seed, P.gen_thr, (uint32_t)j, (uint32_t)i0))
-                                   : ((w0 >> t) & 1u) != 0;
-            if (open && (uint32_t)j < (uint32_t)i0) {
-                l0 |= 1u << t;
-                if (j < m0) { m0 = j; k0 = t; }
-            }
-        }
-        if (t < d1) {
-            const int32_t j = col1[t];
-            jmax = max(jmax, (uint32_t)j);
-            const bool open = kGen ? ((uint32_t)j < (uint32_t)i1 &&
-                                      gen_bond_open(P.gen_seed, P.gen_thr, (uint32_t)j, (uint32_t)i1))
-                                   : ((w1 >> t) & 1u) != 0;
-            if (open && (uint32_t)j < (uint32_t)i1) {
-                l1 |= 1u << t;
-                if (j < m1) { m1 = j; k1 = t; }
-            }
+    for (int k = 0; k < kRows; ++k) {
+        q.off[k] = a[k] - h.ci_lo;
+        col[k] = S.ci + q.off[k];
+        low[k] = 0;
+        m[k] = INT32_MAX;
+        w[k] = 0;
+        if (!kGen) {
+            const int32_t rel = tc.rb0 + a[k];
+            const uint32_t *bw = S.bw + (rel >> 5);
+            // (an empty row's may lie past the copied words)
+            if (kD > 0 || d[k] > 0) w[k] = __funnelshift_r(bw[0], bw[1], (uint32_t)rel & 31u) & 0xffu;
         }
     }
-    if (jmax >= (uint32_t)n) raise_err(P.err, kErrIndex);
-    const int n0 = __popc(l0), n1 = __popc(l1);
-    int32_t lab0 = n0 ? m0 : i0, lab1 = n1 ? m1 : i1;
-    // One pointer jump inside the warp's window of 64 sites [s00, s00 + 64):
-    // a label that points to a window site takes that site's label. The value
-    // taken is an ancestor of the site, so it stays a valid label, and a chain
-    // along a lattice row shortens by half before step (iii) and the analysis
-    // follow it. (A chunk-0 label lies below its site, so inside the window it
-    // points into chunk 0; a chunk-1 label may point into either chunk.) One
-    // jump measured faster end to end than jumping until the window is
-    // settled: the later rounds cost step (i) more than they save afterwards.
-    if (__any_sync(kFull, (uint32_t)(lab0 - s00) < 64u || (uint32_t)(lab1 - s00) < 64u)) {
-        const uint32_t w0 = (uint32_t)(lab0 - s00), w1 = (uint32_t)(lab1 - s00);
-        const int32_t a0v = __shfl_sync(kFull, lab0, (int)(w0 & 31u));
-        const int32_t a1v = __shfl_sync(kFull, lab0, (int)(w1 & 31u));
-        const int32_t b1v = __shfl_sync(kFull, lab1, (int)(w1 & 31u));
-        if (w0 < 32u) lab0 = a0v;
-        if (w1 < 64u) lab1 = w1 < 32u ? a1v : b1v;
+    // Open entries as keys 8 j + t (closed ones above every site's): the
+    // smallest key is the smallest open neighbour and its place, and entry t
+    // is an open lower one iff its key is below 8 i. The signs of the keys'
+    // differences to 8 i collect in `low`, entry t of T at bit T - 1 - t.
+    // Keys need sites below 2^28; kWide keeps the neighbour and its place apart.
+    auto entry = [&](int k, int t, int32_t j) {
+        const int32_t i = s00 + kChunk * k + lane;
+        jmax = max(jmax, (uint32_t)j);
+        bool open = kGen || ((w[k] >> t) & 1u);
+        if (kGen) open = (uint32_t)j < (uint32_t)i && gen_bond_open(P.gen_seed, P.gen_thr, (uint32_t)j, (uint32_t)i);
+        if (kWide) {
+            const bool lower = open && (uint32_t)j < (uint32_t)i;
+            low[k] = 2u * low[k] + (lower ? 1u : 0u);
+            if (lower && j < m[k]) { m[k] = j; w[k] = (w[k] & 0xffu) | ((uint32_t)t << 8); }
+        } else {
+            const int32_t key = open ? (int32_t)(8u * (uint32_t)j + (uint32_t)t) : INT32_MAX;
+            m[k] = min(m[k], key);
+            low[k] = __funnelshift_l((uint32_t)key - 8u * (uint32_t)i, low[k], 1);
+        }
+    };
+    if (kD > 0 && kD % 2 == 0) {
+        // the rows start at even stage indices: two columns per load
+#pragma unroll
+        for (int t = 0; t < kD; t += 2)
+#pragma unroll
+            for (int k = 0; k < kRows; ++k) {
+                const int2 jj = *reinterpret_cast<const int2 *>(col[k] + t);
+                entry(k, t, jj.x);
+                entry(k, t + 1, jj.y);
+            }
+    } else if (kD > 0) {
+#pragma unroll
+        for (int t = 0; t < kD; ++t)
+#pragma unroll
+            for (int k = 0; k < kRows; ++k) entry(k, t, col[k][t]);
+    } else {
+#pragma unroll
+        for (int t = 0; t < kRowRegs; ++t) {
+            if (t >= dmax) break;
+#pragma unroll
+            for (int k = 0; k < kRows; ++k)
+                if (t < d[k]) entry(k, t, col[k][t]);
+                else low[k] <<= 1;
+        }
     }
-    // a label before the window in a tile of this band finished kStages tiles
-    // ago: take that site's label (the band shortcut)
-    if (lab0 < s00) {
-        const int32_t mt = (int32_t)((uint32_t)lab0 / kTileSites);
-        if (mt >= tc.vis_lo && mt <= tc.vis_hi) lab0 = __ldcg(I.labels + lab0);
+    bad = jmax >= (uint32_t)n;
+    q.res = 0;
+    q.last = (kD > 0 ? kD : dmax) - 1;
+#pragma unroll
+    for (int k = 0; k < kRows; ++k) {
+        // (no label comes from a row of a lane that saw a column out of range)
+        const bool any = low[k] != 0 && !bad;
+        const int at = kWide ? (int)(w[k] >> 8) : m[k] & 7;      // place of the smallest
+        q.lab[k] = any ? (kWide ? m[k] : m[k] >> 3) : s00 + kChunk * k + lane;
+        if (any) q.res |= (low[k] & ~(1u << (q.last - at))) << (8 * k);
     }
-    if (lab1 < s00) {
-        const int32_t mt = (int32_t)((uint32_t)lab1 / kTileSites);
-        if (mt >= tc.vis_lo && mt <= tc.vis_hi) lab1 = __ldcg(I.labels + lab1);
+}
+
+// The four chunks of a consumer warp at once, when all their rows exist, are
+// short and staged (the common case). Returns false (having done nothing)
+// otherwise.
+template <bool kGen>
+__device__ __forceinline__ bool init_scan_rows(const Params &P, const Stage &S, const Inst &I, int32_t s00, int lane,
+                                               const TileCtx &tc, const TileHdr &h, RowsRes &q) {
+    const int32_t n = I.n;
+    if (!tc.staged || s00 + kRows * kChunk > n || s00 < h.rp_lo || s00 + kRows * kChunk >= h.rp_hi) return false;
+    const int32_t *rp = S.rp + (s00 - h.rp_lo);
+    int32_t a[kRows], d[kRows];
+#pragma unroll
+    for (int k = 0; k < kRows; ++k) a[k] = rp[lane + kChunk * k];
+    // rows of one degree D throughout (a lattice): a[k] = first + D * (lane + 32 k)
+    const int32_t first = __shfl_sync(kFull, a[0], 0);
+    const uint32_t D = (uint32_t)__shfl_sync(kFull, a[0], 1) - (uint32_t)first;
+    const int32_t last = rp[kRows * kChunk];
+    uint32_t x = (uint32_t)a[0] - (uint32_t)first - D * (uint32_t)lane;
+#pragma unroll
+    for (int k = 1; k < kRows; ++k) x |= (uint32_t)a[k] - (uint32_t)a[k - 1] - kChunk * D;
+    x |= (uint32_t)last - (uint32_t)first - kRows * kChunk * D;
+    const bool one_degree = __all_sync(kFull, x == 0) && first >= h.e0 && last <= h.e1;
+    const bool wide = n > (1 << 28);
+    bool bad = false;
+    if (one_degree && !wide && D == 3) {
+        scan_rows<kGen, 3>(P, S, tc, h, n, s00, lane, a, d, 3, q, bad);
+    } else if (one_degree && !wide && D == 6 && ((first - h.ci_lo) & 1) == 0) {
+        scan_rows<kGen, 6>(P, S, tc, h, n, s00, lane, a, d, 6, q, bad);
+    } else if (one_degree && !wide && D == 4 && ((first - h.ci_lo) & 1) == 0) {
+        scan_rows<kGen, 4>(P, S, tc, h, n, s00, lane, a, d, 4, q, bad);
+    } else {
+        uint32_t dm = 0;
+#pragma unroll
+        for (int k = 0; k < kRows; ++k) {
+            d[k] = rp[lane + kChunk * k + 1] - a[k];
+            dm = max(dm, (uint32_t)d[k]);       // (a row running backwards counts as long)
+        }
+        const int32_t dmax = (int32_t)__reduce_max_sync(kFull, dm);
+        if ((uint32_t)dmax > (uint32_t)kRowRegs || first < h.e0 || last > h.e1) return false;
+        if (wide) scan_rows<kGen, 0, true>(P, S, tc, h, n, s00, lane, a, d, dmax, q, bad);
+        else scan_rows<kGen, 0>(P, S, tc, h, n, s00, lane, a, d, dmax, q, bad);
     }
-    c0.i = i0; c0.a = a0; c0.a_next = b0; c0.mk = k0; c0.lab = lab0; c0.fast = true;
-    c0.resmask = n0 ? (l0 & ~(1u << k0)) : 0u; c0.r = n0 > 1 ? n0 - 1 : 0;
-    c1.i = i1; c1.a = a1; c1.a_next = b1; c1.mk = k1; c1.lab = lab1; c1.fast = true;
-    c1.resmask = n1 ? (l1 & ~(1u << k1)) : 0u; c1.r = n1 > 1 ? n1 - 1 : 0;
+    if (bad) raise_err(P.err, kErrIndex);
+    // One pointer jump inside each chunk: a label that points to a site of the
+    // chunk takes that site's label. The value taken is an ancestor of the
+    // site, so it stays a valid label, and a chain along a lattice row shortens
+    // by half before step (iii) and the analysis follow it.
+#pragma unroll
+    for (int k = 0; k < kRows; ++k) {
+        const uint32_t in = (uint32_t)(q.lab[k] - (s00 + kChunk * k));
+        const int32_t up = __shfl_sync(kFull, q.lab[k], (int)(in & 31u));
+        if (in < 32u) q.lab[k] = up;
+    }
+    // a label in a tile of this band finished kStages tiles ago: take that
+    // site's label (the band shortcut)
+    const uint32_t vis_lo = (uint32_t)tc.vis_lo * kTileSites;
+    const uint32_t vis_n = tc.vis_hi < tc.vis_lo ? 0u : (uint32_t)(tc.vis_hi + 1 - tc.vis_lo) * kTileSites;
+#pragma unroll
+    for (int k = 0; k < kRows; ++k)
+        if ((uint32_t)q.lab[k] - vis_lo < vis_n) q.lab[k] = __ldcg(I.labels + q.lab[k]);
     return true;
 }
 
@@ -555,36 +637,31 @@ __device__ __forceinline__ void init_emit_chunk(const Params &P, const Stage &S,
     }
 }
 
-// Both chunks of a warp on the register path: the residual pairs of a lane's
-// two sites in one loop (chunk 0's bits low, chunk 1's from bit 16), with a
-// warp-uniform trip count, so the warp neither diverges nor loops twice.
-// The queue order is that of init_emit_chunk on chunk 0 then chunk 1.
+// The residual pairs of a lane's four rows on the register path, in one loop
+// with a warp-uniform trip count, so the warp neither diverges nor loops four
+// times. The warp's queue slots have been checked against the queue's end.
 template <bool kBatched>
-__device__ __forceinline__ void init_emit_pair(const Params &P, const Stage &S, const TileHdr &h,
-                                               const ChunkRes &c0, const ChunkRes &c1, int64_t slot, int rr) {
+__device__ __forceinline__ void init_emit_rows(const Params &P, const Stage &S, const TileHdr &h, const RowsRes &q,
+                                               int64_t slot, int rr) {
     const int iters = (int)__reduce_max_sync(kFull, (uint32_t)rr);
-    uint32_t mm = c0.resmask | (c1.resmask << 16);
-    if (slot + rr > P.q_cap) {                  // corrupt rows only
-        if (rr > 0) raise_err(P.err, kErrIndex);
-        mm = 0;
-    }
-    const int32_t offA = c0.a - h.ci_lo, offB = c1.a - h.ci_lo - 16;
+    uint32_t mm = q.res;
     int2 *qp = P.q + slot;
     int32_t *kp = kBatched ? P.qk + slot : nullptr;
     for (int it = 0; it < iters; ++it) {
         if (mm) {
             const int t = __ffs(mm) - 1;
             mm &= mm - 1;
-            const bool hi = t >= 16;
-            const int32_t j = S.ci[(hi ? offB : offA) + t];
-            *qp++ = make_int2(hi ? c1.lab : c0.lab, j);
+            int32_t off = t & 8 ? q.off[1] : q.off[0], up = t & 8 ? q.lab[1] : q.lab[0];
+            const int32_t off2 = t & 8 ? q.off[3] : q.off[2], up2 = t & 8 ? q.lab[3] : q.lab[2];
+            if (t & 16) { off = off2; up = up2; }
+            *qp++ = make_int2(up, S.ci[off + q.last - (t & 7)]);
             if (kBatched) *kp++ = h.k;
         }
     }
 }
 
 template <bool kBatched, bool kGen = false>
-__global__ void __launch_bounds__(kInitThreads, 2) k_init(Params P) {
+__global__ void __launch_bounds__(kInitThreads, kInitCtas) k_init(Params P) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     uint64_t *full = reinterpret_cast<uint64_t *>(smem_raw);
     uint64_t *empty = full + kStages;
@@ -613,7 +690,6 @@ __global__ void __launch_bounds__(kInitThreads, 2) k_init(Params P) {
     uint32_t ph = 0;
     const int32_t ntl = (int32_t)(band_hi - band_lo);
     for (int32_t tl = 0; tl < ntl; ++tl, s = (s + 1 == kStages) ? 0 : s + 1, ph ^= (s == 0) ? 1u : 0u) {
-        const int64_t tile = band_lo + tl;
         if (!mbar_wait_bounded(&full[s], ph)) {
             raise_err(P.err, kErrNonconv);
             break;
@@ -623,23 +699,28 @@ __global__ void __launch_bounds__(kInitThreads, 2) k_init(Params P) {
         TileCtx tc;
         TileHdr th;
         load_tile_hdr(S.h, th, tc);
-        static_assert(kChunksPerConsumer == 2, "a consumer warp scans two chunks per tile");
-        {
-            // both chunks are scanned first; their pairs then take one range of
-            // queue slots (one prefix sum and one band counter update per tile)
-            const int cc0 = warp * 2, cc1 = warp * 2 + 1;
-            ChunkRes c0, c1;
-            c0.r = c1.r = 0;
-            c0.resmask = c1.resmask = 0u;
-            c0.fast = c1.fast = true;
-            const bool has0 = cc0 * kChunk < th.ts, has1 = cc1 * kChunk < th.ts;
-            if (!(has1 && init_scan_pair<kBatched, kGen>(P, S, I, cc0, lane, tc, th, c0, c1))) {
-                if (has0) init_scan_chunk<kBatched, kGen>(P, S, I, cc0, lane, tc, c0);
-                if (has1) init_scan_chunk<kBatched, kGen>(P, S, I, cc1, lane, tc, c1);
+        // The chunks are scanned first; their pairs then take one range of
+        // queue slots (one prefix sum and one band counter update per tile),
+        // taken before the labels are stored: the shortcut's label loads land
+        // meanwhile.
+        const int32_t loc = warp * kRows * kChunk;      // the warp's first site in the tile
+        if (loc < th.ts) {
+            const int32_t s00 = th.s0 + loc;
+            RowsRes q;
+            ChunkRes c[kRows];
+            const bool fast = init_scan_rows<kGen>(P, S, I, s00, lane, tc, th, q);
+            int rr;
+            if (fast) {
+                rr = __popc(q.res);
+            } else {
+                rr = 0;
+#pragma unroll
+                for (int k = 0; k < kRows; ++k) {
+                    c[k].r = 0;
+                    if (loc + k * kChunk < th.ts) init_scan_chunk<kBatched, kGen>(P, S, I, warp * kRows + k, lane, tc, c[k]);
+                    rr += c[k].r;
+                }
             }
-            // the pair count's prefix sum and the band counter first: the
-            // shortcut label loads of the scan (c0.lab, c1.lab) land meanwhile
-            const int rr = c0.r + c1.r;
             const int incl = warp_incl_scan(rr, lane);
             const int total = __shfl_sync(kFull, incl, 31);
             unsigned long long base = 0;
@@ -647,15 +728,33 @@ __global__ void __launch_bounds__(kInitThreads, 2) k_init(Params P) {
                 if (lane == 0) base = atomicAdd(&band_cnt, (unsigned long long)total);
                 base = __shfl_sync(kFull, base, 0);
             }
-            if (has0 && c0.i < I.n) I.labels[c0.i] = c0.lab;
-            if (has1 && c1.i < I.n) I.labels[c1.i] = c1.lab;
+            if (fast) {
+                int32_t *out = I.labels + s00 + lane;
+#pragma unroll
+                for (int k = 0; k < kRows; ++k) out[kChunk * k] = q.lab[k];
+            } else {
+#pragma unroll
+                for (int k = 0; k < kRows; ++k)
+                    if (loc + k * kChunk < th.ts && c[k].i < I.n) I.labels[c[k].i] = c[k].lab;
+            }
             if (total > 0) {
-                const int64_t slot = S.h.qband + (int64_t)base + (incl - rr);
-                if (c0.fast && c1.fast) {
-                    init_emit_pair<kBatched>(P, S, th, c0, c1, slot, rr);
+                int64_t slot = S.h.qband + (int64_t)base;
+                if (slot + total > P.q_cap) {           // corrupt rows only
+                    if (lane == 0) raise_err(P.err, kErrIndex);
+                    // step (iii) reads every slot up to the queue's end
+                    for (int64_t e = slot + lane; e < P.q_cap; e += 32) {
+                        P.q[e] = make_int2(0, 0);
+                        if (kBatched) P.qk[e] = th.k;
+                    }
+                } else if (fast) {
+                    init_emit_rows<kBatched>(P, S, th, q, slot + (incl - rr), rr);
                 } else {
-                    if (c0.r > 0) init_emit_chunk<kBatched, kGen>(P, S, I, c0, slot);
-                    if (c1.r > 0) init_emit_chunk<kBatched, kGen>(P, S, I, c1, slot + c0.r);
+                    slot += incl - rr;
+#pragma unroll
+                    for (int k = 0; k < kRows; ++k) {
+                        if (c[k].r > 0) init_emit_chunk<kBatched, kGen>(P, S, I, c[k], slot);
+                        slot += c[k].r;
+                    }
                 }
             }
         }
@@ -665,7 +764,11 @@ __global__ void __launch_bounds__(kInitThreads, 2) k_init(Params P) {
     // the band's pair count, once every consumer warp has added its own (the
     // producer warp may have returned)
     consumers_sync<32 * kInitConsumers>();
-    if (threadIdx.x == 0) P.band[P.band_off + blockIdx.x].cnt = band_cnt;
+    if (threadIdx.x == 0) {
+        BandRec &rec = P.band[P.band_off + blockIdx.x];
+        const long long room = max((long long)(P.q_cap - rec.qbase), 0ll);      // (less only for corrupt rows)
+        rec.cnt = min(band_cnt, (unsigned long long)room);
+    }
 }
 
 // ---------------------------------------------------------------------------

@@ -14,14 +14,18 @@ constexpr unsigned kFull = 0xffffffffu;
 // producer streams tiles of kTileSites sites through kStages shared-memory
 // stages with bulk asynchronous copies
 constexpr int kTileSites = 1024;
-constexpr int kInitConsumers = 16;
+constexpr int kRows = 4;                   // rows a lane scans at once, one in each of its warp's chunks
+constexpr int kInitConsumers = kTileSites / kChunk / kRows;
 constexpr int kInitThreads = 32 * (kInitConsumers + 1);
-constexpr int kChunksPerConsumer = kTileSites / kChunk / kInitConsumers;
 constexpr int kStages = 3;
+constexpr int kInitCtas = 2;               // CTAs per SM (their stages fill the shared memory)
+// the dense list's kernel: sixteen consumer warps of two chunks
+constexpr int kDenseConsumers = 16;
+constexpr int kDenseTmaThreads = 32 * (kDenseConsumers + 1);
 constexpr int kColCap = 7168;              // column entries a stage holds (7 per site)
 constexpr int kRpBuf = kTileSites + 8;     // row pointers of a tile, + 16-byte rounding
 constexpr int kColBuf = kColCap + 8;
-constexpr int kBitBuf = kColCap / 32 + 12;
+constexpr int kBitBuf = kColCap / 32 + 12;   // (a word past the last one copied may be read)
 constexpr int kRowRegs = 8;                // rows up to this degree are scanned in registers
 
 // steps (ii)/(iv): chunks a warp walks at once

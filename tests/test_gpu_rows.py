@@ -1,0 +1,71 @@
+"""Step (i)'s row scan against the oracle where its variants meet: rows of one
+degree (3, 4 and 6 have their own code), mixed rows, rows past the register
+path, chunk groups that end at 128 sites, and every alignment of an instance's
+entries inside a batch. Labels are integers: equality, no tolerance."""
+import numpy as np
+import pytest
+import torch
+
+import lattices as L
+import oracle
+import paper_1603_08357_gb300 as ccl
+from ccl_testutil import DEV, gpu_label
+
+pytestmark = pytest.mark.gpu
+
+
+def _graph(n, degrees, p, seed):
+    """Rows of the given degrees with uniform random columns (repeats and
+    self-loops included) and Bernoulli(p) entry bits."""
+    rng = np.random.default_rng(seed)
+    rp = np.concatenate([[0], np.cumsum(degrees)]).astype(np.int32)
+    nnz = int(rp[-1])
+    near = rng.random(nnz) < 0.5          # half of the columns close by: chains inside a chunk
+    row = np.repeat(np.arange(n), degrees)
+    col = np.where(near, np.clip(row - rng.integers(0, 40, nnz), 0, n - 1), rng.integers(0, n, nnz)).astype(np.int32)
+    return L.Lattice("random", n, nnz, rp, col, L.pack_bits(rng.random(nnz) < p), p, seed)
+
+
+@pytest.mark.parametrize("degree", [1, 2, 3, 4, 5, 6, 8, 9])
+@pytest.mark.parametrize("n", [127, 128, 129, 1024, 1151, 4000])
+def test_one_degree(ctx, degree, n):
+    for p in (0.0, 0.3, 1.0):
+        lat = _graph(n, np.full(n, degree), p, 100 * degree + n)
+        assert np.array_equal(gpu_label(ctx, lat), oracle.uf_label(lat))
+        assert ccl.ccl_get_stats(ctx).residual_pairs == oracle.steps_label(lat)["n_residual"]
+
+
+@pytest.mark.parametrize("top", [1, 3, 7, 8, 12])
+def test_mixed_degrees(ctx, top):
+    for n in (128, 1000, 5000):
+        deg = np.random.default_rng(n + top).integers(0, top + 1, n)
+        lat = _graph(n, deg, 0.6, n)
+        assert np.array_equal(gpu_label(ctx, lat), oracle.uf_label(lat))
+
+
+def test_batch_alignments(ctx):
+    """Instances of odd entry counts one after another: entries, bits, row
+    pointers and labels of later instances start at every offset of 16 bytes."""
+    lats = [_graph(n, np.full(n, d), 0.45, 7 * n + d) for d in (3, 4, 6, 5) for n in (129, 1025, 641, 2047)]
+    so = np.concatenate([[0], np.cumsum([x.n for x in lats])])
+    eo = np.concatenate([[0], np.cumsum([x.nnz for x in lats])])
+    bits = L.pack_bits(np.concatenate([L.unpack_bits(x.open_bits, x.nnz) for x in lats]))
+    dev = [torch.from_numpy(np.concatenate(a)).to(DEV) for a in ([x.row_ptr for x in lats], [x.col_idx for x in lats])]
+    out = torch.full((int(so[-1]),), -1, dtype=torch.int32, device=DEV)
+    assert ccl.ccl_label_batched(ctx, len(lats), so, eo, *dev, torch.from_numpy(bits.view(np.int32)).to(DEV), out) == ccl.CCL_OK
+    assert ccl.ccl_sync(ctx) == ccl.CCL_OK
+    got = out.cpu().numpy()
+    for k, x in enumerate(lats):
+        assert np.array_equal(got[so[k]:so[k + 1]], oracle.uf_label(x)), k
+
+
+@pytest.mark.parametrize("degree", [3, 4, 5, 6])
+@pytest.mark.parametrize("value", [-1, 4000, 2**28 + 5, 2**31 - 1])
+def test_column_out_of_range_is_reported(ctx, degree, value):
+    lat = _graph(4000, np.full(4000, degree), 1.0, degree)
+    lat.col_idx[1234 * degree + 1] = value
+    rp, ci = torch.from_numpy(lat.row_ptr).to(DEV), torch.from_numpy(lat.col_idx).to(DEV)
+    out = torch.empty(lat.n, dtype=torch.int32, device=DEV)
+    assert ccl.ccl_label(ctx, lat.n, lat.nnz, rp, ci, torch.from_numpy(lat.open_bits.view(np.int32)).to(DEV), out) == ccl.CCL_OK
+    assert ccl.ccl_sync(ctx) == ccl.CCL_ERR_INDEX_OUT_OF_RANGE
+    assert int(out.min()) >= 0 and int(out.max()) < lat.n
