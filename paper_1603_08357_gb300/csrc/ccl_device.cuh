@@ -201,20 +201,61 @@ __device__ __forceinline__ void cta_band(const Params &P, int64_t &band_lo, int6
     band_hi = P.tile_off + min(lo + per, P.n_tiles);
 }
 
+// Tiles of band `band` of a launch of P.init_bands bands. Bands come in rounds
+// of one per CTA, those of round r of P.round_per[r] tiles. A CTA takes band
+// blockIdx.x and then, while there are bands left, the next one from a ticket
+// counter.
+__device__ __forceinline__ void band_tiles(const Params &P, int32_t band, int64_t &lo, int64_t &hi) {
+    int32_t r = 0, in = band;
+    int64_t first = 0;
+    for (; in >= (int32_t)gridDim.x; ++r, in -= (int32_t)gridDim.x) first += (int64_t)gridDim.x * P.round_per[r];
+    lo = P.tile_off + min(first + (int64_t)in * P.round_per[r], P.n_tiles);
+    hi = P.tile_off + min(first + (int64_t)(in + 1) * P.round_per[r], P.n_tiles);
+}
+
+// The bands a CTA has under way (shared memory): at most kStages tiles are, so
+// band number `seq` of the CTA can use the place of band seq - kBandSlots.
+constexpr int kBandSlots = kStages + 1;
+struct BandSlots {
+    unsigned long long cnt[kBandSlots];     // pairs found so far
+    int32_t band[kBandSlots];
+    int32_t taken;                          // bands the CTA has taken
+};
+
+// Stores the pair count of a finished band.
+__device__ __forceinline__ void store_band(const Params &P, const BandSlots &B, int slot) {
+    BandRec &rec = P.band[P.band_off + B.band[slot]];
+    const long long room = max((long long)(P.q_cap - rec.qbase), 0ll);      // (less only for corrupt rows)
+    rec.cnt = min(B.cnt[slot], (unsigned long long)room);
+}
+
 template <bool kBatched, bool kGen = false>
 __device__ __forceinline__ void init_produce(const Params &P, Stage *st, uint64_t *full,
-                                             uint64_t *empty) {
-    int64_t band_lo, band_hi;
-    cta_band(P, band_lo, band_hi);
+                                             uint64_t *empty, BandSlots &B) {
     int64_t t_local = 0;
     int64_t qband = 0;
     int kc = 0;                              // cached instance and its tile range
     int64_t kc_lo = 0, kc_hi = kBatched ? 0 : P.n_tiles;
+    int32_t band = blockIdx.x, next = 0;
+    bool ok = true;
+    for (int32_t seq = 0; ok && band < P.init_bands; ++seq, band = next) {
+    int64_t band_lo, band_hi;
+    band_tiles(P, band, band_lo, band_hi);
+    // the next band is known before this one's last tile is published
+    next = gridDim.x < (unsigned)P.init_bands ? (int32_t)(gridDim.x + atomicAdd(P.ticket, 1u)) : P.init_bands;
+    // every tile but the last kStages has been consumed, hence all of the
+    // band that had this place
+    const int slot = seq % kBandSlots;
+    if (seq >= kBandSlots) store_band(P, B, slot);
+    B.cnt[slot] = 0;
+    B.band[slot] = band;
+    B.taken = seq + 1;
     for (int64_t tile = band_lo; tile < band_hi; ++tile, ++t_local) {
         const int s = (int)(t_local % kStages);
         const int64_t use = t_local / kStages;
         if (use > 0 && !mbar_wait_bounded(&empty[s], (uint32_t)((use - 1) & 1))) {
             raise_err(P.err, kErrNonconv);
+            ok = false;
             break;
         }
         if (kBatched && (tile < kc_lo || tile >= kc_hi)) {
@@ -242,11 +283,13 @@ __device__ __forceinline__ void init_produce(const Params &P, Stage *st, uint64_
         h.i_tile_begin = I.tile_begin;
         h.i_n = I.n;
         h.i_nnz = I.nnz;
-        if (t_local == 0) {
+        if (tile == band_lo) {
             qband = I.q_off + (h.status ? 0 : h.e0);
-            P.band[P.band_off + blockIdx.x].qbase = qband;
+            P.band[P.band_off + band].qbase = qband;
         }
         h.qband = qband;
+        h.slot = slot;
+        h.last = tile + 1 == band_hi && next >= P.init_bands;
         int64_t lo, hi;
         copy_window(I.row_ptr, h.s0, (int64_t)h.s0 + h.ts + 1, I.rp_lo, I.rp_hi, kRpBuf, lo, hi);
         h.rp_lo = (int32_t)lo;
@@ -281,6 +324,7 @@ __device__ __forceinline__ void init_produce(const Params &P, Stage *st, uint64_
         if (b_rp) bulk_g2s(st[s].rp, I.row_ptr + h.rp_lo, b_rp, &full[s]);
         if (b_ci) bulk_g2s(st[s].ci, I.col_idx + h.ci_lo, b_ci, &full[s]);
         if (b_bw) bulk_g2s(st[s].bw, I.bits + h.w_lo, b_bw, &full[s]);
+    }
     }
     drain_armed(full, t_local, P.err);
 }
@@ -675,25 +719,23 @@ __global__ void __launch_bounds__(kInitThreads, kInitCtas) k_init(Params P) {
         }
         mbar_fence_init();
     }
-    __shared__ unsigned long long band_cnt;
-    if (threadIdx.x == 0) band_cnt = 0;
+    __shared__ BandSlots bands;
+    if (threadIdx.x == 0) bands.taken = 0;
     __syncthreads();
     if (warp == kInitConsumers) {               // producer warp
-        if (lane == 0) init_produce<kBatched, kGen>(P, st, full, empty);
+        if (lane == 0) init_produce<kBatched, kGen>(P, st, full, empty, bands);
         return;
     }
-    int64_t band_lo, band_hi;
-    cta_band(P, band_lo, band_hi);
-    // stage s = tl % kStages and phase parity (tl / kStages) & 1 of local tile
-    // tl, kept incrementally in 32-bit (no 64-bit division per tile)
+    // stage and phase parity of the CTA's tile number t are t % kStages and
+    // (t / kStages) & 1, kept incrementally in 32-bit (no 64-bit division)
     int s = 0;
     uint32_t ph = 0;
-    const int32_t ntl = (int32_t)(band_hi - band_lo);
-    for (int32_t tl = 0; tl < ntl; ++tl, s = (s + 1 == kStages) ? 0 : s + 1, ph ^= (s == 0) ? 1u : 0u) {
+    for (bool last = false; !last; s = (s + 1 == kStages) ? 0 : s + 1, ph ^= (s == 0) ? 1u : 0u) {
         if (!mbar_wait_bounded(&full[s], ph)) {
             raise_err(P.err, kErrNonconv);
             break;
         }
+        last = st[s].h.last != 0;
         const Stage &S = st[s];
         const Inst I = stage_inst<kBatched>(P, S.h);
         TileCtx tc;
@@ -725,7 +767,7 @@ __global__ void __launch_bounds__(kInitThreads, kInitCtas) k_init(Params P) {
             const int total = __shfl_sync(kFull, incl, 31);
             unsigned long long base = 0;
             if (total > 0) {
-                if (lane == 0) base = atomicAdd(&band_cnt, (unsigned long long)total);
+                if (lane == 0) base = atomicAdd(&bands.cnt[S.h.slot], (unsigned long long)total);
                 base = __shfl_sync(kFull, base, 0);
             }
             if (fast) {
@@ -761,14 +803,11 @@ __global__ void __launch_bounds__(kInitThreads, kInitCtas) k_init(Params P) {
         __syncwarp();
         if (lane == 0) mbar_arrive(&empty[s]);
     }
-    // the band's pair count, once every consumer warp has added its own (the
-    // producer warp may have returned)
+    // the last bands' pair counts, once every consumer warp has added its own
+    // (the producer warp may have returned)
     consumers_sync<32 * kInitConsumers>();
-    if (threadIdx.x == 0) {
-        BandRec &rec = P.band[P.band_off + blockIdx.x];
-        const long long room = max((long long)(P.q_cap - rec.qbase), 0ll);      // (less only for corrupt rows)
-        rec.cnt = min(band_cnt, (unsigned long long)room);
-    }
+    if (threadIdx.x == 0)
+        for (int32_t q = max(bands.taken - kBandSlots, 0); q < bands.taken; ++q) store_band(P, bands, q % kBandSlots);
 }
 
 // ---------------------------------------------------------------------------
@@ -1015,71 +1054,115 @@ __device__ __forceinline__ int32_t red_load(const int32_t *p) { return __ldca(p)
 //  kStatic = true: lane l serves pairs wbeg + l, wbeg + l + 32, ... and loads
 //    its next pair a round before a slot needs it: fewer instructions per
 //    round and no exposed queue load (lattices).
-template <bool kBatched, bool kStatic>
-__global__ void __launch_bounds__(256) k_reduce(Params P) {
-    __shared__ long long s_pref[kMaxBands + 1];
-    if (threadIdx.x < 32) {
-        // exclusive prefix of the band counts by warp 0: each lane sums a
-        // contiguous slice, then a warp scan of the slice totals
-        const int lane = threadIdx.x;
-        const int per = (P.n_bands + 31) / 32;
-        const int b0 = min(lane * per, P.n_bands), b1 = min(b0 + per, P.n_bands);
-        long long part = 0;
-        for (int b = b0; b < b1; ++b) part += (long long)P.band[b].cnt;
-        long long incl = part;
+//
+// The pairs are cut into windows inside each band, so a window's pairs are
+// consecutive queue slots. Every CTA finds the windows of all bands by itself:
+// s_win[b] = windows before band b, in dynamic shared memory, only as much as
+// there are bands (the rest of the SM's memory is cache for the labels).
+// Against one index space over all bands (8 KB of 64-bit prefix sums, a band
+// look-up per pair): triangle 16384^2 1.46 -> 1.37 ms.
+constexpr int kRedThreads = 256;
+
+// Exclusive prefix sum of one value per thread over the CTA; *sum = the total.
+__device__ __forceinline__ long long block_excl_scan(long long v, long long *s_warp, long long *sum) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    long long incl = v;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const long long t = __shfl_up_sync(kFull, incl, o);
-            if (lane >= o) incl += t;
-        }
-        long long acc = incl - part;
-        for (int b = b0; b < b1; ++b) {
-            s_pref[b] = acc;
-            acc += (long long)P.band[b].cnt;
-        }
-        if (lane == 31) s_pref[P.n_bands] = incl;
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long t = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += t;
+    }
+    if (lane == 31) s_warp[warp] = incl;
+    __syncthreads();
+    long long before = 0, all = 0;
+#pragma unroll
+    for (int w = 0; w < kRedThreads / 32; ++w) {
+        if (w < warp) before += s_warp[w];
+        all += s_warp[w];
     }
     __syncthreads();
-    const long long total = s_pref[P.n_bands];
-    // the call's statistics (a call in parts adds its later parts' pairs)
+    *sum = all;
+    return before + incl - v;
+}
+
+template <bool kBatched, bool kStatic>
+__global__ void __launch_bounds__(kRedThreads, kBatched ? 4 : 5) k_reduce(Params P) {
+    extern __shared__ uint32_t s_win[];             // [n_bands + 1]
+    __shared__ long long s_warp[kRedThreads / 32];
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    const long long nwarps = (long long)gridDim.x * (kRedThreads / 32);
+    // one window per warp when the queue is short (bands round their window
+    // counts up: at most one more each), at least 64 pairs
+    const auto window = [&](long long total) {
+        const long long wmax = P.red_window > 0 ? P.red_window : kRedWindowMax;
+        const long long room = max(nwarps - P.n_bands, nwarps / 2);
+        return min(max((total + room - 1) / room, 64ll), wmax);
+    };
+    long long total;
+    if (P.n_bands <= 32) {
+        // a small call: every warp by itself, without barriers (all write the
+        // same values)
+        const long long cnt = lane < P.n_bands ? (long long)P.band[lane].cnt : 0;
+        total = cnt;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(kFull, total, o);
+        const long long win = window(total);
+        const int nw = (int)((cnt + win - 1) / win), upto = warp_incl_scan(nw, lane);
+        if (lane < P.n_bands) s_win[lane + 1] = (uint32_t)upto;
+        if (lane == 0) s_win[0] = 0;
+        __syncwarp();
+    } else {
+        const int per = (P.n_bands + kRedThreads - 1) / kRedThreads;
+        const int b0 = min((int)threadIdx.x * per, P.n_bands), b1 = min(b0 + per, P.n_bands);
+        long long part = 0, sum;
+        for (int b = b0; b < b1; ++b) part += (long long)P.band[b].cnt;
+        block_excl_scan(part, s_warp, &total);
+        const long long win = window(total);
+        long long nw = 0;
+        for (int b = b0; b < b1; ++b) nw += ((long long)P.band[b].cnt + win - 1) / win;
+        long long acc = block_excl_scan(nw, s_warp, &sum);
+        for (int b = b0; b < b1; ++b) {
+            s_win[b] = (uint32_t)acc;
+            acc += ((long long)P.band[b].cnt + win - 1) / win;
+        }
+        if (threadIdx.x == 0) s_win[P.n_bands] = (uint32_t)sum;
+        __syncthreads();
+    }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
+        // the call's statistics (a call in parts adds its later parts' pairs)
         if (P.more_pairs) P.counters[0] += (unsigned long long)total;
         else P.counters[0] = (unsigned long long)total;
     }
-    const int lane = threadIdx.x & 31;
-    const unsigned lt = (1u << lane) - 1u;
-    const long long nwarps = (long long)gridDim.x * (blockDim.x >> 5);
-    const long long wmax = P.red_window > 0 ? P.red_window : kRedWindowMax;
-    long long win = (total + nwarps - 1) / nwarps;
-    win = win < 64 ? 64 : (win > wmax ? wmax : win);
-    const long long nwin = (total + win - 1) / win;
+    const long long nwin = s_win[P.n_bands];
 #ifdef CCL_DEVICE_STATS
     unsigned long long st_hops = 0, st_atom = 0, st_iter = 0;
 #endif
     for (long long w = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w < nwin; w += nwarps) {
-        const long long wbeg = w * win;
-        const int wlen = (int)(min(wbeg + win, total) - wbeg);
+        // band of the window: the last one with at most w windows before it
+        // (all lanes search; smem broadcast)
+        int band = 0;
+        for (int hi = P.n_bands - 1; band < hi;) {
+            const int mid = (band + hi + 1) >> 1;
+            if (s_win[mid] <= (uint32_t)w) band = mid; else hi = mid - 1;
+        }
+        // the band's pairs are spread evenly over its windows
+        const long long bcnt = (long long)P.band[band].cnt;
+        const int bwin = (int)(s_win[band + 1] - s_win[band]);
+        const long long wmost = (bcnt + bwin - 1) / bwin;
+        const long long wbeg = (long long)((uint32_t)w - s_win[band]) * wmost;
+        const int wlen = (int)max(min(wbeg + wmost, bcnt) - wbeg, 0ll);
+        const int2 *wq = P.q + P.band[band].qbase + wbeg;
+        const int32_t *wqk = kBatched ? P.qk + P.band[band].qbase + wbeg : nullptr;
         // A pair needs at most 4n + 8 rounds (its chains and Algorithm 1's loop
         // are bounded by the instance's n <= 32 n_chunks); a lane serves at most
         // wlen pairs. Past this many rounds the window is abandoned with an error.
         const long long round_cap = P.iter_cap > 0 ? (long long)P.iter_cap
                                                     : (128ll * P.n_chunks + 8) * (long long)wlen;
         long long rounds = 0;
-        // band of the window's first pair (all lanes search; smem broadcast)
-        int band = 0;
-        {
-            int lo = 0, hi = P.n_bands - 1;
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (s_pref[mid] <= wbeg) lo = mid; else hi = mid - 1;
-            }
-            band = lo;
-        }
         int nxt = 0;        // pairs of the window handed to slots so far
         // kStatic: the lane's next pair, loaded ahead
-        long long pnext = wbeg + lane;
-        const long long wend = wbeg + wlen;
-        int cur = band;             // band cursor of this lane (its pairs increase)
+        int pnext = lane;
         int2 pf = make_int2(0, 0);
         int pfk = 0;
         bool pf_ok = false;
@@ -1087,19 +1170,13 @@ __global__ void __launch_bounds__(256) k_reduce(Params P) {
         // of a lane mostly come from one instance)
         int lk = 0;
         int32_t *llab = kBatched ? P.insts[0].labels : P.one.labels;
-        // queue slot of pair p = qoff + p inside band `cur`
-        long long qoff = P.band[cur].qbase - s_pref[cur];
-        auto fetch = [&](long long p) {
-            if (s_pref[cur + 1] <= p) {
-                do { ++cur; } while (s_pref[cur + 1] <= p);
-                qoff = P.band[cur].qbase - s_pref[cur];
-            }
-            const long long slot = qoff + p;
-            pf = P.q[slot];
-            if (kBatched) pfk = P.qk[slot];
+        auto fetch = [&]() {
+            pf = wq[pnext];
+            if (kBatched) pfk = wqk[pnext];
             pf_ok = true;
+            pnext += 32;
         };
-        if (kStatic && pnext < wend) { fetch(pnext); pnext += 32; }
+        if (kStatic && pnext < wlen) fetch();
         int32_t *L[kRedSlots];
         int32_t a[kRedSlots], b[kRedSlots], st[kRedSlots];
 #pragma unroll
@@ -1123,7 +1200,7 @@ __global__ void __launch_bounds__(256) k_reduce(Params P) {
                     for (int u = 0; u < kRedSlots; ++u)
                         if (u == take) { a[u] = na; b[u] = nb; st[u] = kTaskChase; L[u] = nl; }
                     pf_ok = false;
-                    if (pnext < wend) { fetch(pnext); pnext += 32; }
+                    if (pnext < wlen) fetch();
                 }
             } else {
                 // refill empty slots with the window's next pairs, in order (the
@@ -1135,13 +1212,9 @@ __global__ void __launch_bounds__(256) k_reduce(Params P) {
                         if (need == 0) continue;
                         const int pos = nxt + __popc(need & lt);
                         if (st[u] == kTaskDone && pos < wlen) {
-                            const long long p = wbeg + pos;
-                            int bb = band;
-                            while (s_pref[bb + 1] <= p) ++bb;
-                            const long long slot = P.band[bb].qbase + (p - s_pref[bb]);
-                            const int2 pr = P.q[slot];
+                            const int2 pr = wq[pos];
                             if (kBatched) {
-                                const int k = P.qk[slot];
+                                const int k = wqk[pos];
                                 if (k != lk) { lk = k; llab = P.insts[k].labels; }
                                 L[u] = llab;
                             }
@@ -1150,8 +1223,6 @@ __global__ void __launch_bounds__(256) k_reduce(Params P) {
                             st[u] = kTaskChase;
                         }
                         nxt = min(nxt + __popc(need), wlen);
-                        const long long pn = wbeg + nxt;
-                        while (band < P.n_bands - 1 && s_pref[band + 1] <= pn) ++band;
                         if (nxt >= wlen) break;
                     }
                 }

@@ -138,7 +138,8 @@ extern "C" ccl_status ccl_label_noalloc(int32_t n, int64_t nnz, const int32_t *r
     g = std::max<int64_t>(g, 1);
     const int64_t per = (P.n_tiles + g - 1) / g;
     const int64_t g_init = (P.n_tiles + per - 1) / per;
-    P.n_bands = (int32_t)g_init;
+    P.n_bands = P.init_bands = (int32_t)g_init;
+    P.round_per[0] = (int32_t)per;
     const int64_t ana_warps = (P.n_chunks + kAnaChunks - 1) / kAnaChunks;
     const int64_t g_ana = std::max<int64_t>(1, std::min<int64_t>((int64_t)d->num_sms * d->ana_per_sm, (ana_warps + 7) / 8));
     const int64_t g_red = (int64_t)d->num_sms * d->red_per_sm;
@@ -148,7 +149,7 @@ extern "C" ccl_status ccl_label_noalloc(int32_t n, int64_t nnz, const int32_t *r
     cudaError_t e = cudaMemsetAsync(d->scratch + kOffErr, 0, sizeof(unsigned), s);
     if (e == cudaSuccess) {
         k_init<false><<<(unsigned)g_init, kInitThreads, kInitSmem, s>>>(P);
-        k_reduce<false, true><<<(unsigned)g_red, 256, 0, s>>>(P);
+        k_reduce<false, true><<<(unsigned)g_red, kRedThreads, sizeof(uint32_t) * (size_t)(g_init + 1), s>>>(P);
         k_analysis<false, true><<<(unsigned)g_ana, 256, 0, s>>>(P);
         e = cudaGetLastError();
     }

@@ -45,7 +45,8 @@ constexpr int kAnaChunksBatched = CCL_ANA_CHUNKS_BATCHED;
 #endif
 constexpr int kRedSlots = CCL_RED_SLOTS;
 constexpr int kRedWindowMax = 2048;   // default most pairs per warp window (fewer for small queues)
-constexpr int kMaxBands = 1024;
+constexpr int kMaxBands = 4096;
+constexpr int kRounds = 12;           // most bands a CTA of step (i) takes
 
 // latched device error bits
 constexpr unsigned kErrIndex = 1u;         // col_idx or row_ptr out of range
@@ -94,6 +95,9 @@ struct Params {
     uint64_t gen_thr;          // ... and threshold (bond open iff output >> 11 < gen_thr)
     const int32_t *nn;         // dense neighbour list (slot k of site i at nn[i + k*n]), or null
     int64_t nn_width;          // slots per site of the dense list
+    int32_t init_bands;        // bands of a step (i) launch: rounds of one per CTA (the last may be short) ...
+    int32_t round_per[kRounds];    // ... and the tiles of a band of each round
+    unsigned *ticket;          // bands taken beyond the first of every CTA (cleared before a launch in rounds)
     int64_t tile_off;          // step (i) on part of the tiles: its first tile ...
     int32_t band_off;          // ... and its first band record
     int32_t more_pairs;        // 1: the pairs of this step (iii) add to counters[0], 0: they replace it
@@ -125,7 +129,8 @@ struct __align__(16) StageHdr {
     // stage-relative bit index of local entry 0, bits present, whether the
     // stage holds the tile's whole entry range, and the instance-local tiles
     // [vis_lo, vis_hi] of the band whose labels are final and visible
-    int32_t t_rb0, t_nbits, t_staged, t_vis_lo, t_vis_hi, pad2_;
+    int32_t t_rb0, t_nbits, t_staged, t_vis_lo, t_vis_hi;
+    int32_t slot, last;        // place of the tile's band in BandSlots; 1: the CTA's last tile
 };
 
 // the consumers load {k, s0, ts, e0}, {e1, rp_lo, rp_hi, ci_lo} and {t_rb0,

@@ -9,7 +9,7 @@ import torch
 import lattices as L
 import oracle
 import paper_1603_08357_gb300 as ccl
-from ccl_testutil import DEV, gpu_label
+from ccl_testutil import DEV, gpu_label, gpu_label_batched
 
 pytestmark = pytest.mark.gpu
 
@@ -69,3 +69,17 @@ def test_column_out_of_range_is_reported(ctx, degree, value):
     assert ccl.ccl_label(ctx, lat.n, lat.nnz, rp, ci, torch.from_numpy(lat.open_bits.view(np.int32)).to(DEV), out) == ccl.CCL_OK
     assert ccl.ccl_sync(ctx) == ccl.CCL_ERR_INDEX_OUT_OF_RANGE
     assert int(out.min()) >= 0 and int(out.max()) < lat.n
+
+
+def test_bands_in_rounds(ctx):
+    """A batch large enough for step (i) to hand its tiles out in rounds of
+    bands (64 tiles per CTA at least): every label and the pair count."""
+    specs = [s for s in L.batched_mix_specs(64, seed=12) if s["kind"] != "cayley" or s["shells"] > 3]
+    b = L.make_batch(specs)
+    assert b.n_total > 64 * 1024 * 2 * 160, "too few tiles for the rounds"
+    got = gpu_label_batched(ctx, b)
+    want, _ = oracle.uf_label_batched_threads(b)
+    assert np.array_equal(got, want[:b.n_total])
+    st = ccl.ccl_get_stats(ctx)
+    assert np.array_equal(gpu_label_batched(ctx, b), got)          # again: the ticket starts over
+    assert ccl.ccl_get_stats(ctx).residual_pairs == st.residual_pairs > 0
