@@ -886,6 +886,9 @@ ccl_status ccl_context_create(ccl_context **out, int device) {
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_init_dense_tma<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)kDenseSmem);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_span_few, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 2 * kSpanTop * (int)sizeof(int32_t));
     if (e != cudaSuccess) {
         (void)cudaGetLastError();
         ccl_context_destroy(ctx);
@@ -1204,6 +1207,14 @@ ccl_status ensure_aux(ccl_context *ctx, int64_t bytes) {
 }
 }  // namespace
 
+namespace {
+// CTAs of 256 threads of the kernels that give every warp one run of 128-site
+// groups (warp_run): all the SM's warps, fewer for short inputs.
+int64_t run_grid(const ccl_context *ctx, int64_t n) {
+    return std::max<int64_t>(1, std::min<int64_t>((int64_t)ctx->num_sms * 8, (n + 1023) / 1024));
+}
+}  // namespace
+
 ccl_status ccl_relabel(ccl_context *ctx, int32_t n, const int32_t *labels, int32_t *seq,
                        int32_t *n_clusters, int32_t *sizes, void *stream) {
     if (!ctx || n < 0 || !n_clusters) return CCL_ERR_INVALID_ARGUMENT;
@@ -1221,9 +1232,7 @@ ccl_status ccl_relabel(ccl_context *ctx, int32_t n, const int32_t *labels, int32
     k_root_counts<<<(unsigned)nb, kRelThreads, 0, s>>>(n, labels, cnt);
     k_scan_counts<<<1, 1024, 0, s>>>((int32_t)nb, cnt, n_clusters);
     k_root_ids<<<(unsigned)nb, kRelThreads, 0, s>>>(n, labels, cnt, seq, sizes);
-    const int64_t g = std::min<int64_t>((int64_t)ctx->num_sms * 8, ((int64_t)n + 255) / 256);
-    k_site_ids<<<(unsigned)g, 256, 0, s>>>(n, labels, seq);
-    if (sizes) k_sizes<<<(unsigned)g, 256, 0, s>>>(n, seq, sizes);
+    k_site_ids<<<(unsigned)run_grid(ctx, n), 256, 0, s>>>(n, labels, seq, sizes);
     CCL_CUDA(cudaGetLastError());
     return CCL_OK;
 }
@@ -1236,6 +1245,14 @@ ccl_status ccl_spanning(ccl_context *ctx, int32_t n, const int32_t *labels, cons
     if ((n_top > 0 && !top) || (n_bottom > 0 && !bottom)) return CCL_ERR_INVALID_ARGUMENT;
     DeviceGuard guard(ctx->device);
     cudaStream_t s = (cudaStream_t)stream;
+    if (n_top <= kSpanTop && n_bottom <= 16 * kSpanTop) {
+        int32_t slots = 64;
+        while (slots < 2 * n_top) slots *= 2;
+        k_span_few<<<1, kSpanThreads, (size_t)slots * sizeof(int32_t), s>>>(n, labels, top, n_top, bottom, n_bottom,
+                                                                          slots, result, ctx->d_err);
+        CCL_CUDA(cudaGetLastError());
+        return CCL_OK;
+    }
     const int64_t words = ((int64_t)n + 31) / 32;
     ccl_status st = ensure_aux(ctx, std::max<int64_t>(words, 1) * (int64_t)sizeof(uint32_t));
     if (st != CCL_OK) return st;
@@ -1245,7 +1262,6 @@ ccl_status ccl_spanning(ccl_context *ctx, int32_t n, const int32_t *labels, cons
     const int64_t gb = std::max<int64_t>(1, std::min<int64_t>(ctx->num_sms * 4, ((int64_t)n_bottom + 255) / 256));
     k_span_mark<<<(unsigned)gt, 256, 0, s>>>(n, labels, top, n_top, flags, result, ctx->d_err);
     k_span_check<<<(unsigned)gb, 256, 0, s>>>(n, labels, bottom, n_bottom, flags, result, ctx->d_err);
-    k_span_finish<<<1, 1, 0, s>>>(result);
     CCL_CUDA(cudaGetLastError());
     return CCL_OK;
 }
@@ -1256,18 +1272,13 @@ ccl_status ccl_largest_cluster(ccl_context *ctx, int32_t n, const int32_t *label
     if (n > 0 && !labels) return CCL_ERR_INVALID_ARGUMENT;
     DeviceGuard guard(ctx->device);
     cudaStream_t s = (cudaStream_t)stream;
-    // scratch: the 64-bit best key, then one count per site
-    ccl_status st = ensure_aux(ctx, 16 + (int64_t)n * (int64_t)sizeof(int32_t));
+    // scratch: the best key and the finished CTAs, then one count per site
+    ccl_status st = ensure_aux(ctx, (int64_t)sizeof(LargestScratch) + (int64_t)n * (int64_t)sizeof(int32_t));
     if (st != CCL_OK) return st;
-    unsigned long long *best = (unsigned long long *)ctx->d_aux;
-    int32_t *cnt = (int32_t *)((char *)ctx->d_aux + 16);
-    CCL_CUDA(cudaMemsetAsync(ctx->d_aux, 0, 16 + (size_t)n * sizeof(int32_t), s));
-    if (n > 0) {
-        const int64_t g = std::max<int64_t>(1, std::min<int64_t>((int64_t)ctx->num_sms * 8, ((int64_t)n + 255) / 256));
-        k_label_counts<<<(unsigned)g, 256, 0, s>>>(n, labels, cnt, ctx->d_err);
-        k_largest<<<(unsigned)g, 256, 0, s>>>(n, cnt, best);
-    }
-    k_largest_finish<<<1, 1, 0, s>>>(best, result);
+    LargestScratch *scratch = (LargestScratch *)ctx->d_aux;
+    int32_t *cnt = (int32_t *)(scratch + 1);
+    CCL_CUDA(cudaMemsetAsync(ctx->d_aux, 0, sizeof(LargestScratch) + (size_t)n * sizeof(int32_t), s));
+    k_largest<<<(unsigned)run_grid(ctx, n), 256, 0, s>>>(n, labels, cnt, scratch, result, ctx->d_err);
     CCL_CUDA(cudaGetLastError());
     return CCL_OK;
 }

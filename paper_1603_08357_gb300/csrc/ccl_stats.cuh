@@ -65,57 +65,133 @@ __global__ void __launch_bounds__(1024) k_scan_counts(int32_t nb, int32_t *__res
 }
 
 // sequential id of every root: its block's offset plus the roots before it in
-// the block, in site order; zeroes the size counter of each id
+// the block, in site order; zeroes the size counter of each id. A warp takes
+// 1024 consecutive sites, keeps the 32 root ballots one per lane and needs the
+// other warps' totals once, so the block meets at one barrier (stepping the
+// whole block through 256 sites at a time took 96 barriers).
 __global__ void __launch_bounds__(kRelThreads) k_root_ids(int32_t n, const int32_t *__restrict__ lab,
                                                           const int32_t *__restrict__ block_off,
                                                           int32_t *__restrict__ out, int32_t *__restrict__ sizes) {
     __shared__ int32_t s_w[kRelThreads / 32];
-    __shared__ int32_t s_run;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t base = (int64_t)blockIdx.x * kRelBlock;
-    if (threadIdx.x == 0) s_run = block_off[blockIdx.x];
-    __syncthreads();
+    const int64_t base = (int64_t)blockIdx.x * kRelBlock + warp * (32 * kRelPerThread) + lane;
+    static_assert(kRelPerThread == 32, "one ballot per lane");
+    unsigned mine = 0;                  // lane u: the roots among the warp's u-th 32 sites
+#pragma unroll 8
     for (int u = 0; u < kRelPerThread; ++u) {
-        const int64_t i = base + (int64_t)u * kRelThreads + threadIdx.x;
-        const bool root = i < n && __ldg(lab + i) == (int32_t)i;
-        const unsigned b = __ballot_sync(kFull, root);
-        if (lane == 0) s_w[warp] = __popc(b);
-        __syncthreads();
-        int before = s_run;
-        for (int w = 0; w < warp; ++w) before += s_w[w];
-        if (root) {
-            const int32_t id = before + __popc(b & ((1u << lane) - 1u));
-            out[i] = id;
+        const int64_t i = base + 32 * u;
+        const unsigned b = __ballot_sync(kFull, i < n && __ldg(lab + i) == (int32_t)i);
+        if (lane == u) mine = b;
+    }
+    int incl = __popc(mine);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += t;
+    }
+    if (lane == 31) s_w[warp] = incl;
+    __syncthreads();
+    int32_t off = block_off[blockIdx.x];
+    for (int w = 0; w < warp; ++w) off += s_w[w];
+    const int32_t before = off + incl - __popc(mine);
+    for (int u = 0; u < kRelPerThread; ++u) {
+        const unsigned b = __shfl_sync(kFull, mine, u);
+        const int32_t id = __shfl_sync(kFull, before, u) + __popc(b & ((1u << lane) - 1u));
+        if ((b >> lane) & 1u) {
+            out[base + 32 * u] = id;
             if (sizes) sizes[id] = 0;
         }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            int t = 0;
-            for (int w = 0; w < kRelThreads / 32; ++w) t += s_w[w];
-            s_run += t;
+    }
+}
+
+// Counts of a warp's values (cluster ids or labels), added to cnt[value] with
+// as few atomics as the values allow: lanes with the same value add once, and
+// the value that fills the warp (the giant cluster above the threshold) is
+// counted in a register until another takes its place. Without the register
+// every warp of the GPU adds to the giant cluster's counter, one address:
+// a realisation of honeycomb 2896^2 at 1.25 p_c (labelling, spanning, largest
+// cluster) took 845 us that way and 448 this way; relabelling triangle 4096^2
+// at 0.9 p_c, whose ids and sizes are one pass now, 205 and 118.
+// Tracks the largest (count, smallest value) key seen after an add.
+struct WarpCounter {
+    int32_t *cnt;
+    int32_t hot = -1;           // warp-uniform
+    int held = 0;
+    unsigned long long key = 0;
+
+    __device__ __forceinline__ explicit WarpCounter(int32_t *c) : cnt(c) {}
+    __device__ __forceinline__ void put(int32_t v, int c) {
+        const unsigned long long now = (unsigned)(atomicAdd(cnt + v, c) + c);
+        const unsigned long long k = (now << 32) | (0xffffffffu - (uint32_t)v);
+        key = k > key ? k : key;
+    }
+    // adds one of value v for every lane (v < 0: none); the whole warp calls
+    __device__ __forceinline__ void add(int32_t v, int lane) {
+        const bool is_hot = v >= 0 && v == hot;
+        const int hits = __popc(__ballot_sync(kFull, is_hot));
+        held += hits;
+        if (is_hot) v = -1;
+        if (!__any_sync(kFull, v >= 0)) return;
+        const unsigned peers = __match_any_sync(kFull, v);
+        const bool lead = v >= 0 && __ffs(peers) - 1 == lane;
+        const int c = __popc(peers);
+        // a value on more lanes than the held one's, and on at least a quarter
+        // of the warp, is held instead of it
+        const unsigned big = __reduce_max_sync(kFull, lead ? (unsigned)c * 32u + (unsigned)lane : 0u);
+        const bool swap = (int)(big >> 5) >= 8 && (int)(big >> 5) > hits;
+        const int by = (int)(big & 31u);
+        const int32_t next = __shfl_sync(kFull, v, by);
+        if (lead && !(swap && lane == by)) put(v, c);
+        if (swap) {
+            flush(lane);
+            hot = next;
+            held = (int)(big >> 5);
         }
-        __syncthreads();
     }
+    __device__ __forceinline__ void flush(int lane) {
+        if (lane == 0 && held > 0) put(hot, held);
+        held = 0;
+    }
+};
+
+// Sites [lo, hi) of this warp when n sites are cut into runs of whole 128-site
+// groups, one run per warp of the grid (consecutive sites share clusters, so a
+// run keeps its held value).
+__device__ __forceinline__ void warp_run(int64_t n, int64_t &lo, int64_t &hi) {
+    const int64_t groups = (n + 127) / 128, warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    const int64_t per = (groups + warps - 1) / warps;
+    const int64_t w = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    lo = min(w * per * 128, n);
+    hi = min((w + 1) * per * 128, n);
 }
 
-// every other site takes its root's id
-__global__ void k_site_ids(int32_t n, const int32_t *__restrict__ lab, int32_t *__restrict__ out) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        const int32_t l = __ldg(lab + i);
-        if (l != (int32_t)i) out[i] = out[l];
+// every other site takes its root's id; with sizes, every site is counted
+// under its id in the same pass
+__global__ void __launch_bounds__(256) k_site_ids(int32_t n, const int32_t *__restrict__ lab, int32_t *out,
+                                                  int32_t *__restrict__ sizes) {
+    const int lane = threadIdx.x & 31;
+    int64_t lo, hi;
+    warp_run(n, lo, hi);
+    WarpCounter wc(sizes);
+    for (int64_t g = lo; g < hi; g += 128) {
+        int32_t l[4], id[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int64_t i = g + 32 * u + lane;
+            l[u] = i < hi ? __ldg(lab + i) : -1;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) id[u] = l[u] >= 0 ? out[l[u]] : -1;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int64_t i = g + 32 * u + lane;
+            if (l[u] >= 0 && l[u] != (int32_t)i) out[i] = id[u];
+        }
+        if (sizes)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) wc.add((uint32_t)id[u] < (uint32_t)n ? id[u] : -1, lane);
     }
-}
-
-// cluster sizes; lanes of a warp holding the same id add once
-__global__ void k_sizes(int32_t n, const int32_t *__restrict__ out, int32_t *__restrict__ sizes) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x; i0 < n; i0 += stride) {
-        const int64_t i = i0 + threadIdx.x;
-        const int32_t id = i < n ? out[i] : -1;
-        const unsigned peers = __match_any_sync(kFull, id);
-        if (id >= 0 && (__ffs(peers) - 1) == (int)(threadIdx.x & 31)) atomicAdd(sizes + id, __popc(peers));
-    }
+    if (sizes) wc.flush(lane);
 }
 
 // spanning: mark the labels of the top sites, then look for them at the bottom
@@ -130,7 +206,7 @@ __global__ void k_span_mark(int32_t n, const int32_t *__restrict__ lab, const in
         if ((uint32_t)l >= (uint32_t)n) { atomicOr(err, kErrIndex); continue; }
         atomicOr(flags + (l >> 5), 1u << (l & 31));
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) *best = INT32_MAX;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *best = -1;     // none (the largest as unsigned)
 }
 
 __global__ void k_span_check(int32_t n, const int32_t *__restrict__ lab, const int32_t *__restrict__ bottom,
@@ -142,52 +218,97 @@ __global__ void k_span_check(int32_t n, const int32_t *__restrict__ lab, const i
         if ((uint32_t)s >= (uint32_t)n) { atomicOr(err, kErrIndex); continue; }
         const int32_t l = lab[s];
         if ((uint32_t)l >= (uint32_t)n) { atomicOr(err, kErrIndex); continue; }
-        if ((__ldg(flags + (l >> 5)) >> (l & 31)) & 1u) atomicMin(best, l);
+        if ((__ldg(flags + (l >> 5)) >> (l & 31)) & 1u) atomicMin((unsigned *)best, (unsigned)l);
     }
 }
 
-__global__ void k_span_finish(int32_t *best) {
-    if (*best == INT32_MAX) *best = -1;
+// The spanning test of few top sites in one launch: the top labels go into a
+// hash set in shared memory (open addressing, at most half full), the bottom
+// labels are looked up in it. Clearing a bit per site, marking, checking and
+// finishing took four launches.
+constexpr int kSpanTop = 8192;              // most top sites of this path
+constexpr int kSpanThreads = 1024;
+__global__ void __launch_bounds__(kSpanThreads) k_span_few(int32_t n, const int32_t *__restrict__ lab,
+                                                           const int32_t *__restrict__ top, int32_t n_top,
+                                                           const int32_t *__restrict__ bottom, int32_t n_bottom,
+                                                           int32_t slots, int32_t *__restrict__ best, unsigned *err) {
+    extern __shared__ int32_t s_set[];      // `slots`, a power of two, -1 where empty
+    __shared__ unsigned s_best;
+    for (int t = threadIdx.x; t < slots; t += kSpanThreads) s_set[t] = -1;
+    if (threadIdx.x == 0) s_best = 0xffffffffu;         // -1: no cluster spans
+    __syncthreads();
+    const unsigned mask = (unsigned)slots - 1u;
+    for (int t = threadIdx.x; t < n_top; t += kSpanThreads) {
+        const int32_t s = top[t];
+        const int32_t l = (uint32_t)s < (uint32_t)n ? lab[s] : -1;
+        if ((uint32_t)l >= (uint32_t)n) { atomicOr(err, kErrIndex); continue; }
+        unsigned h = ((unsigned)l * 2654435761u >> 16) & mask;
+        for (int probe = 0; probe < slots; ++probe, h = (h + 1u) & mask) {
+            const int32_t was = atomicCAS(&s_set[h], -1, l);
+            if (was == -1 || was == l) break;
+        }
+    }
+    __syncthreads();
+    unsigned mine = 0xffffffffu;
+    for (int t = threadIdx.x; t < n_bottom; t += kSpanThreads) {
+        const int32_t s = bottom[t];
+        const int32_t l = (uint32_t)s < (uint32_t)n ? lab[s] : -1;
+        if ((uint32_t)l >= (uint32_t)n) { atomicOr(err, kErrIndex); continue; }
+        if ((unsigned)l >= mine) continue;
+        unsigned h = ((unsigned)l * 2654435761u >> 16) & mask;
+        for (int probe = 0; probe < slots && s_set[h] != -1; ++probe, h = (h + 1u) & mask)
+            if (s_set[h] == l) { mine = (unsigned)l; break; }
+    }
+    mine = __reduce_min_sync(kFull, mine);
+    if ((threadIdx.x & 31) == 0) atomicMin(&s_best, mine);
+    __syncthreads();
+    if (threadIdx.x == 0) *best = (int32_t)s_best;
 }
 
 // Largest cluster (Section 4's largest-cluster statistic): cnt[l] = sites
-// whose canonical label is l (lanes holding the same label add once), then the
-// largest count over the roots, ties to the smallest label, as one 64-bit key
-// (count << 32) | (0xffffffff - label) under atomicMax.
-__global__ void k_label_counts(int32_t n, const int32_t *__restrict__ lab, int32_t *__restrict__ cnt,
-                               unsigned *err) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x; i0 < n; i0 += stride) {
-        const int64_t i = i0 + threadIdx.x;
-        int32_t l = i < n ? __ldg(lab + i) : -1;
-        if (i < n && (uint32_t)l >= (uint32_t)n) { atomicOr(err, kErrIndex); l = -1; }
-        const unsigned peers = __match_any_sync(kFull, l);
-        if (l >= 0 && (__ffs(peers) - 1) == (int)(threadIdx.x & 31)) atomicAdd(cnt + l, __popc(peers));
-    }
-}
-
-__global__ void k_largest(int32_t n, const int32_t *__restrict__ cnt, unsigned long long *__restrict__ best) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    unsigned long long key = 0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        const int32_t c = __ldg(cnt + i);
-        if (c > 0) {
-            const unsigned long long k = ((unsigned long long)(uint32_t)c << 32) | (0xffffffffu - (uint32_t)i);
-            key = k > key ? k : key;
+// whose canonical label is l. Every add returns the count so far, and the last
+// add of a label its size, so the largest (size, smallest label) key over all
+// adds is the answer: no pass over the counters. The last CTA to finish
+// writes the result. (scratch: the best key, the finished CTAs.)
+struct LargestScratch {
+    unsigned long long best;
+    unsigned done, pad_;
+};
+__global__ void __launch_bounds__(256) k_largest(int32_t n, const int32_t *__restrict__ lab, int32_t *__restrict__ cnt,
+                                                 LargestScratch *scratch, int32_t *__restrict__ result, unsigned *err) {
+    const int lane = threadIdx.x & 31;
+    int64_t lo, hi;
+    warp_run(n, lo, hi);
+    WarpCounter wc(cnt);
+    bool bad = false;
+    for (int64_t g = lo; g < hi; g += 128) {
+        int32_t l[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int64_t i = g + 32 * u + lane;
+            l[u] = i < hi ? __ldg(lab + i) : -1;
+            bad |= i < hi && (uint32_t)l[u] >= (uint32_t)n;
         }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) wc.add((uint32_t)l[u] < (uint32_t)n ? l[u] : -1, lane);
     }
+    wc.flush(lane);
+    if (bad) atomicOr(err, kErrIndex);
+    unsigned long long key = wc.key;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         const unsigned long long t = __shfl_xor_sync(kFull, key, o);
         key = t > key ? t : key;
     }
-    if ((threadIdx.x & 31) == 0 && key) atomicMax(best, key);
-}
-
-__global__ void k_largest_finish(const unsigned long long *best, int32_t *result) {
-    const unsigned long long k = *best;
-    result[0] = (int32_t)(k >> 32);
-    result[1] = k ? (int32_t)(0xffffffffu - (uint32_t)(k & 0xffffffffu)) : -1;
+    if (lane == 0 && key > *(volatile unsigned long long *)&scratch->best) atomicMax(&scratch->best, key);
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(&scratch->done, 1u) == gridDim.x - 1) {
+        __threadfence();
+        const unsigned long long k = atomicMax(&scratch->best, 0ull);
+        result[0] = (int32_t)(k >> 32);
+        result[1] = k ? (int32_t)(0xffffffffu - (uint32_t)(k & 0xffffffffu)) : -1;
+    }
 }
 
 }  // namespace ccl
