@@ -164,8 +164,8 @@ int blocks_per_sm(ccl_context *ctx, int kernel_id, int threads) {
         case 6: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_init<false, true>, kInitThreads, kInitSmem); break;
         case 7: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_init_dense<false>, kDenseThreads, 0); break;
         case 8: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_init_dense<true>, kDenseThreads, 0); break;
-        case 9: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_init_dense_tma<false>, kDenseTmaThreads, kDenseSmem); break;
-        case 10: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_init_dense_tma<true>, kDenseTmaThreads, kDenseSmem); break;
+        case 9: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_init_dense_tma<false>, kInitThreads, kDenseSmem); break;
+        case 10: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_init_dense_tma<true>, kInitThreads, kDenseSmem); break;
         case 11: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_analysis_park<false>, 32 * kParkWarps, 0); break;
         case 12: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_analysis_park<true>, 32 * kParkWarps, 0); break;
         default: break;
@@ -328,7 +328,7 @@ TuneChoice choice_for(ccl_context *ctx, int64_t n, int64_t nnz) {
 int64_t init_grid(ccl_context *ctx, const Params &P, bool batched, int64_t max_bands) {
     const bool gen = P.gen_thr != kNoGen;
     int64_t g;
-    if (P.dense && P.nn_width <= kRowRegs) g = grid_init(ctx, gen ? 10 : 9, kDenseTmaThreads, P.n_tiles);
+    if (P.dense && P.nn_width <= kRowRegs) g = grid_init(ctx, gen ? 10 : 9, kInitThreads, P.n_tiles);
     else if (P.dense) g = grid_init(ctx, gen ? 8 : 7, kDenseThreads, P.n_tiles);
     else g = grid_init(ctx, batched ? 1 : (gen ? 6 : 0), kInitThreads, P.n_tiles);
     if (g > max_bands) {     // fewer, longer bands
@@ -370,8 +370,8 @@ ccl_status launch_init(const Params &P, bool batched, int64_t g, cudaStream_t s)
     const bool gen = P.gen_thr != kNoGen;
     if (P.init_bands > g) CCL_CUDA(cudaMemsetAsync(P.ticket, 0, sizeof(unsigned), s));
     if (P.dense && P.nn_width <= kRowRegs) {
-        if (gen) k_init_dense_tma<true><<<(unsigned)g, kDenseTmaThreads, kDenseSmem, s>>>(P);
-        else k_init_dense_tma<false><<<(unsigned)g, kDenseTmaThreads, kDenseSmem, s>>>(P);
+        if (gen) k_init_dense_tma<true><<<(unsigned)g, kInitThreads, kDenseSmem, s>>>(P);
+        else k_init_dense_tma<false><<<(unsigned)g, kInitThreads, kDenseSmem, s>>>(P);
     } else if (P.dense) {
         if (gen) k_init_dense<true><<<(unsigned)g, kDenseThreads, 0, s>>>(P);
         else k_init_dense<false><<<(unsigned)g, kDenseThreads, 0, s>>>(P);
@@ -591,7 +591,7 @@ ccl_status run(ccl_context *ctx, Params P, bool batched, const TuneChoice &tc, c
                const std::vector<Inst> *table, uint64_t shape_hash, bool allow_graph = true,
                const std::vector<int64_t> *offsets = nullptr) {
     for (int kid = 0; kid < 13; ++kid)
-        (void)blocks_per_sm(ctx, kid, kid >= 11 ? 32 * kParkWarps : kid >= 9 ? kDenseTmaThreads : kid >= 7 ? kDenseThreads
+        (void)blocks_per_sm(ctx, kid, kid >= 11 ? 32 * kParkWarps : kid >= 9 ? kInitThreads : kid >= 7 ? kDenseThreads
                                                : (kid < 2 || kid == 6) ? kInitThreads : (kid >= 4 ? 256 : tc.threads));
     ctx->last.used_graph = 0;
     const bool capturing = stream_capturing(s);

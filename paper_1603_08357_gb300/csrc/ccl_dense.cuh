@@ -185,9 +185,12 @@ __global__ void __launch_bounds__(kDenseThreads) k_init_dense(Params P) {
 // kRowRegs slots, a producer lane streams each 1024-site tile's W slot slabs
 // (slot k: the tile's sites' entries nn[s0 + k*N ...], contiguous) and their
 // bit words into a 3-stage shared-memory ring with bulk asynchronous copies;
-// 16 consumer warps scan two 32-site chunks each, store labels after both are
-// scanned (the band shortcut's load overlaps the second scan) and append the
-// residual pairs of both through one prefix sum.
+// eight consumer warps scan four 32-site chunks each (k_init's scan on slots),
+// store the labels after all are scanned and append the residual pairs of all
+// through one prefix sum. As in k_init the scan's instructions bound it:
+// against sixteen warps of two chunks, step (i) of the cubic lattice 200^3 (8M
+// sites, six slots) went from 105 to 89 us, and to 66 with the producer's work
+// spread over its lanes (below).
 
 constexpr int kDenseSlab = kTileSites + 8;        // a slot's slab, + 16-byte rounding
 constexpr int kDenseWords = kTileSites / 32 + 8;  // its bit words, + rounding
@@ -212,8 +215,12 @@ struct __align__(16) DenseStage {
 
 constexpr size_t kDenseSmem = 64 + sizeof(DenseStage) * kStages;
 
+// The producer warp: lane k computes and issues slot k's two copies. (One lane
+// working through the slots took longer than the consumers: 3.4 us a tile of
+// six slots, now 2.6.)
 template <bool kGen>
-__device__ __forceinline__ void dense_produce(const Params &P, DenseStage *st, uint64_t *full, uint64_t *empty) {
+__device__ __forceinline__ void dense_produce(const Params &P, DenseStage *st, uint64_t *full, uint64_t *empty,
+                                              int lane) {
     int64_t band_lo, band_hi;
     cta_band(P, band_lo, band_hi);
     const int64_t n = P.one.n;
@@ -222,54 +229,53 @@ __device__ __forceinline__ void dense_produce(const Params &P, DenseStage *st, u
     const int32_t *nn_end = P.nn + (int64_t)W * n;
     const uint32_t *bits_end = kGen ? nullptr : P.one.bits + n_words;
     const int64_t qband = min(band_lo * kTileSites, n) * W;
-    if (band_lo < band_hi) P.band[P.band_off + blockIdx.x].qbase = qband;
+    if (lane == 0 && band_lo < band_hi) P.band[P.band_off + blockIdx.x].qbase = qband;
     int64_t t_local = 0;
     for (int64_t tile = band_lo; tile < band_hi; ++tile, ++t_local) {
         const int s = (int)(t_local % kStages);
         const int64_t use = t_local / kStages;
-        if (use > 0 && !mbar_wait_bounded(&empty[s], (uint32_t)((use - 1) & 1))) {
-            raise_err(P.err, kErrNonconv);
+        if (use > 0 && !__all_sync(kFull, mbar_wait_bounded(&empty[s], (uint32_t)((use - 1) & 1)))) {
+            if (lane == 0) raise_err(P.err, kErrNonconv);
             break;
         }
-        DenseStageHdr &h = st[s].h;
+        DenseStage &T = st[s];
+        DenseStageHdr &h = T.h;
         const int64_t s0 = tile * kTileSites;
         const int64_t ts = min((int64_t)kTileSites, n - s0);
-        h.s0 = (int32_t)s0;
-        h.ts = (int32_t)ts;
-        h.qband = qband;
-        uint32_t bytes = 0;
-        int staged = 1;
-        for (int k = 0; k < W; ++k) {
-            const int64_t e0 = s0 + (int64_t)k * n, e1 = e0 + ts;
-            int64_t lo, hi;
-            copy_window(P.nn, e0, e1, P.nn, nn_end, kDenseSlab, lo, hi);
-            h.nn_lo[k] = lo;
-            h.nn_cnt[k] = (int32_t)(hi - lo);
-            staged &= lo <= e0 && hi >= e1;
-            bytes += 4u * (uint32_t)(hi - lo);
+        int64_t nn_lo = 0, nn_hi = 0, w_lo = 0, w_hi = 0;
+        bool staged = true;
+        if (lane < W) {
+            const int64_t e0 = s0 + (int64_t)lane * n, e1 = e0 + ts;
+            copy_window(P.nn, e0, e1, P.nn, nn_end, kDenseSlab, nn_lo, nn_hi);
+            staged = nn_lo <= e0 && nn_hi >= e1;
             if (!kGen) {
                 const int64_t w0 = e0 >> 5, w1 = ((e1 - 1) >> 5) + 1;
-                copy_window(P.one.bits, w0, w1, P.one.bits, bits_end, kDenseWords, lo, hi);
-                h.w_lo[k] = lo;
-                h.w_cnt[k] = (int32_t)(hi - lo);
-                staged &= lo <= w0 && hi >= w1;
-                bytes += 4u * (uint32_t)(hi - lo);
+                copy_window(P.one.bits, w0, w1, P.one.bits, bits_end, kDenseWords, w_lo, w_hi);
+                staged = staged && w_lo <= w0 && w_hi >= w1;
             }
+            h.nn_lo[lane] = nn_lo;
+            h.nn_cnt[lane] = (int32_t)(nn_hi - nn_lo);
+            h.w_lo[lane] = w_lo;
+            h.w_cnt[lane] = (int32_t)(w_hi - w_lo);
+            if (staged) h.off[lane] = make_int2((int32_t)(e0 - nn_lo), kGen ? 0 : (int32_t)(e0 - 32 * w_lo));
         }
-        h.staged = staged;
-        if (staged)
-            for (int k = 0; k < W; ++k) {
-                const int64_t e0 = s0 + (int64_t)k * n;
-                h.off[k] = make_int2((int32_t)(e0 - h.nn_lo[k]), kGen ? 0 : (int32_t)(e0 - 32 * h.w_lo[k]));
-            }
-        mbar_arrive_expect_tx(&full[s], bytes);
-        for (int k = 0; k < W; ++k) {
-            if (h.nn_cnt[k]) bulk_g2s(st[s].nn[k], P.nn + h.nn_lo[k], 4u * (uint32_t)h.nn_cnt[k], &full[s]);
-            if (!kGen && h.w_cnt[k])
-                bulk_g2s(st[s].bw[k], P.one.bits + h.w_lo[k], 4u * (uint32_t)h.w_cnt[k], &full[s]);
+        const uint32_t b_nn = 4u * (uint32_t)(nn_hi - nn_lo), b_w = 4u * (uint32_t)(w_hi - w_lo);
+        const uint32_t bytes = __reduce_add_sync(kFull, b_nn + b_w);
+        staged = __all_sync(kFull, staged);
+        __syncwarp();                   // the lanes' header fields come before the barrier's release
+        if (lane == 0) {
+            h.s0 = (int32_t)s0;
+            h.ts = (int32_t)ts;
+            h.qband = qband;
+            h.staged = staged ? 1 : 0;
+            mbar_arrive_expect_tx(&full[s], bytes);
         }
+        __syncwarp();
+        if (b_nn) bulk_g2s(T.nn[lane], P.nn + nn_lo, b_nn, &full[s]);
+        if (b_w) bulk_g2s(T.bw[lane], P.one.bits + w_lo, b_w, &full[s]);
     }
-    drain_armed(full, t_local, P.err);
+    if (lane == 0) drain_armed(full, t_local, P.err);
+    __syncwarp();
 }
 
 // one lane's site of a staged chunk: slot k's neighbour and its open bit
@@ -289,9 +295,9 @@ __device__ __forceinline__ void dense_slot(const Params &P, const DenseStage &S,
 }
 
 struct DenseChunk {
-    int32_t i, lab, m;
+    int32_t i, lab;
     uint32_t lowmask;       // open lower slots
-    int32_t mk, r;
+    int32_t r;
 };
 
 template <bool kGen>
@@ -347,67 +353,87 @@ __device__ __forceinline__ void dense_scan_chunk(const Params &P, const DenseSta
     }
     c.i = i;
     c.lab = lab;
-    c.m = m;
-    c.mk = mk;
     c.lowmask = cnt ? (lowmask & ~(1u << mk)) : 0u;
     c.r = cnt > 1 ? cnt - 1 : 0;
 }
 
-// Both chunks of a consumer warp at once on a staged tile whose two chunks
-// are full: each slot's header offsets are read once and the two chunks'
-// loads interleave. Returns false (having done nothing) otherwise.
-template <bool kGen>
-__device__ __forceinline__ bool dense_scan_pair(const Params &P, const DenseStage &S, int cc0, int lane,
-                                                const TileCtx &tc, DenseChunk &c0, DenseChunk &c1) {
+// The four chunks of a consumer warp at once, on a staged tile that has them
+// whole: slot k of the lane's sites i0 + 32 c. Keys, place bits and kWide as in
+// scan_rows (bit W - 1 - k of `low` is slot k).
+struct DenseRows {
+    int32_t lab[kRows];
+    uint32_t res;           // residual slots: slot k of row c at bit 8 c + W - 1 - k
+};
+
+template <bool kGen, bool kWide>
+__device__ __forceinline__ void dense_scan_rows(const Params &P, const DenseStage &S, int loc0, const TileCtx &tc,
+                                                DenseRows &q) {
     const DenseStageHdr &h = S.h;
-    const int64_t n = P.one.n;
+    const uint32_t n = (uint32_t)P.one.n;
     const int W = (int)P.nn_width;
-    const int32_t loc0 = cc0 * kChunk + lane, loc1 = loc0 + kChunk;
-    if (!tc.staged || (cc0 + 2) * kChunk > h.ts) return false;
-    const int32_t i0 = h.s0 + loc0, i1 = i0 + kChunk;
-    int32_t m0 = INT32_MAX, m1 = INT32_MAX, k0 = 0, k1 = 0;
-    uint32_t l0 = 0, l1 = 0;
-    bool bad = false;
+    const int32_t i0 = h.s0 + loc0;
+    uint32_t low[kRows], at[kRows], jmax = 0;
+    int32_t m[kRows];
+#pragma unroll
+    for (int c = 0; c < kRows; ++c) {
+        low[c] = at[c] = 0;
+        m[c] = INT32_MAX;
+    }
 #pragma unroll
     for (int k = 0; k < kRowRegs; ++k) {
         if (k >= W) break;
         const int2 off = h.off[k];
-        const int32_t j0 = S.nn[k][off.x + loc0], j1 = S.nn[k][off.x + loc1];
-        bool o0, o1;
-        if (kGen) {
-            o0 = (uint32_t)j0 < (uint32_t)i0 && gen_bond_open(P.gen_seed, P.gen_thr, (uint32_t)j0, (uint32_t)i0);
-            o1 = (uint32_t)j1 < (uint32_t)i1 && gen_bond_open(P.gen_seed, P.gen_thr, (uint32_t)j1, (uint32_t)i1);
-        } else {
-            const int32_t b0 = off.y + loc0, b1 = b0 + kChunk;
-            o0 = (S.bw[k][b0 >> 5] >> (b0 & 31)) & 1u;
-            o1 = (S.bw[k][b1 >> 5] >> (b1 & 31)) & 1u;
-        }
-        bad |= (uint32_t)(j0 + 1) > (uint32_t)n || (uint32_t)(j1 + 1) > (uint32_t)n;
-        if (o0 && (uint32_t)j0 < (uint32_t)i0) {
-            l0 |= 1u << k;
-            if (j0 < m0) { m0 = j0; k0 = k; }
-        }
-        if (o1 && (uint32_t)j1 < (uint32_t)i1) {
-            l1 |= 1u << k;
-            if (j1 < m1) { m1 = j1; k1 = k; }
+        const int32_t *nn = S.nn[k] + off.x + loc0;
+        const int32_t b = off.y + loc0;
+        const uint32_t *bw = S.bw[k] + (b >> 5);        // the lane's bit of chunk c: bit b & 31 of bw[c]
+#pragma unroll
+        for (int c = 0; c < kRows; ++c) {
+            const int32_t i = i0 + kChunk * c;
+            const int32_t j = nn[kChunk * c];           // -1: an empty slot, whatever its bit
+            jmax = max(jmax, (uint32_t)j + 1u);
+            const bool open = kGen ? (uint32_t)j < (uint32_t)i &&
+                                         gen_bond_open(P.gen_seed, P.gen_thr, (uint32_t)j, (uint32_t)i)
+                                   : ((bw[c] >> (b & 31)) & 1u) && j >= 0;
+            if (kWide) {
+                const bool lower = open && (uint32_t)j < (uint32_t)i;
+                low[c] = 2u * low[c] + (lower ? 1u : 0u);
+                if (lower && j < m[c]) { m[c] = j; at[c] = (uint32_t)k; }
+            } else {
+                const int32_t key = open ? (int32_t)(8u * (uint32_t)j + (uint32_t)k) : INT32_MAX;
+                m[c] = min(m[c], key);
+                low[c] = __funnelshift_l((uint32_t)key - 8u * (uint32_t)i, low[c], 1);
+            }
         }
     }
+    const bool bad = jmax > n;          // j < -1 or j >= n
     if (bad) raise_err(P.err, kErrIndex);
-    const int n0 = __popc(l0), n1 = __popc(l1);
-    int32_t lab0 = n0 ? m0 : i0, lab1 = n1 ? m1 : i1;
-    if (n0) {
-        const int32_t mt = (int32_t)((uint32_t)m0 / kTileSites);
-        if (mt >= tc.vis_lo && mt <= tc.vis_hi) lab0 = __ldcg(P.one.labels + m0);
+    q.res = 0;
+#pragma unroll
+    for (int c = 0; c < kRows; ++c) {
+        const bool any = low[c] != 0 && !bad;
+        const int place = kWide ? (int)at[c] : m[c] & 7;
+        q.lab[c] = any ? (kWide ? m[c] : m[c] >> 3) : i0 + kChunk * c;
+        if (any) q.res |= (low[c] & ~(1u << (W - 1 - place))) << (8 * c);
     }
-    if (n1) {
-        const int32_t mt = (int32_t)((uint32_t)m1 / kTileSites);
-        if (mt >= tc.vis_lo && mt <= tc.vis_hi) lab1 = __ldcg(P.one.labels + m1);
+    jump_and_shortcut(P.one.labels, h.s0 + (loc0 & ~31), tc, q.lab);
+}
+
+template <bool kGen>
+__device__ __forceinline__ void dense_emit_rows(const Params &P, const DenseStage &S, const DenseRows &q, int loc0,
+                                                int64_t slot, int rr) {
+    const int iters = (int)__reduce_max_sync(kFull, (uint32_t)rr);
+    const int last = (int)P.nn_width - 1;
+    uint32_t mm = q.res;
+    int2 *qp = P.q + slot;
+    for (int it = 0; it < iters; ++it) {
+        if (mm) {
+            const int t = __ffs(mm) - 1;
+            mm &= mm - 1;
+            const int k = last - (t & 7);
+            const int32_t up = t & 8 ? q.lab[1] : q.lab[0], up2 = t & 8 ? q.lab[3] : q.lab[2];
+            *qp++ = make_int2(t & 16 ? up2 : up, S.nn[k][S.h.off[k].x + loc0 + kChunk * (t >> 3)]);
+        }
     }
-    c0.i = i0; c0.lab = lab0; c0.m = m0; c0.mk = k0;
-    c0.lowmask = n0 ? (l0 & ~(1u << k0)) : 0u; c0.r = n0 > 1 ? n0 - 1 : 0;
-    c1.i = i1; c1.lab = lab1; c1.m = m1; c1.mk = k1;
-    c1.lowmask = n1 ? (l1 & ~(1u << k1)) : 0u; c1.r = n1 > 1 ? n1 - 1 : 0;
-    return true;
 }
 
 template <bool kGen>
@@ -431,7 +457,7 @@ __device__ __forceinline__ void dense_emit_chunk(const Params &P, const DenseSta
 }
 
 template <bool kGen>
-__global__ void __launch_bounds__(kDenseTmaThreads, 2) k_init_dense_tma(Params P) {
+__global__ void __launch_bounds__(kInitThreads, kInitCtas) k_init_dense_tma(Params P) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     uint64_t *full = reinterpret_cast<uint64_t *>(smem_raw);
     uint64_t *empty = full + kStages;
@@ -441,15 +467,15 @@ __global__ void __launch_bounds__(kDenseTmaThreads, 2) k_init_dense_tma(Params P
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
             mbar_init(&full[s], 1);
-            mbar_init(&empty[s], kDenseConsumers);
+            mbar_init(&empty[s], kInitConsumers);
         }
         mbar_fence_init();
     }
     __shared__ unsigned long long band_cnt;
     if (threadIdx.x == 0) band_cnt = 0;
     __syncthreads();
-    if (warp == kDenseConsumers) {
-        if (lane == 0) dense_produce<kGen>(P, st, full, empty);
+    if (warp == kInitConsumers) {
+        dense_produce<kGen>(P, st, full, empty, lane);
         return;
     }
     int64_t band_lo, band_hi;
@@ -471,31 +497,57 @@ __global__ void __launch_bounds__(kDenseTmaThreads, 2) k_init_dense_tma(Params P
             tc.vis_lo = (int32_t)band_lo;
             tc.vis_hi = hi < band_lo ? -1 : (int32_t)hi;
         }
-        const int cc0 = warp * 2, cc1 = warp * 2 + 1;
-        DenseChunk c0, c1;
-        c0.r = c1.r = 0;
-        const bool has0 = cc0 * kChunk < S.h.ts, has1 = cc1 * kChunk < S.h.ts;
-        if (!(has1 && dense_scan_pair<kGen>(P, S, cc0, lane, tc, c0, c1))) {
-            if (has0) dense_scan_chunk<kGen>(P, S, cc0, lane, tc, c0);
-            if (has1) dense_scan_chunk<kGen>(P, S, cc1, lane, tc, c1);
-        }
-        if (has0 && c0.i < P.one.n) P.one.labels[c0.i] = c0.lab;
-        if (has1 && c1.i < P.one.n) P.one.labels[c1.i] = c1.lab;
-        const int rr = c0.r + c1.r;
-        const int incl = warp_incl_scan(rr, lane);
-        const int total = __shfl_sync(kFull, incl, 31);
-        if (total > 0) {
+        const int loc = warp * kRows * kChunk, loc0 = loc + lane;       // the warp's first site, the lane's
+        if (loc < S.h.ts) {
+            DenseRows q;
+            DenseChunk c[kRows];
+            const bool fast = tc.staged && loc + kRows * kChunk <= S.h.ts;
+            int rr = 0;
+            if (fast) {
+                if (P.one.n > (1 << 28)) dense_scan_rows<kGen, true>(P, S, loc0, tc, q);
+                else dense_scan_rows<kGen, false>(P, S, loc0, tc, q);
+                rr = __popc(q.res);
+            } else {
+#pragma unroll
+                for (int k = 0; k < kRows; ++k) {
+                    c[k].r = 0;
+                    if (loc + k * kChunk < S.h.ts) dense_scan_chunk<kGen>(P, S, warp * kRows + k, lane, tc, c[k]);
+                    rr += c[k].r;
+                }
+            }
+            const int incl = warp_incl_scan(rr, lane);
+            const int total = __shfl_sync(kFull, incl, 31);
             unsigned long long base = 0;
-            if (lane == 0) base = atomicAdd(&band_cnt, (unsigned long long)total);
-            base = __shfl_sync(kFull, base, 0);
-            const int64_t slot = S.h.qband + (int64_t)base + (incl - rr);
-            if (c0.r > 0) dense_emit_chunk<kGen>(P, S, c0, tc.staged, slot);
-            if (c1.r > 0) dense_emit_chunk<kGen>(P, S, c1, tc.staged, slot + c0.r);
+            if (total > 0) {
+                if (lane == 0) base = atomicAdd(&band_cnt, (unsigned long long)total);
+                base = __shfl_sync(kFull, base, 0);
+            }
+            if (fast) {
+                int32_t *out = P.one.labels + S.h.s0 + loc0;
+#pragma unroll
+                for (int k = 0; k < kRows; ++k) out[kChunk * k] = q.lab[k];
+            } else {
+#pragma unroll
+                for (int k = 0; k < kRows; ++k)
+                    if (loc + k * kChunk < S.h.ts && c[k].i < P.one.n) P.one.labels[c[k].i] = c[k].lab;
+            }
+            if (total > 0) {
+                int64_t slot = S.h.qband + (int64_t)base + (incl - rr);
+                if (fast) {
+                    dense_emit_rows<kGen>(P, S, q, loc0, slot, rr);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < kRows; ++k) {
+                        if (c[k].r > 0) dense_emit_chunk<kGen>(P, S, c[k], tc.staged, slot);
+                        slot += c[k].r;
+                    }
+                }
+            }
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&empty[s]);
     }
-    consumers_sync<32 * kDenseConsumers>();
+    consumers_sync<32 * kInitConsumers>();
     if (threadIdx.x == 0) P.band[P.band_off + blockIdx.x].cnt = band_cnt;
 }
 

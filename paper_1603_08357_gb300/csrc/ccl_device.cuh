@@ -586,6 +586,28 @@ __device__ __forceinline__ void scan_rows(const Params &P, const Stage &S, const
     }
 }
 
+// The labels of a warp's four chunks from site s00 on before they are stored.
+__device__ __forceinline__ void jump_and_shortcut(const int32_t *labels, int32_t s00, const TileCtx &tc,
+                                                  int32_t (&lab)[kRows]) {
+    // One pointer jump inside each chunk: a label that points to a site of the
+    // chunk takes that site's label. The value taken is an ancestor of the
+    // site, so it stays a valid label, and a chain along a lattice row shortens
+    // by half before step (iii) and the analysis follow it.
+#pragma unroll
+    for (int k = 0; k < kRows; ++k) {
+        const uint32_t in = (uint32_t)(lab[k] - (s00 + kChunk * k));
+        const int32_t up = __shfl_sync(kFull, lab[k], (int)(in & 31u));
+        if (in < 32u) lab[k] = up;
+    }
+    // a label in a tile of this band finished kStages tiles ago: take that
+    // site's label (the band shortcut)
+    const uint32_t vis_lo = (uint32_t)tc.vis_lo * kTileSites;
+    const uint32_t vis_n = tc.vis_hi < tc.vis_lo ? 0u : (uint32_t)(tc.vis_hi + 1 - tc.vis_lo) * kTileSites;
+#pragma unroll
+    for (int k = 0; k < kRows; ++k)
+        if ((uint32_t)lab[k] - vis_lo < vis_n) lab[k] = __ldcg(labels + lab[k]);
+}
+
 // The four chunks of a consumer warp at once, when all their rows exist, are
 // short and staged (the common case). Returns false (having done nothing)
 // otherwise.
@@ -628,23 +650,7 @@ __device__ __forceinline__ bool init_scan_rows(const Params &P, const Stage &S, 
         else scan_rows<kGen, 0>(P, S, tc, h, n, s00, lane, a, d, dmax, q, bad);
     }
     if (bad) raise_err(P.err, kErrIndex);
-    // One pointer jump inside each chunk: a label that points to a site of the
-    // chunk takes that site's label. The value taken is an ancestor of the
-    // site, so it stays a valid label, and a chain along a lattice row shortens
-    // by half before step (iii) and the analysis follow it.
-#pragma unroll
-    for (int k = 0; k < kRows; ++k) {
-        const uint32_t in = (uint32_t)(q.lab[k] - (s00 + kChunk * k));
-        const int32_t up = __shfl_sync(kFull, q.lab[k], (int)(in & 31u));
-        if (in < 32u) q.lab[k] = up;
-    }
-    // a label in a tile of this band finished kStages tiles ago: take that
-    // site's label (the band shortcut)
-    const uint32_t vis_lo = (uint32_t)tc.vis_lo * kTileSites;
-    const uint32_t vis_n = tc.vis_hi < tc.vis_lo ? 0u : (uint32_t)(tc.vis_hi + 1 - tc.vis_lo) * kTileSites;
-#pragma unroll
-    for (int k = 0; k < kRows; ++k)
-        if ((uint32_t)q.lab[k] - vis_lo < vis_n) q.lab[k] = __ldcg(I.labels + q.lab[k]);
+    jump_and_shortcut(I.labels, s00, tc, q.lab);
     return true;
 }
 

@@ -19,9 +19,6 @@ constexpr int kInitConsumers = kTileSites / kChunk / kRows;
 constexpr int kInitThreads = 32 * (kInitConsumers + 1);
 constexpr int kStages = 3;
 constexpr int kInitCtas = 2;               // CTAs per SM (their stages fill the shared memory)
-// the dense list's kernel: sixteen consumer warps of two chunks
-constexpr int kDenseConsumers = 16;
-constexpr int kDenseTmaThreads = 32 * (kDenseConsumers + 1);
 constexpr int kColCap = 7168;              // column entries a stage holds (7 per site)
 constexpr int kRpBuf = kTileSites + 8;     // row pointers of a tile, + 16-byte rounding
 constexpr int kColBuf = kColCap + 8;
