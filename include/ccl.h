@@ -110,23 +110,22 @@ typedef enum {
                                   without locality) */
     CCL_OPT_ITER_CAP = 8,      /* 0 (default): the loops of steps (ii)-(iv) stop only at caps
                                   derived from the input size, which a valid input never reaches.
-                                  v > 0: a chase of step (ii)/(iv) gives up after v iterations and
-                                  a warp of step (iii) abandons its window after v rounds, latching
+                                  v > 0: a chase of step (ii)/(iv) gives up after v iterations
+                                  (two at least) and a warp of step (iii) abandons its window after v rounds, latching
                                   CCL_ERR_NONCONVERGED (ccl_sync); the labels are then incomplete.
                                   For testing the failure path; setting it drops cached graphs. */
     CCL_OPT_REDUCE_WINDOW = 9, /* step (iii): most residual pairs a warp drains per window
                                   (64..65536); 0 (default): 2048 when the call's labels fit in
                                   three quarters of L2, else 512 */
     CCL_OPT_ANALYSIS_GROUP = 10, /* steps (ii)/(iv) in contiguous order: G > 0 visits the sites in
-                                  super-chunks, every warp taking its next G groups of 64 sites
+                                  super-chunks, every warp taking its next G groups of 96 sites
                                   of each, so the labels in use stay in L2; 0 one range per
                                   warp; -1 (default): 0 when the call's labels fit in three
                                   quarters of L2, else 16 */
     CCL_OPT_ANALYSIS_PARK = 11 /* steps (ii)/(iv) in contiguous order: 1 chains still unfinished
                                   after 4 rounds are set aside and finished 32 at a time, one per
                                   lane; 0 every warp runs its longest chain to the end; -1
-                                  (default): 1 when the call's labels fit in three quarters of
-                                  L2, else 0 */
+                                  (default): 0 */
 } ccl_option;
 
 CCL_API ccl_status ccl_set_option(ccl_context *ctx, int option, int64_t value);

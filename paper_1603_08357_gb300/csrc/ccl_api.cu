@@ -33,7 +33,7 @@ struct TuneChoice {
     int ana_seq = 1;        // steps (ii)/(iv): 1 contiguous ranges per warp, 0 interleaved
     int red_window = 0;     // step (iii): most pairs per warp window; 0 by size (see resolve_tail)
     int ana_group = -1;     // steps (ii)/(iv), contiguous order: super-chunk run length; -1 by size
-    int ana_park = -1;      // steps (ii)/(iv), contiguous order: 1 park long chains, 0 not; -1 by size
+    int ana_park = -1;      // steps (ii)/(iv), contiguous order: 1 set long chains aside, 0 not; -1 not
 };
 
 struct GraphEntry {
@@ -148,6 +148,9 @@ struct DeviceGuard {
 };
 
 
+// Dynamic shared memory of the analysis kernel that sets long chains aside.
+size_t park_smem(int threads) { return (size_t)(threads / 32) * 2 * kParkCap * sizeof(int); }
+
 int blocks_per_sm(ccl_context *ctx, int kernel_id, int threads) {
     auto key = std::make_pair(kernel_id, threads);
     auto it = ctx->occ.find(key);
@@ -157,8 +160,8 @@ int blocks_per_sm(ccl_context *ctx, int kernel_id, int threads) {
     switch (kernel_id) {
         case 0: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_init<false>, kInitThreads, kInitSmem); break;
         case 1: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_init<true>, kInitThreads, kInitSmem); break;
-        case 2: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_analysis<false, true>, threads, 0); break;
-        case 3: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_analysis<true, true, kAnaChunksBatched>, threads, 0); break;
+        case 2: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_analysis<false, false>, threads, 0); break;
+        case 3: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_analysis<true, false>, threads, 0); break;
         case 4: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_reduce<false, true>, threads, 0); break;
         case 5: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_reduce<true, true>, threads, 0); break;
         case 6: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_init<false, true>, kInitThreads, kInitSmem); break;
@@ -166,8 +169,8 @@ int blocks_per_sm(ccl_context *ctx, int kernel_id, int threads) {
         case 8: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_init_dense<true>, kDenseThreads, 0); break;
         case 9: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_init_dense_tma<false>, kInitThreads, kDenseSmem); break;
         case 10: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_init_dense_tma<true>, kInitThreads, kDenseSmem); break;
-        case 11: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_analysis_park<false>, 32 * kParkWarps, 0); break;
-        case 12: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_analysis_park<true>, 32 * kParkWarps, 0); break;
+        case 11: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_analysis<false, true>, threads, park_smem(threads)); break;
+        case 12: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_analysis<true, true>, threads, park_smem(threads)); break;
         default: break;
     }
     if (e != cudaSuccess || nb < 1) { (void)cudaGetLastError(); nb = 1; }
@@ -401,11 +404,10 @@ void resolve_tail(const ccl_context *ctx, const TuneChoice &tc, Params &P) {
     P.ana_group = tc.ana_group >= 0 ? tc.ana_group : (fits ? 0 : 16);
 }
 
-// Parking of long chains in steps (ii)/(iv) (contiguous order only): explicit
-// setting, else on when the call's labels fit in three quarters of L2.
-bool resolve_park(const ccl_context *ctx, const TuneChoice &tc, const Params &P) {
-    if (!tc.ana_seq || P.iter_cap > 0) return false;    // the iteration-cap test option uses k_analysis
-    return tc.ana_park >= 0 ? tc.ana_park != 0 : labels_fit_l2(ctx, P);
+// Setting long chains aside in steps (ii)/(iv) (contiguous order only): only
+// when asked for.
+bool resolve_park(const TuneChoice &tc, const Params &P) {
+    return tc.ana_seq && P.iter_cap == 0 && tc.ana_park > 0;    // (the iteration-cap test option takes the plain walk)
 }
 
 // Whether step (ii) runs as a pass of its own: as set, else not. Steps (i) and
@@ -426,7 +428,7 @@ void note_settings(ccl_context *ctx, const TuneChoice &tc, const Params &P) {
     ctx->last.analysis_order = tc.ana_seq;
     ctx->last.reduce_window = P.red_window;
     ctx->last.analysis_group = tc.ana_seq ? P.ana_group : 0;
-    ctx->last.analysis_park = resolve_park(ctx, tc, P) ? 1 : 0;
+    ctx->last.analysis_park = resolve_park(tc, P) ? 1 : 0;
 }
 
 // Dynamic shared memory of step (iii): its windows per band.
@@ -439,31 +441,19 @@ ccl_status enqueue_tail(ccl_context *ctx, const Params &P0, bool batched, const 
     resolve_tail(ctx, tc, P);
     note_settings(ctx, tc, P);
     const int T = tc.threads;
-    const int64_t warps_chunks = (P.n_chunks + kAnaChunks - 1) / kAnaChunks;
-    const int64_t warps_chunks_b = (P.n_chunks + kAnaChunksBatched - 1) / kAnaChunksBatched;
     const int64_t g_red = (int64_t)ctx->num_sms * blocks_per_sm(ctx, batched ? 5 : 4, 256);
     if (profile) CCL_CUDA(cudaEventRecord(ctx->ev[1], s));
-    const bool park = resolve_park(ctx, tc, P);
+    const bool park = resolve_park(tc, P);
     auto analysis = [&]() {
-        if (park) {
-            // a full SM of warps (the kernel's registers and shared memory allow
-            // it; the occupancy query can assume a smaller shared-memory carveout)
-            const int64_t per_sm = std::max<int64_t>(blocks_per_sm(ctx, batched ? 12 : 11, 32 * kParkWarps),
-                                                     2048 / (32 * kParkWarps));
-            const int64_t need = (warps_chunks + kParkWarps - 1) / kParkWarps;
-            const unsigned gp = (unsigned)std::max<int64_t>(1, std::min<int64_t>((int64_t)ctx->num_sms * per_sm, need));
-            if (batched) k_analysis_park<true><<<gp, 32 * kParkWarps, 0, s>>>(P);
-            else k_analysis_park<false><<<gp, 32 * kParkWarps, 0, s>>>(P);
-            return;
-        }
-        const unsigned g = (unsigned)grid_for(ctx, batched ? 3 : 2, tc, batched ? warps_chunks_b : warps_chunks);
-        if (batched) {
-            if (tc.ana_seq) k_analysis<true, true, kAnaChunksBatched><<<g, T, 0, s>>>(P);
-            else k_analysis<true, false, kAnaChunksBatched><<<g, T, 0, s>>>(P);
-        } else {
-            if (tc.ana_seq) k_analysis<false, true><<<g, T, 0, s>>>(P);
-            else k_analysis<false, false><<<g, T, 0, s>>>(P);
-        }
+        Params A = P;
+        if (!tc.ana_seq) A.ana_group = 1;       // groups interleaved over the warps
+        const int64_t groups = (P.n_chunks + kAnaChunks - 1) / kAnaChunks;
+        const unsigned g = (unsigned)grid_for(ctx, (park ? 11 : 2) + (batched ? 1 : 0), tc, groups);
+        const size_t smem = park ? park_smem(T) : 0;
+        if (batched && park) k_analysis<true, true><<<g, T, smem, s>>>(A);
+        else if (batched) k_analysis<true, false><<<g, T, smem, s>>>(A);
+        else if (park) k_analysis<false, true><<<g, T, smem, s>>>(A);
+        else k_analysis<false, false><<<g, T, smem, s>>>(A);
     };
     if (resolve_pre(tc)) {
         analysis();
@@ -591,7 +581,7 @@ ccl_status run(ccl_context *ctx, Params P, bool batched, const TuneChoice &tc, c
                const std::vector<Inst> *table, uint64_t shape_hash, bool allow_graph = true,
                const std::vector<int64_t> *offsets = nullptr) {
     for (int kid = 0; kid < 13; ++kid)
-        (void)blocks_per_sm(ctx, kid, kid >= 11 ? 32 * kParkWarps : kid >= 9 ? kInitThreads : kid >= 7 ? kDenseThreads
+        (void)blocks_per_sm(ctx, kid, kid >= 11 ? tc.threads : kid >= 9 ? kInitThreads : kid >= 7 ? kDenseThreads
                                                : (kid < 2 || kid == 6) ? kInitThreads : (kid >= 4 ? 256 : tc.threads));
     ctx->last.used_graph = 0;
     const bool capturing = stream_capturing(s);

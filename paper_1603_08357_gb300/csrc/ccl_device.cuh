@@ -16,9 +16,9 @@
 //  * Step (iii) runs Algorithm 1 over the queue: each warp drains a window of
 //    pairs with kRedSlots (six) pairs per lane in lockstep rounds (one load
 //    or atomicMin per live pair per round, next state from a small table).
-//  * Steps (ii)/(iv) chase every site's chain to its root, two chains per
-//    lane at once (four in a batch), each warp over a contiguous range of
-//    sites (or interleaved, for inputs without locality).
+//  * Steps (ii)/(iv) chase every site's chain to its root, three chains per
+//    lane at once, each warp over contiguous runs of sites (or interleaved,
+//    for inputs without locality).
 #pragma once
 #include <stdint.h>
 #include <cuda_runtime.h>
@@ -820,191 +820,155 @@ __global__ void __launch_bounds__(kInitThreads, kInitCtas) k_init(Params P) {
 // Steps (ii) and (iv): analysis. Every site follows its label chain to the
 // root and stores the root. No atomics run concurrently with this kernel and
 // every value written is an ancestor of the site, so plain stores are safe.
-// A warp walks kCh chunks at once (one chain per lane per chunk) so that
-// their dependent loads overlap: kAnaChunks for one instance, more for a
-// batch, whose labels do not fit L2 (longer latencies to cover).
-
-// kSeq = true: warp w walks contiguous runs of chunk groups in increasing
-// order, so the chains of its later sites run into roots it has already
-// stored (lattices numbered row by row) and, batched, the instance of a chunk
-// changes rarely. With P.ana_group = 0 each warp walks one range (the label
-// array fits in L2); with P.ana_group = G > 0 the groups are cut into
-// super-chunks of G groups per warp, all warps working inside one super-chunk
-// at a time, so the labels in use (and the roots their chains reach, in the
-// same instances) stay within L2 when the whole array does not fit.
-// kSeq = false: groups are interleaved over the warps (grid stride), which
-// balances inputs without locality (randomly numbered trees).
-template <bool kBatched, bool kSeq, int kCh = kAnaChunks>
-__global__ void __launch_bounds__(512) k_analysis(Params P) {
-    const int lane = threadIdx.x & 31;
-    const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    const int64_t ngroups = (P.n_chunks + kCh - 1) / kCh;
-    const int64_t wid = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int64_t per = (ngroups + nwarps - 1) / nwarps;
-    // run length G and super-chunk stride: one run of `per` groups per warp,
-    // or runs of ana_group groups every nwarps * ana_group groups
-    const int64_t G = !kSeq ? 1 : (P.ana_group > 0 && P.ana_group < per ? (int64_t)P.ana_group : per);
-    const int64_t sc_stride = kSeq ? nwarps * G : nwarps;
-    // the instance of the current chunks, its chunk range and the fields used,
-    // kept in registers until a chunk of another instance comes
-    int64_t kc_lo = 0, kc_hi = kBatched ? 0 : P.n_chunks;
-    int32_t *kc_lab = P.one.labels;
-    int32_t kc_n = P.one.n;
-    for (int64_t run = wid * G; run < ngroups; run += sc_stride)
-    for (int64_t gidx = run; gidx < min(run + G, ngroups); ++gidx) {
-        int32_t *L[kCh];
-        int32_t site[kCh], x[kCh], first[kCh];
-        int32_t cap = 0;
-        bool act[kCh];
-#pragma unroll
-        for (int u = 0; u < kCh; ++u) {
-            const int64_t c = gidx * kCh + u;
-            act[u] = false;
-            L[u] = nullptr;
-            site[u] = 0;
-            if (c < P.n_chunks) {
-                if (kBatched && (c < kc_lo || c >= kc_hi)) {
-                    const int kc = find_inst(P, c);
-                    kc_lo = P.insts[kc].chunk_begin;
-                    kc_hi = kc + 1 < P.K ? P.insts[kc + 1].chunk_begin : P.n_chunks;
-                    kc_lab = P.insts[kc].labels;
-                    kc_n = P.insts[kc].n;
-                }
-                site[u] = (int32_t)((c - (kBatched ? kc_lo : P.one.chunk_begin)) * kChunk) + lane;
-                L[u] = kc_lab;
-                cap = max(cap, kc_n);
-                act[u] = site[u] < kc_n;
-            }
-        }
-        // all loads of a round are issued before any result is used, so the
-        // kCh chains of a lane are in flight together
-#pragma unroll
-        for (int u = 0; u < kCh; ++u) x[u] = act[u] ? L[u][site[u]] : 0;
-#pragma unroll
-        for (int u = 0; u < kCh; ++u) {
-            first[u] = x[u];
-            act[u] = act[u] && x[u] != site[u];
-        }
-        for (int32_t it = 0;; ++it) {
-            int32_t y[kCh];
-#pragma unroll
-            for (int u = 0; u < kCh; ++u) y[u] = act[u] ? L[u][x[u]] : 0;
-            bool any = false;
-#pragma unroll
-            for (int u = 0; u < kCh; ++u) {
-                if (act[u]) {
-                    if (y[u] == x[u]) act[u] = false;
-                    else { x[u] = y[u]; any = true; }
-                }
-            }
-            if (!any) break;
-            if (it > cap || (P.iter_cap > 0 && it + 1 >= P.iter_cap)) { raise_err(P.err, kErrNonconv); break; }
-        }
-#pragma unroll
-        for (int u = 0; u < kCh; ++u)
-            if (L[u] && x[u] != first[u] && site[u] < cap) L[u][site[u]] = x[u];
-    }
-}
-
-// Steps (ii)/(iv) with parking, for inputs whose chains are mostly short but
-// have a long tail: every chain first gets kAnaRounds rounds in lockstep with
-// its warp (coalesced first loads, as k_analysis); the chains still
-// unfinished are appended to a per-warp list in shared memory and finished 32
-// at a time, one per lane, so a few long chains no longer hold up the lanes
-// of a whole group. Same visiting order (runs of P.ana_group groups, or one
-// range per warp) and the same results as k_analysis<kBatched, true>. (The
-// test option P.iter_cap is served by k_analysis alone.)
-constexpr int kAnaRounds = 4;
-constexpr int kParkWarps = 8;                        // warps per CTA (256 threads)
+//
+// A warp visits groups of kAnaChunks chunks, one chain per lane and chunk, all
+// chains of a round in flight together; a finished chain is predicated off (its
+// repeated loads would take the L1's gather bandwidth). Runs of P.ana_group = G
+// groups go to the warps in turn, so all warps work inside one super-chunk of
+// nwarps * G groups at a time and the labels in use (and the roots the chains
+// reach, in the same instances) stay in L2 when the whole array does not fit;
+// G = 0: one run per warp (everything fits). Sites come in increasing order
+// inside a run, so its later chains run into roots it has already stored.
+//
+// The gathers hit L1 and L2 for the most part; what bounds the kernel is their
+// latency and the instructions around them, so a run is cut into stretches of
+// one instance with 32-bit site numbers, and a round is a load, a compare and
+// a move per chain. Against the same walk with the instance, 64-bit chunk
+// numbers and caps looked at for every chunk (94 to 108 warp instructions per
+// chunk): 1024 mixed instances 2.54 -> 1.24 ms, triangle 16384^2 1.16 -> 0.67 ms,
+// triangle 4096^2 66 -> 47.5 us (2.8 TB/s of its 8 bytes per site), honeycomb
+// 2048^2 39 -> 28.5 us, 256 small instances 28.6 -> 16.5 us, Bethe lattice of
+// 24 shells 287 -> 282 us (random gathers over 201 MB). Three chunks a group
+// beat two (870 us on triangle 16384^2) and four (790), two rounds between
+// votes beat one (700) and equal three; 256 threads of 32 registers fill the SM.
+constexpr int kAnaRounds = 4;                        // rounds before a chain is set aside (kPark)
 constexpr int kParkCap = 32 * kAnaChunks + 32;       // < 32 left + one group's chains
-template <bool kBatched>
-__global__ void __launch_bounds__(256) k_analysis_park(Params P) {
-    __shared__ int s_site[8][kParkCap];
-    __shared__ int s_x[8][kParkCap];
-    __shared__ int s_k[kBatched ? 8 : 1][kBatched ? kParkCap : 1];
+
+// kPark = true (an option): a chain unfinished after kAnaRounds rounds goes to
+// a per-warp list in shared memory, finished 32 at a time, one per lane, so a
+// few long chains do not hold up the lanes of a whole group. (Slower than
+// waiting on every input measured: triangle 4096^2 55 us, 1024 mixed instances
+// 1.53 ms.)
+template <bool kBatched, bool kPark>
+__global__ void __launch_bounds__(512, 4) k_analysis(Params P) {
+    extern __shared__ int s_park[];                  // kPark: site and label of kParkCap chains per warp
     const int lane = threadIdx.x & 31;
-    const int wl = threadIdx.x >> 5;
-    const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    const int64_t ngroups = (P.n_chunks + kAnaChunks - 1) / kAnaChunks;
-    const int64_t wid = (int64_t)blockIdx.x * (blockDim.x >> 5) + wl;
-    const int64_t per = (ngroups + nwarps - 1) / nwarps;
-    const int64_t G = (P.ana_group > 0 && P.ana_group < per ? (int64_t)P.ana_group : per);
-    const int64_t sc_stride = nwarps * G;
-    int kc = 0;
-    int64_t kc_lo = 0, kc_hi = kBatched ? 0 : P.n_chunks;
-    int cnt = 0;
+    int *s_site = s_park + (threadIdx.x >> 5) * (2 * kParkCap), *s_x = s_site + kParkCap;
     const unsigned lt = (1u << lane) - 1u;
-    const int32_t capit = (int32_t)min(32 * P.n_chunks, (int64_t)INT32_MAX - 1);
-    auto drain = [&](int take) {
+    const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    const int64_t wid = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int64_t ngroups = (P.n_chunks + kAnaChunks - 1) / kAnaChunks;
+    const int64_t per = (ngroups + nwarps - 1) / nwarps;
+    const int64_t G = P.ana_group > 0 && P.ana_group < per ? (int64_t)P.ana_group : per;
+    // the instance of the current stretch: its chunks, labels and sites
+    int64_t kc_lo = 0, kc_hi = kBatched ? 0 : P.n_chunks;
+    int32_t *lab = P.one.labels;
+    int32_t n = P.one.n;
+    int cnt = 0;                                     // chains set aside
+    // no chain of valid labels is longer than n
+    const auto cap = [&]() { return P.iter_cap > 0 ? P.iter_cap : n; };
+    const auto drain = [&](int take) {
         const int base = cnt - take;
-        const bool act0 = lane < take;
+        const bool mine = lane < take;
         int site = 0, x = 0;
-        int32_t *Lp = P.one.labels;
-        if (act0) {
-            site = s_site[wl][base + lane];
-            x = s_x[wl][base + lane];
-            if (kBatched) Lp = P.insts[s_k[wl][base + lane]].labels;
+        if (mine) {
+            site = s_site[base + lane];
+            x = s_x[base + lane];
         }
-        bool act = act0;
+        bool act = mine;
         for (int32_t it = 0;; ++it) {
-            const int32_t y = act ? Lp[x] : 0;
-            if (act) { if (y == x) act = false; else x = y; }
+            int32_t y = x;
+            if (act) y = lab[x];
+            act = y != x;
+            x = y;
             if (!__any_sync(kFull, act)) break;
-            if (it > capit || (P.iter_cap > 0 && it + 1 + kAnaRounds >= P.iter_cap)) { raise_err(P.err, kErrNonconv); break; }
+            if (it >= cap()) { raise_err(P.err, kErrNonconv); break; }
         }
-        if (act0) Lp[site] = x;
+        if (mine) lab[site] = x;
         cnt = base;
         __syncwarp();
     };
-    for (int64_t run = wid * G; run < ngroups; run += sc_stride)
-    for (int64_t gidx = run; gidx < min(run + G, ngroups); ++gidx) {
-        int32_t *L[kAnaChunks];
-        int32_t site[kAnaChunks], x[kAnaChunks], first[kAnaChunks];
-        int kk[kAnaChunks];
-        bool act[kAnaChunks];
+    for (int64_t run = wid * G; run < ngroups; run += nwarps * G) {
+        int64_t c = run * kAnaChunks;
+        const int64_t c_end = min((run + G) * kAnaChunks, P.n_chunks);
+        while (c < c_end) {
+            if (kBatched && (c < kc_lo || c >= kc_hi)) {
+                const int kc = find_inst(P, c);
+                kc_lo = P.insts[kc].chunk_begin;
+                kc_hi = kc + 1 < P.K ? P.insts[kc + 1].chunk_begin : P.n_chunks;
+                lab = P.insts[kc].labels;
+                n = P.insts[kc].n;
+            }
+            // the stretch of this run inside the instance: the lane's sites s
+            // + 32 u below s_end
+            const int64_t ce = min(c_end, kc_hi);
+            int32_t s = (int32_t)((c - kc_lo) * kChunk) + lane;
+            const int32_t s_end = (int32_t)min((ce - kc_lo) * kChunk, (int64_t)n);
+            c = ce;
+            for (; s - lane < s_end; s += kChunk * kAnaChunks) {
+                int32_t x[kAnaChunks], first[kAnaChunks];
+                bool act[kAnaChunks];
+                int32_t *p = lab + s;
 #pragma unroll
-        for (int u = 0; u < kAnaChunks; ++u) {
-            const int64_t c = gidx * kAnaChunks + u;
-            act[u] = false; L[u] = nullptr; site[u] = 0; kk[u] = 0;
-            if (c < P.n_chunks) {
-                if (kBatched && (c < kc_lo || c >= kc_hi)) {
-                    kc = find_inst(P, c);
-                    kc_lo = P.insts[kc].chunk_begin;
-                    kc_hi = kc + 1 < P.K ? P.insts[kc + 1].chunk_begin : P.n_chunks;
+                for (int u = 0; u < kAnaChunks; ++u) {
+                    x[u] = s + kChunk * u;
+                    if (s + kChunk * u < s_end) x[u] = p[kChunk * u];
                 }
-                const Inst I = inst_of<kBatched>(P, kc);
-                site[u] = (int32_t)((c - I.chunk_begin) * kChunk) + lane;
-                L[u] = I.labels; kk[u] = kc;
-                act[u] = site[u] < I.n;
+#pragma unroll
+                for (int u = 0; u < kAnaChunks; ++u) {
+                    first[u] = x[u];
+                    act[u] = x[u] != s + kChunk * u;
+                }
+                const auto round = [&]() {
+                    int32_t y[kAnaChunks];
+#pragma unroll
+                    for (int u = 0; u < kAnaChunks; ++u) {
+                        y[u] = x[u];
+                        if (act[u]) y[u] = lab[x[u]];
+                    }
+#pragma unroll
+                    for (int u = 0; u < kAnaChunks; ++u) {
+                        act[u] = y[u] != x[u];
+                        x[u] = y[u];
+                    }
+                };
+                if (kPark) {
+#pragma unroll
+                    for (int r = 0; r < kAnaRounds; ++r) round();
+#pragma unroll
+                    for (int u = 0; u < kAnaChunks; ++u) {
+                        if (!act[u] && x[u] != first[u]) p[kChunk * u] = x[u];
+                        const unsigned pk = __ballot_sync(kFull, act[u]);
+                        if (pk) {
+                            const int pos = cnt + __popc(pk & lt);
+                            if (act[u]) {
+                                s_site[pos] = s + kChunk * u;
+                                s_x[pos] = x[u];
+                            }
+                            cnt += __popc(pk);
+                            __syncwarp();
+                            if (cnt >= 32) drain(32);
+                        }
+                    }
+                } else {
+                    for (int32_t it = 2;; it += 2) {
+                        round();
+                        round();
+                        bool any = false;
+#pragma unroll
+                        for (int u = 0; u < kAnaChunks; ++u) any |= act[u];
+                        if (!__any_sync(kFull, any)) break;
+                        if (it >= cap()) { raise_err(P.err, kErrNonconv); break; }
+                    }
+#pragma unroll
+                    for (int u = 0; u < kAnaChunks; ++u)
+                        if (x[u] != first[u]) p[kChunk * u] = x[u];
+                }
             }
-        }
-#pragma unroll
-        for (int u = 0; u < kAnaChunks; ++u) x[u] = act[u] ? L[u][site[u]] : 0;
-#pragma unroll
-        for (int u = 0; u < kAnaChunks; ++u) { first[u] = x[u]; act[u] = act[u] && x[u] != site[u]; }
-#pragma unroll
-        for (int r = 0; r < kAnaRounds; ++r) {
-            int32_t y[kAnaChunks];
-#pragma unroll
-            for (int u = 0; u < kAnaChunks; ++u) y[u] = act[u] ? L[u][x[u]] : 0;
-#pragma unroll
-            for (int u = 0; u < kAnaChunks; ++u)
-                if (act[u]) { if (y[u] == x[u]) act[u] = false; else x[u] = y[u]; }
-        }
-#pragma unroll
-        for (int u = 0; u < kAnaChunks; ++u) {
-            if (!act[u] && L[u] && x[u] != first[u]) L[u][site[u]] = x[u];
-            const unsigned pk = __ballot_sync(kFull, act[u]);
-            if (pk) {
-                const int pos = cnt + __popc(pk & lt);
-                if (act[u]) { s_site[wl][pos] = site[u]; s_x[wl][pos] = x[u]; if (kBatched) s_k[wl][pos] = kk[u]; }
-                cnt += __popc(pk);
-                __syncwarp();
-                if (cnt >= 32) drain(32);
-            }
+            if (kPark && kBatched) while (cnt > 0) drain(min(cnt, 32));     // (they belong to this instance)
         }
     }
-    while (cnt > 0) drain(min(cnt, 32));
+    if (kPark) while (cnt > 0) drain(min(cnt, 32));
 }
 
 // ---------------------------------------------------------------------------

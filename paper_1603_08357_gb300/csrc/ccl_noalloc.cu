@@ -70,7 +70,7 @@ ccl_status setup_device(int dev, DeviceSetup **out) {
         if (e == cudaSuccess)
             e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.init_per_sm, k_init<false>, kInitThreads, kInitSmem);
         if (e == cudaSuccess)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.ana_per_sm, k_analysis<false, true>, 256, 0);
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.ana_per_sm, k_analysis<false, false>, 256, 0);
         if (e == cudaSuccess)
             e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.red_per_sm, k_reduce<false, true>, 256, 0);
         if (e != cudaSuccess) {
@@ -150,7 +150,7 @@ extern "C" ccl_status ccl_label_noalloc(int32_t n, int64_t nnz, const int32_t *r
     if (e == cudaSuccess) {
         k_init<false><<<(unsigned)g_init, kInitThreads, kInitSmem, s>>>(P);
         k_reduce<false, true><<<(unsigned)g_red, kRedThreads, sizeof(uint32_t) * (size_t)(g_init + 1), s>>>(P);
-        k_analysis<false, true><<<(unsigned)g_ana, 256, 0, s>>>(P);
+        k_analysis<false, false><<<(unsigned)g_ana, 256, 0, s>>>(P);
         e = cudaGetLastError();
     }
     // the error word comes back on the call's own stream (no wait on other

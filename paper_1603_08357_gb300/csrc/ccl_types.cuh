@@ -25,15 +25,7 @@ constexpr int kColBuf = kColCap + 8;
 constexpr int kBitBuf = kColCap / 32 + 12;   // (a word past the last one copied may be read)
 constexpr int kRowRegs = 8;                // rows up to this degree are scanned in registers
 
-// steps (ii)/(iv): chunks a warp walks at once
-#ifndef CCL_ANA_CHUNKS
-#define CCL_ANA_CHUNKS 2
-#endif
-constexpr int kAnaChunks = CCL_ANA_CHUNKS;
-#ifndef CCL_ANA_CHUNKS_BATCHED
-#define CCL_ANA_CHUNKS_BATCHED 4
-#endif
-constexpr int kAnaChunksBatched = CCL_ANA_CHUNKS_BATCHED;
+constexpr int kAnaChunks = 3;              // steps (ii)/(iv): chunks a warp walks at once
 
 // step (iii): pairs a lane carries at once; pairs a warp drains per window;
 // most step-(i) CTAs (bands)
