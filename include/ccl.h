@@ -101,9 +101,10 @@ typedef enum {
                                   root, as in Algorithm 1; 1 under the node the other chain has
                                   reached (same atomicMin loop, shorter walks on trees) */
     CCL_OPT_REFILL = 6,        /* step (iii): 1 (default) each thread serves a fixed stride of the
-                                  residual pairs and loads its next one ahead; 0 a warp hands its
-                                  pairs out in order to whichever threads are free (balances
-                                  uneven chains) */
+                                  residual pairs (and, when the call's labels take at most three
+                                  eighths of L2, pairs with long chains are set aside and finished
+                                  together); 0 a warp hands its pairs out in order to whichever
+                                  threads are free (balances uneven chains) */
     CCL_OPT_ANALYSIS_ORDER = 7, /* steps (ii)/(iv): 1 (default) each warp walks a contiguous range of
                                   sites in increasing order (chains meet roots it already stored);
                                   0 the sites are interleaved over the warps (balances inputs

@@ -171,6 +171,8 @@ int blocks_per_sm(ccl_context *ctx, int kernel_id, int threads) {
         case 10: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_init_dense_tma<true>, kInitThreads, kDenseSmem); break;
         case 11: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_analysis<false, true>, threads, park_smem(threads)); break;
         case 12: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_analysis<true, true>, threads, park_smem(threads)); break;
+        case 13: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_reduce_park<false>, threads, 0); break;
+        case 14: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_reduce_park<true>, threads, 0); break;
         default: break;
     }
     if (e != cudaSuccess || nb < 1) { (void)cudaGetLastError(); nb = 1; }
@@ -441,7 +443,10 @@ ccl_status enqueue_tail(ccl_context *ctx, const Params &P0, bool batched, const 
     resolve_tail(ctx, tc, P);
     note_settings(ctx, tc, P);
     const int T = tc.threads;
-    const int64_t g_red = (int64_t)ctx->num_sms * blocks_per_sm(ctx, batched ? 5 : 4, 256);
+    // short walks for labels of at most three eighths of L2, else (and where
+    // the hand-out or the iteration cap is asked for) the slots
+    const bool short_walk = tc.refill && P.iter_cap == 0 && 4 * kChunk * P.n_chunks <= ctx->l2_bytes * 3 / 8;
+    const int64_t g_red = (int64_t)ctx->num_sms * blocks_per_sm(ctx, (short_walk ? 13 : 4) + (batched ? 1 : 0), kRedThreads);
     if (profile) CCL_CUDA(cudaEventRecord(ctx->ev[1], s));
     const bool park = resolve_park(tc, P);
     auto analysis = [&]() {
@@ -460,7 +465,10 @@ ccl_status enqueue_tail(ccl_context *ctx, const Params &P0, bool batched, const 
         CCL_CUDA(cudaGetLastError());
     }
     if (profile) CCL_CUDA(cudaEventRecord(ctx->ev[2], s));
-    if (batched) {
+    if (short_walk) {
+        if (batched) k_reduce_park<true><<<(unsigned)g_red, kRedThreads, red_smem(P), s>>>(P);
+        else k_reduce_park<false><<<(unsigned)g_red, kRedThreads, red_smem(P), s>>>(P);
+    } else if (batched) {
         if (tc.refill) k_reduce<true, true><<<(unsigned)g_red, kRedThreads, red_smem(P), s>>>(P);
         else k_reduce<true, false><<<(unsigned)g_red, kRedThreads, red_smem(P), s>>>(P);
     } else {
@@ -580,8 +588,8 @@ ccl_status upload_table(ccl_context *ctx, const std::vector<Inst> &table, cudaSt
 ccl_status run(ccl_context *ctx, Params P, bool batched, const TuneChoice &tc, cudaStream_t s,
                const std::vector<Inst> *table, uint64_t shape_hash, bool allow_graph = true,
                const std::vector<int64_t> *offsets = nullptr) {
-    for (int kid = 0; kid < 13; ++kid)
-        (void)blocks_per_sm(ctx, kid, kid >= 11 ? tc.threads : kid >= 9 ? kInitThreads : kid >= 7 ? kDenseThreads
+    for (int kid = 0; kid < 15; ++kid)
+        (void)blocks_per_sm(ctx, kid, kid >= 13 ? kRedThreads : kid >= 11 ? tc.threads : kid >= 9 ? kInitThreads : kid >= 7 ? kDenseThreads
                                                : (kid < 2 || kid == 6) ? kInitThreads : (kid >= 4 ? 256 : tc.threads));
     ctx->last.used_graph = 0;
     const bool capturing = stream_capturing(s);

@@ -1055,13 +1055,10 @@ __device__ __forceinline__ long long block_excl_scan(long long v, long long *s_w
     return before + incl - v;
 }
 
-template <bool kBatched, bool kStatic>
-__global__ void __launch_bounds__(kRedThreads, kBatched ? 4 : 5) k_reduce(Params P) {
-    extern __shared__ uint32_t s_win[];             // [n_bands + 1]
-    __shared__ long long s_warp[kRedThreads / 32];
-    const int lane = threadIdx.x & 31;
-    const unsigned lt = (1u << lane) - 1u;
-    const long long nwarps = (long long)gridDim.x * (kRedThreads / 32);
+// Cuts the call's pairs into windows: fills s_win[0 .. n_bands], stores the
+// statistics and returns the number of windows. The whole CTA calls.
+__device__ __forceinline__ uint32_t red_windows(const Params &P, uint32_t *s_win, long long *s_warp, int lane,
+                                                long long nwarps) {
     // one window per warp when the queue is short (bands round their window
     // counts up: at most one more each), at least 64 pairs
     const auto window = [&](long long total) {
@@ -1104,31 +1101,61 @@ __global__ void __launch_bounds__(kRedThreads, kBatched ? 4 : 5) k_reduce(Params
         if (P.more_pairs) P.counters[0] += (unsigned long long)total;
         else P.counters[0] = (unsigned long long)total;
     }
-    const long long nwin = s_win[P.n_bands];
+    return s_win[P.n_bands];
+}
+
+// Window w: its pairs and, batched, their instances.
+struct RedWindow {
+    const int2 *q;
+    const int32_t *qk;
+    int len;
+};
+template <bool kBatched>
+__device__ __forceinline__ RedWindow red_window(const Params &P, const uint32_t *s_win, uint32_t w) {
+    // its band: the last one with at most w windows before it (all lanes
+    // search; smem broadcast)
+    int band = 0;
+    for (int hi = P.n_bands - 1; band < hi;) {
+        const int mid = (band + hi + 1) >> 1;
+        if (s_win[mid] <= w) band = mid; else hi = mid - 1;
+    }
+    // the band's pairs are spread evenly over its windows
+    const long long cnt = (long long)P.band[band].cnt;
+    const uint32_t before = s_win[band];
+    const int wins = (int)(s_win[band + 1] - before);
+    const long long most = (cnt + wins - 1) / wins;
+    const long long beg = (long long)(w - before) * most;
+    RedWindow r;
+    r.len = (int)max(min(beg + most, cnt) - beg, 0ll);
+    r.q = P.q + P.band[band].qbase + beg;
+    r.qk = kBatched ? P.qk + P.band[band].qbase + beg : nullptr;
+    return r;
+}
+
+// A pair needs at most 4n + 8 rounds (its chains and Algorithm 1's loop are
+// bounded by the instance's n <= 32 n_chunks); a lane serves at most len pairs.
+// Past this many rounds a window is abandoned with an error.
+__device__ __forceinline__ long long red_round_cap(const Params &P, int len) {
+    return P.iter_cap > 0 ? (long long)P.iter_cap : (128ll * P.n_chunks + 8) * (long long)len;
+}
+
+template <bool kBatched, bool kStatic>
+__global__ void __launch_bounds__(kRedThreads, kBatched ? 4 : 5) k_reduce(Params P) {
+    extern __shared__ uint32_t s_win[];             // [n_bands + 1]
+    __shared__ long long s_warp[kRedThreads / 32];
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    const long long nwarps = (long long)gridDim.x * (kRedThreads / 32);
+    const long long nwin = red_windows(P, s_win, s_warp, lane, nwarps);
 #ifdef CCL_DEVICE_STATS
     unsigned long long st_hops = 0, st_atom = 0, st_iter = 0;
 #endif
     for (long long w = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w < nwin; w += nwarps) {
-        // band of the window: the last one with at most w windows before it
-        // (all lanes search; smem broadcast)
-        int band = 0;
-        for (int hi = P.n_bands - 1; band < hi;) {
-            const int mid = (band + hi + 1) >> 1;
-            if (s_win[mid] <= (uint32_t)w) band = mid; else hi = mid - 1;
-        }
-        // the band's pairs are spread evenly over its windows
-        const long long bcnt = (long long)P.band[band].cnt;
-        const int bwin = (int)(s_win[band + 1] - s_win[band]);
-        const long long wmost = (bcnt + bwin - 1) / bwin;
-        const long long wbeg = (long long)((uint32_t)w - s_win[band]) * wmost;
-        const int wlen = (int)max(min(wbeg + wmost, bcnt) - wbeg, 0ll);
-        const int2 *wq = P.q + P.band[band].qbase + wbeg;
-        const int32_t *wqk = kBatched ? P.qk + P.band[band].qbase + wbeg : nullptr;
-        // A pair needs at most 4n + 8 rounds (its chains and Algorithm 1's loop
-        // are bounded by the instance's n <= 32 n_chunks); a lane serves at most
-        // wlen pairs. Past this many rounds the window is abandoned with an error.
-        const long long round_cap = P.iter_cap > 0 ? (long long)P.iter_cap
-                                                    : (128ll * P.n_chunks + 8) * (long long)wlen;
+        const RedWindow win = red_window<kBatched>(P, s_win, (uint32_t)w);
+        const int wlen = win.len;
+        const int2 *wq = win.q;
+        const int32_t *wqk = win.qk;
+        const long long round_cap = red_round_cap(P, wlen);
         long long rounds = 0;
         int nxt = 0;        // pairs of the window handed to slots so far
         // kStatic: the lane's next pair, loaded ahead
@@ -1240,6 +1267,161 @@ __global__ void __launch_bounds__(kRedThreads, kBatched ? 4 : 5) k_reduce(Params
                 break;
             }
         }
+    }
+#ifdef CCL_DEVICE_STATS
+    if (st_hops) atomicAdd(P.counters + 1, st_hops);
+    if (st_atom) atomicAdd(P.counters + 2, st_atom);
+    if (lane == 0 && st_iter) atomicAdd(P.counters + 3, st_iter);
+#endif
+}
+
+// Step (iii) for calls whose labels take at most three eighths of L2: two pairs
+// a lane start together
+// with their warp and run a fixed number of steps, both ends of a pair walking
+// at once; the pairs whose ends are roots by then are linked by Algorithm 1's
+// atomicMin, and what is not finished goes to a per-warp list in shared memory,
+// 32 of which at a time, one per lane, run on. The code of a step is a fraction
+// of k_reduce's (no slot to choose, no state table), the first steps of
+// consecutive pairs stay coalesced, and few pairs need more: honeycomb 256^2
+// 28 -> 21 us, 256 small instances 39 -> 24, honeycomb 2048^2 66 -> 43, cubic
+// 200^3 33 -> 30. It loads more labels than k_reduce (which walks only the
+// larger node). At half of L2 the two are even (triangle 4096^2 94 -> 85,
+// honeycomb 2896^2 at 1.25 p_c 131 -> 147), beyond L2 the loads cost more than
+// the code saves (triangle 16384^2 1.37 -> 1.91 ms, 1024 mixed instances
+// 2.53 -> 3.07).
+constexpr int kParkSteps = 4;                   // steps before a pair is set aside
+constexpr int kParkPairs = 2;                   // pairs a lane starts together
+constexpr int kParkList = 64;                   // < 32 left + one pair per lane
+template <bool kBatched>
+__global__ void __launch_bounds__(kRedThreads, kBatched ? 6 : 8) k_reduce_park(Params P) {
+    extern __shared__ uint32_t s_win[];             // [n_bands + 1]
+    __shared__ long long s_warp[kRedThreads / 32];
+    __shared__ int2 s_pair[kRedThreads / 32][kParkList];
+    __shared__ int s_k[kBatched ? kRedThreads / 32 : 1][kBatched ? kParkList : 1];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    const long long nwarps = (long long)gridDim.x * (kRedThreads / 32);
+    const long long nwin = red_windows(P, s_win, s_warp, lane, nwarps);
+    const bool eager = P.link_mode != 0;            // link a root to the other end's node, not its root
+    // the labels of the lane's last instance
+    int lk = -1;
+    int32_t *llab = P.one.labels;
+#ifdef CCL_DEVICE_STATS
+    unsigned long long st_hops = 0, st_atom = 0, st_iter = 0;
+#endif
+    struct Pair {
+        int32_t a, b;
+        bool ra, rb, act;           // a, b are roots; the pair is not done
+    };
+    const auto step = [&](Pair &p, const int32_t *L) {
+        int32_t ya = p.a, yb = p.b;
+        if (p.act && !p.ra) ya = red_load(L + p.a);
+        if (p.act && !p.rb) yb = red_load(L + p.b);
+#ifdef CCL_DEVICE_STATS
+        st_hops += (p.act && !p.ra) + (p.act && !p.rb);
+#endif
+        p.ra = ya == p.a;
+        p.rb = yb == p.b;
+        p.a = ya;
+        p.b = yb;
+        p.act = p.act && ya != yb;
+    };
+    const auto link = [&](Pair &p, int32_t *L) {
+        const int32_t hi = max(p.a, p.b), lo = min(p.a, p.b);
+        if (p.act && (eager ? (p.a > p.b ? p.ra : p.rb) : (p.ra && p.rb))) {
+            // old == hi: linked; old == lo: linked already; else Algorithm 1
+            // goes on with the displaced label
+            const int32_t old = atomicMin(L + hi, lo);
+#ifdef CCL_DEVICE_STATS
+            ++st_atom;
+#endif
+            p.act = old != hi && old != lo;
+            p.a = old;
+            p.b = lo;
+            p.ra = p.rb = false;
+        }
+    };
+    for (long long w = (long long)blockIdx.x * (kRedThreads / 32) + warp; w < nwin; w += nwarps) {
+        const RedWindow win = red_window<kBatched>(P, s_win, (uint32_t)w);
+        const int round_cap = (int)min(red_round_cap(P, win.len), (long long)INT32_MAX - 3);
+        int rounds = 0;
+        int cnt = 0;                // pairs set aside; below 32 whenever pairs are added
+        const auto set_aside = [&](const Pair &p, int k) {
+            const unsigned m = __ballot_sync(kFull, p.act);
+            if (m == 0) return;
+            if (p.act) {
+                const int pos = cnt + __popc(m & lt);
+                s_pair[warp][pos] = make_int2(p.a, p.b);
+                if (kBatched) s_k[warp][pos] = k;
+            }
+            cnt += __popc(m);
+            __syncwarp();
+        };
+        // runs up to 32 of the set-aside pairs on: a few steps, or to the end
+        const auto resume = [&](bool to_end) {
+            const int take = min(cnt, 32);
+            cnt -= take;
+            Pair p{0, 0, false, false, lane < take};
+            int k = 0;
+            if (p.act) {
+                const int2 q = s_pair[warp][cnt + lane];
+                if (kBatched) k = s_k[warp][cnt + lane];
+                p.a = q.x;
+                p.b = q.y;
+            }
+            int32_t *L = kBatched ? P.insts[k].labels : P.one.labels;
+            __syncwarp();
+            for (int it = 0; to_end || it < 2; ++it) {
+#ifdef CCL_DEVICE_STATS
+                st_iter += 2;
+#endif
+                step(p, L);
+                step(p, L);
+                link(p, L);
+                if (!__any_sync(kFull, p.act)) return;
+                if ((rounds += 3) > round_cap) {        // the pairs are dropped
+                    raise_err(P.err, kErrNonconv);
+                    return;
+                }
+            }
+            set_aside(p, k);
+        };
+        for (int p0 = lane; p0 - lane < win.len; p0 += 32 * kParkPairs) {
+            Pair pr[kParkPairs];
+            int k[kParkPairs];
+            int32_t *L[kParkPairs];
+#pragma unroll
+            for (int u = 0; u < kParkPairs; ++u) {
+                pr[u] = Pair{0, 0, false, false, p0 + 32 * u < win.len};
+                k[u] = 0;
+                if (pr[u].act) {
+                    const int2 q = win.q[p0 + 32 * u];
+                    if (kBatched) k[u] = win.qk[p0 + 32 * u];
+                    pr[u].a = q.x;
+                    pr[u].b = q.y;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < kParkPairs; ++u) {
+                if (kBatched && k[u] != lk) { lk = k[u]; llab = P.insts[lk].labels; }
+                L[u] = kBatched ? llab : P.one.labels;
+            }
+#ifdef CCL_DEVICE_STATS
+            st_iter += kParkSteps;
+#endif
+#pragma unroll
+            for (int r = 0; r < kParkSteps; ++r)
+#pragma unroll
+                for (int u = 0; u < kParkPairs; ++u) step(pr[u], L[u]);
+#pragma unroll
+            for (int u = 0; u < kParkPairs; ++u) link(pr[u], L[u]);
+#pragma unroll
+            for (int u = 0; u < kParkPairs; ++u) {
+                set_aside(pr[u], k[u]);
+                while (cnt >= 32) resume(false);        // (every step shortens a walk: this ends)
+            }
+        }
+        while (cnt > 0) resume(true);
     }
 #ifdef CCL_DEVICE_STATS
     if (st_hops) atomicAdd(P.counters + 1, st_hops);

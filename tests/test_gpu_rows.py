@@ -83,3 +83,32 @@ def test_bands_in_rounds(ctx):
     st = ccl.ccl_get_stats(ctx)
     assert np.array_equal(gpu_label_batched(ctx, b), got)          # again: the ticket starts over
     assert ccl.ccl_get_stats(ctx).residual_pairs == st.residual_pairs > 0
+
+
+def _ladder(rungs, seed):
+    """Two paths joined by rungs, numbered at random along the paths: every
+    label chain is long, and every rung but the first closes a cycle."""
+    rng = np.random.default_rng(seed)
+    num = rng.permutation(2 * rungs) if seed else np.arange(2 * rungs)
+    a, b = num[:rungs], num[rungs:]
+    u = np.concatenate([a[:-1], b[:-1], a])
+    v = np.concatenate([a[1:], b[1:], b])
+    rows, cols = np.concatenate([u, v]), np.concatenate([v, u])
+    order = np.argsort(rows, kind="stable")
+    rp = np.concatenate([[0], np.cumsum(np.bincount(rows, minlength=2 * rungs))]).astype(np.int32)
+    nnz = rows.size
+    return L.Lattice("random", 2 * rungs, nnz, rp, cols[order].astype(np.int32), L.pack_bits(np.ones(nnz, bool)), 1.0, seed)
+
+
+@pytest.mark.parametrize("rungs", [1, 2, 31, 33, 64, 65, 1000, 20_000])
+@pytest.mark.parametrize("link", [0, 1])
+def test_long_chains(rungs, link):
+    """Pairs that are set aside again and again, at the edges of the list."""
+    c = ccl.ccl_context_create(0)
+    try:
+        assert ccl.ccl_set_option(c, ccl.CCL_OPT_LINK_MODE, link) == ccl.CCL_OK
+        for seed in (0, 1, 2):
+            lat = _ladder(rungs, seed)
+            assert np.array_equal(gpu_label(c, lat), oracle.uf_label(lat))
+    finally:
+        ccl.ccl_context_destroy(c)
