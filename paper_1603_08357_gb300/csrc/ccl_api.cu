@@ -162,8 +162,8 @@ int blocks_per_sm(ccl_context *ctx, int kernel_id, int threads) {
         case 1: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_init<true>, kInitThreads, kInitSmem); break;
         case 2: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_analysis<false, false>, threads, 0); break;
         case 3: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_analysis<true, false>, threads, 0); break;
-        case 4: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_reduce<false, true>, threads, 0); break;
-        case 5: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_reduce<true, true>, threads, 0); break;
+        case 4: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_reduce<false, true, false>, threads, 0); break;
+        case 5: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_reduce<true, true, true>, threads, 0); break;
         case 6: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_init<false, true>, kInitThreads, kInitSmem); break;
         case 7: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_init_dense<false>, kDenseThreads, 0); break;
         case 8: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_init_dense<true>, kDenseThreads, 0); break;
@@ -173,6 +173,7 @@ int blocks_per_sm(ccl_context *ctx, int kernel_id, int threads) {
         case 12: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_analysis<true, true>, threads, park_smem(threads)); break;
         case 13: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_reduce_park<false>, threads, 0); break;
         case 14: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_reduce_park<true>, threads, 0); break;
+        case 15: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_reduce<true, true, false>, threads, 0); break;
         default: break;
     }
     if (e != cudaSuccess || nb < 1) { (void)cudaGetLastError(); nb = 1; }
@@ -394,15 +395,20 @@ ccl_status launch_init(const Params &P, bool batched, int64_t g, cudaStream_t s)
 // The step (iii) window and the step (ii)/(iv) visiting order of a call:
 // explicit settings win; otherwise, when the call's labels fit in three
 // quarters of L2, long windows and one contiguous range per warp (every
-// gather hits L2 anyway), else windows of 512 pairs and super-chunks of 16
-// chunk groups per warp, so the labels the warps touch at once stay in L2.
+// gather hits L2 anyway), else windows of at most 1024 pairs and super-chunks of
+// 16 chunk groups per warp, so the labels the warps touch at once stay in L2.
+// (Windows of 512 / 1024 / 2048 pairs: triangle 16384^2 1.41 / 1.17 / 1.59 ms,
+// 1024 mixed instances 2.76 / 2.24 / 3.0; with instances far apart, six slots,
+// 2.53 / 2.73 / 3.76.)
+bool batched_far(const Params &P) { return P.K > 1 && !P.lab_base; }
+
 bool labels_fit_l2(const ccl_context *ctx, const Params &P) {
     return 4 * kChunk * P.n_chunks <= ctx->l2_bytes * 3 / 4;
 }
 
 void resolve_tail(const ccl_context *ctx, const TuneChoice &tc, Params &P) {
     const bool fits = labels_fit_l2(ctx, P);
-    P.red_window = tc.red_window > 0 ? tc.red_window : (fits ? kRedWindowMax : 512);
+    P.red_window = tc.red_window > 0 ? tc.red_window : (fits ? kRedWindowMax : batched_far(P) ? 512 : 1024);
     P.ana_group = tc.ana_group >= 0 ? tc.ana_group : (fits ? 0 : 16);
 }
 
@@ -446,7 +452,13 @@ ccl_status enqueue_tail(ccl_context *ctx, const Params &P0, bool batched, const 
     // short walks for labels of at most three eighths of L2, else (and where
     // the hand-out or the iteration cap is asked for) the slots
     const bool short_walk = tc.refill && P.iter_cap == 0 && 4 * kChunk * P.n_chunks <= ctx->l2_bytes * 3 / 8;
-    const int64_t g_red = (int64_t)ctx->num_sms * blocks_per_sm(ctx, (short_walk ? 13 : 4) + (batched ? 1 : 0), kRedThreads);
+    const bool near = batched && tc.refill && P.lab_base != nullptr;
+    int red_per_sm = blocks_per_sm(ctx, short_walk ? (batched ? 14 : 13) : near ? 15 : batched ? 5 : 4, kRedThreads);
+    // beyond L2 fewer warps at once keep more of the labels in use in it:
+    // triangle 16384^2 1.27 ms with five CTAs per SM, 1.17 with four (1.32 with
+    // three), all with windows of 1024 pairs
+    if (!batched && !short_walk && !labels_fit_l2(ctx, P)) red_per_sm = std::min(red_per_sm, 4);
+    const int64_t g_red = (int64_t)ctx->num_sms * red_per_sm;
     if (profile) CCL_CUDA(cudaEventRecord(ctx->ev[1], s));
     const bool park = resolve_park(tc, P);
     auto analysis = [&]() {
@@ -469,11 +481,12 @@ ccl_status enqueue_tail(ccl_context *ctx, const Params &P0, bool batched, const 
         if (batched) k_reduce_park<true><<<(unsigned)g_red, kRedThreads, red_smem(P), s>>>(P);
         else k_reduce_park<false><<<(unsigned)g_red, kRedThreads, red_smem(P), s>>>(P);
     } else if (batched) {
-        if (tc.refill) k_reduce<true, true><<<(unsigned)g_red, kRedThreads, red_smem(P), s>>>(P);
-        else k_reduce<true, false><<<(unsigned)g_red, kRedThreads, red_smem(P), s>>>(P);
+        if (near) k_reduce<true, true, false><<<(unsigned)g_red, kRedThreads, red_smem(P), s>>>(P);
+        else if (tc.refill) k_reduce<true, true, true><<<(unsigned)g_red, kRedThreads, red_smem(P), s>>>(P);
+        else k_reduce<true, false, true><<<(unsigned)g_red, kRedThreads, red_smem(P), s>>>(P);
     } else {
-        if (tc.refill) k_reduce<false, true><<<(unsigned)g_red, kRedThreads, red_smem(P), s>>>(P);
-        else k_reduce<false, false><<<(unsigned)g_red, kRedThreads, red_smem(P), s>>>(P);
+        if (tc.refill) k_reduce<false, true, false><<<(unsigned)g_red, kRedThreads, red_smem(P), s>>>(P);
+        else k_reduce<false, false, false><<<(unsigned)g_red, kRedThreads, red_smem(P), s>>>(P);
     }
     CCL_CUDA(cudaGetLastError());
     if (profile) CCL_CUDA(cudaEventRecord(ctx->ev[3], s));
@@ -584,14 +597,27 @@ ccl_status upload_table(ccl_context *ctx, const std::vector<Inst> &table, cudaSt
     return CCL_OK;
 }
 
+// The lowest labels of the instances if every instance's lie within 2^32 labels
+// of them (whole batches do: their labels are one array), else null.
+int32_t *label_base(const std::vector<Inst> &table) {
+    uintptr_t lo = UINTPTR_MAX, hi = 0;
+    for (const Inst &I : table) {
+        if (I.n == 0) continue;
+        lo = std::min(lo, (uintptr_t)I.labels);
+        hi = std::max(hi, (uintptr_t)(I.labels + I.n));
+    }
+    return lo < hi && (hi - lo) / sizeof(int32_t) <= ((uint64_t)1 << 32) ? (int32_t *)lo : nullptr;
+}
+
 // Runs P on stream s: through a cached graph when allowed, else directly.
 ccl_status run(ccl_context *ctx, Params P, bool batched, const TuneChoice &tc, cudaStream_t s,
                const std::vector<Inst> *table, uint64_t shape_hash, bool allow_graph = true,
                const std::vector<int64_t> *offsets = nullptr) {
-    for (int kid = 0; kid < 15; ++kid)
+    for (int kid = 0; kid < 16; ++kid)
         (void)blocks_per_sm(ctx, kid, kid >= 13 ? kRedThreads : kid >= 11 ? tc.threads : kid >= 9 ? kInitThreads : kid >= 7 ? kDenseThreads
                                                : (kid < 2 || kid == 6) ? kInitThreads : (kid >= 4 ? 256 : tc.threads));
     ctx->last.used_graph = 0;
+    if (batched) P.lab_base = label_base(*table);
     const bool capturing = stream_capturing(s);
     if (ctx->profile || !ctx->use_graphs || capturing || !allow_graph) {
         if (batched) {
@@ -1556,6 +1582,7 @@ ccl_status ccl_label_batched_host(ccl_context *ctx, int32_t K, const int64_t *si
             st = upload_table(ctx, tg, s);
             if (st != CCL_OK) return fail(st);
             P.insts = ctx->d_insts;
+            P.lab_base = label_base(tg);
         } else {
             P.one = tg[0];
         }

@@ -14,7 +14,7 @@
 //    smallest lower neighbour lies in a band tile finished kStages tiles
 //    earlier takes that neighbour's label (most of step (ii) on lattices).
 //  * Step (iii) runs Algorithm 1 over the queue: each warp drains a window of
-//    pairs with kRedSlots (six) pairs per lane in lockstep rounds (one load
+//    pairs with six or eight pairs per lane in lockstep rounds (one load
 //    or atomicMin per live pair per round, next state from a small table).
 //  * Steps (ii)/(iv) chase every site's chain to its root, three chains per
 //    lane at once, each warp over contiguous runs of sites (or interleaved,
@@ -976,7 +976,7 @@ __global__ void __launch_bounds__(512, 4) k_analysis(Params P) {
 // The pairs of all bands form one flat index space (prefix sums of the band
 // counts, in shared memory). A warp drains a window of pairs (at most
 // kRedWindowMax, fewer when the queue is short so every warp has one); each
-// lane carries kRedSlots pairs and takes the next pair of the window as soon
+// lane carries six or eight pairs and takes the next pair of the window as soon
 // as one finishes, so a long walk holds up one slot, not the warp. Every
 // round issues one load or one atomicMin per live slot before any result is
 // used, so a lane's slots are in flight together.
@@ -1059,12 +1059,16 @@ __device__ __forceinline__ long long block_excl_scan(long long v, long long *s_w
 // statistics and returns the number of windows. The whole CTA calls.
 __device__ __forceinline__ uint32_t red_windows(const Params &P, uint32_t *s_win, long long *s_warp, int lane,
                                                 long long nwarps) {
-    // one window per warp when the queue is short (bands round their window
-    // counts up: at most one more each), at least 64 pairs
+    // Every warp takes as many windows as every other, the fewest that keeps
+    // them below the limit: a last round of a few windows leaves the chip idle
+    // (Bethe lattice of 24 shells, 5.5M pairs: 254 us with windows of 1024 pairs,
+    // 1.1 rounds; 233 with two rounds). Bands round their window counts up, at
+    // most one more each. At least 64 pairs.
     const auto window = [&](long long total) {
         const long long wmax = P.red_window > 0 ? P.red_window : kRedWindowMax;
         const long long room = max(nwarps - P.n_bands, nwarps / 2);
-        return min(max((total + room - 1) / room, 64ll), wmax);
+        const long long waves = max((total + room * wmax - 1) / (room * wmax), 1ll);
+        return min(max((total + room * waves - 1) / (room * waves), 64ll), wmax);
     };
     long long total;
     if (P.n_bands <= 32) {
@@ -1139,8 +1143,18 @@ __device__ __forceinline__ long long red_round_cap(const Params &P, int len) {
     return P.iter_cap > 0 ? (long long)P.iter_cap : (128ll * P.n_chunks + 8) * (long long)len;
 }
 
-template <bool kBatched, bool kStatic>
-__global__ void __launch_bounds__(kRedThreads, kBatched ? 4 : 5) k_reduce(Params P) {
+//
+// kFar: the labels of a batch's instances lie anywhere, and a slot carries
+// their address; else they lie within 2^32 labels from P.lab_base on, and a slot
+// carries a 32-bit offset. That leaves registers for eight slots instead of
+// six, and fewer warps with more slots keep the labels in use in the caches:
+// 1024 mixed instances 2.53 ms (six slots with addresses, four CTAs per SM,
+// windows of 512 pairs) -> 2.24 (eight with offsets, three CTAs, 1024; six with
+// offsets: 2.37).
+template <bool kBatched, bool kStatic, bool kFar>
+__global__ void __launch_bounds__(kRedThreads, !kBatched ? 5 : kFar ? 4 : 3) k_reduce(Params P) {
+    constexpr bool kOff = kBatched && !kFar;
+    constexpr int kRedSlots = kOff ? 8 : 6;
     extern __shared__ uint32_t s_win[];             // [n_bands + 1]
     __shared__ long long s_warp[kRedThreads / 32];
     const int lane = threadIdx.x & 31;
@@ -1166,7 +1180,10 @@ __global__ void __launch_bounds__(kRedThreads, kBatched ? 4 : 5) k_reduce(Params
         // batched: the labels of the lane's last instance (consecutive pairs
         // of a lane mostly come from one instance)
         int lk = 0;
-        int32_t *llab = kBatched ? P.insts[0].labels : P.one.labels;
+        int32_t *llab = kFar ? P.insts[0].labels : nullptr;
+        uint32_t loff = kOff ? (uint32_t)(P.insts[0].labels - P.lab_base) : 0u;
+        // node x of slot u: its own address, or an offset from one base
+        int32_t *const base = kBatched ? P.lab_base : P.one.labels;
         auto fetch = [&]() {
             pf = wq[pnext];
             if (kBatched) pfk = wqk[pnext];
@@ -1175,11 +1192,13 @@ __global__ void __launch_bounds__(kRedThreads, kBatched ? 4 : 5) k_reduce(Params
         };
         if (kStatic && pnext < wlen) fetch();
         int32_t *L[kRedSlots];
+        uint32_t off[kRedSlots];
         int32_t a[kRedSlots], b[kRedSlots], st[kRedSlots];
 #pragma unroll
         for (int u = 0; u < kRedSlots; ++u) {
             st[u] = kTaskDone;
-            L[u] = P.one.labels;
+            L[u] = nullptr;
+            off[u] = 0;
             a[u] = b[u] = 0;
         }
         for (;;) {
@@ -1191,11 +1210,20 @@ __global__ void __launch_bounds__(kRedThreads, kBatched ? 4 : 5) k_reduce(Params
                     if (st[u] == kTaskDone) take = u;
                 if (take >= 0 && pf_ok) {
                     const int32_t na = max(pf.x, pf.y), nb = min(pf.x, pf.y);
-                    if (kBatched && pfk != lk) { lk = pfk; llab = P.insts[pfk].labels; }
-                    int32_t *nl = llab;
+                    if (kBatched && pfk != lk) {
+                        lk = pfk;
+                        int32_t *l = P.insts[pfk].labels;
+                        if (kFar) llab = l; else loff = (uint32_t)(l - base);
+                    }
 #pragma unroll
                     for (int u = 0; u < kRedSlots; ++u)
-                        if (u == take) { a[u] = na; b[u] = nb; st[u] = kTaskChase; L[u] = nl; }
+                        if (u == take) {
+                            a[u] = na;
+                            b[u] = nb;
+                            st[u] = kTaskChase;
+                            if (kFar) L[u] = llab;
+                            if (kOff) off[u] = loff;
+                        }
                     pf_ok = false;
                     if (pnext < wlen) fetch();
                 }
@@ -1212,8 +1240,13 @@ __global__ void __launch_bounds__(kRedThreads, kBatched ? 4 : 5) k_reduce(Params
                             const int2 pr = wq[pos];
                             if (kBatched) {
                                 const int k = wqk[pos];
-                                if (k != lk) { lk = k; llab = P.insts[k].labels; }
-                                L[u] = llab;
+                                if (k != lk) {
+                                    lk = k;
+                                    int32_t *l = P.insts[k].labels;
+                                    if (kFar) llab = l; else loff = (uint32_t)(l - base);
+                                }
+                                if (kFar) L[u] = llab;
+                                if (kOff) off[u] = loff;
                             }
                             a[u] = max(pr.x, pr.y);
                             b[u] = min(pr.x, pr.y);
@@ -1231,7 +1264,8 @@ __global__ void __launch_bounds__(kRedThreads, kBatched ? 4 : 5) k_reduce(Params
             int32_t v[kRedSlots];
 #pragma unroll
             for (int u = 0; u < kRedSlots; ++u) {
-                int32_t *ptr = L[u] + (st[u] == kTaskRoot ? b[u] : a[u]);
+                const int32_t x = st[u] == kTaskRoot ? b[u] : a[u];
+                int32_t *ptr = kFar ? L[u] + x : base + (uint32_t)((kOff ? off[u] : 0u) + (uint32_t)x);
                 v[u] = 0;
                 if (st[u] == kTaskMerge) v[u] = atomicMin(ptr, b[u]);
                 else if (st[u] != kTaskDone) v[u] = red_load(ptr);

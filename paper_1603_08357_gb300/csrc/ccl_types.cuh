@@ -27,12 +27,7 @@ constexpr int kRowRegs = 8;                // rows up to this degree are scanned
 
 constexpr int kAnaChunks = 3;              // steps (ii)/(iv): chunks a warp walks at once
 
-// step (iii): pairs a lane carries at once; pairs a warp drains per window;
-// most step-(i) CTAs (bands)
-#ifndef CCL_RED_SLOTS
-#define CCL_RED_SLOTS 6
-#endif
-constexpr int kRedSlots = CCL_RED_SLOTS;
+// step (iii): pairs a warp drains per window; most step-(i) CTAs' bands
 constexpr int kRedWindowMax = 2048;   // default most pairs per warp window (fewer for small queues)
 constexpr int kMaxBands = 4096;
 constexpr int kRounds = 12;           // most bands a CTA of step (i) takes
@@ -69,6 +64,7 @@ struct __align__(16) BandRec {
 
 struct Params {
     const Inst *insts;         // device table, K entries (K > 1)
+    int32_t *lab_base;         // K > 1: the lowest labels, when all lie within 2^32 labels of them; else null
     Inst one;                  // the instance when K == 1
     int32_t K;
     int32_t link_mode;         // step (iii): 0 root to root, 1 root to the other chain's node
