@@ -439,6 +439,25 @@ void note_settings(ccl_context *ctx, const TuneChoice &tc, const Params &P) {
     ctx->last.analysis_park = resolve_park(tc, P) ? 1 : 0;
 }
 
+// Launches a kernel of steps (ii)-(iv); as a programmatic dependent of the
+// kernel before it in the same call when `chain` is set (chain_wait in the
+// kernel).
+template <typename K>
+cudaError_t launch_tail(K kernel, unsigned grid, unsigned threads, size_t smem, cudaStream_t s, bool chain,
+                        const Params &P) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = chain ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, P);
+}
+
 // Dynamic shared memory of step (iii): its windows per band.
 size_t red_smem(const Params &P) { return sizeof(uint32_t) * (size_t)(P.n_bands + 1); }
 
@@ -452,13 +471,23 @@ ccl_status enqueue_tail(ccl_context *ctx, const Params &P0, bool batched, const 
     // short walks for labels of at most three eighths of L2, else (and where
     // the hand-out or the iteration cap is asked for) the slots
     const bool short_walk = tc.refill && P.iter_cap == 0 && 4 * kChunk * P.n_chunks <= ctx->l2_bytes * 3 / 8;
+    // Programmatic launches for calls of at most one step (i) CTA per SM: the
+    // launch latencies between the steps overlap. Not for larger ones: the next
+    // kernel would start on SMs still set to step (i)'s shared memory and run
+    // without most of its L1 (triangle 4096^2 313 -> 516 us).
+    const bool chain = short_walk && P.n_tiles <= ctx->num_sms;
     const bool near = batched && tc.refill && P.lab_base != nullptr;
     int red_per_sm = blocks_per_sm(ctx, short_walk ? (batched ? 14 : 13) : near ? 15 : batched ? 5 : 4, kRedThreads);
     // beyond L2 fewer warps at once keep more of the labels in use in it:
     // triangle 16384^2 1.27 ms with five CTAs per SM, 1.17 with four (1.32 with
     // three), all with windows of 1024 pairs
     if (!batched && !short_walk && !labels_fit_l2(ctx, P)) red_per_sm = std::min(red_per_sm, 4);
-    const int64_t g_red = (int64_t)ctx->num_sms * red_per_sm;
+    int64_t g_red = (int64_t)ctx->num_sms * red_per_sm;
+    if (!batched) {
+        // no more warps than windows of 64 pairs, a pair per entry at most
+        const int64_t entries = P.dense ? (int64_t)P.one.n * P.nn_width : (int64_t)P.one.nnz;
+        g_red = std::min(g_red, entries / (64 * kRedThreads / 32) + 1);
+    }
     if (profile) CCL_CUDA(cudaEventRecord(ctx->ev[1], s));
     const bool park = resolve_park(tc, P);
     auto analysis = [&]() {
@@ -467,31 +496,20 @@ ccl_status enqueue_tail(ccl_context *ctx, const Params &P0, bool batched, const 
         const int64_t groups = (P.n_chunks + kAnaChunks - 1) / kAnaChunks;
         const unsigned g = (unsigned)grid_for(ctx, (park ? 11 : 2) + (batched ? 1 : 0), tc, groups);
         const size_t smem = park ? park_smem(T) : 0;
-        if (batched && park) k_analysis<true, true><<<g, T, smem, s>>>(A);
-        else if (batched) k_analysis<true, false><<<g, T, smem, s>>>(A);
-        else if (park) k_analysis<false, true><<<g, T, smem, s>>>(A);
-        else k_analysis<false, false><<<g, T, smem, s>>>(A);
+        return launch_tail(batched ? (park ? k_analysis<true, true> : k_analysis<true, false>)
+                                   : (park ? k_analysis<false, true> : k_analysis<false, false>),
+                           g, (unsigned)T, smem, s, chain, A);
     };
-    if (resolve_pre(tc)) {
-        analysis();
-        CCL_CUDA(cudaGetLastError());
-    }
+    if (resolve_pre(tc)) CCL_CUDA(analysis());
     if (profile) CCL_CUDA(cudaEventRecord(ctx->ev[2], s));
-    if (short_walk) {
-        if (batched) k_reduce_park<true><<<(unsigned)g_red, kRedThreads, red_smem(P), s>>>(P);
-        else k_reduce_park<false><<<(unsigned)g_red, kRedThreads, red_smem(P), s>>>(P);
-    } else if (batched) {
-        if (near) k_reduce<true, true, false><<<(unsigned)g_red, kRedThreads, red_smem(P), s>>>(P);
-        else if (tc.refill) k_reduce<true, true, true><<<(unsigned)g_red, kRedThreads, red_smem(P), s>>>(P);
-        else k_reduce<true, false, true><<<(unsigned)g_red, kRedThreads, red_smem(P), s>>>(P);
-    } else {
-        if (tc.refill) k_reduce<false, true, false><<<(unsigned)g_red, kRedThreads, red_smem(P), s>>>(P);
-        else k_reduce<false, false, false><<<(unsigned)g_red, kRedThreads, red_smem(P), s>>>(P);
-    }
-    CCL_CUDA(cudaGetLastError());
+    auto reduce = k_reduce<false, true, false>;
+    if (short_walk) reduce = batched ? k_reduce_park<true> : k_reduce_park<false>;
+    else if (near) reduce = k_reduce<true, true, false>;
+    else if (batched) reduce = tc.refill ? k_reduce<true, true, true> : k_reduce<true, false, true>;
+    else if (!tc.refill) reduce = k_reduce<false, false, false>;
+    CCL_CUDA(launch_tail(reduce, (unsigned)g_red, kRedThreads, red_smem(P), s, chain, P));
     if (profile) CCL_CUDA(cudaEventRecord(ctx->ev[3], s));
-    analysis();
-    CCL_CUDA(cudaGetLastError());
+    CCL_CUDA(analysis());
     if (profile) CCL_CUDA(cudaEventRecord(ctx->ev[4], s));
     return CCL_OK;
 }

@@ -473,6 +473,7 @@ __global__ void __launch_bounds__(kInitThreads, kInitCtas) k_init_dense_tma(Para
     }
     __shared__ unsigned long long band_cnt;
     if (threadIdx.x == 0) band_cnt = 0;
+    chain_next();
     __syncthreads();
     if (warp == kInitConsumers) {
         dense_produce<kGen>(P, st, full, empty, lane);

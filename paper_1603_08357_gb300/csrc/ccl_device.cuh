@@ -135,6 +135,13 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
     return ok != 0;
 }
 
+// Small calls run their kernels as a programmatic chain: each lets the next
+// one start while it still runs (chain_next), and the next one waits, before it
+// touches memory, until the one before has finished and its writes are visible
+// (chain_wait; both do nothing in a kernel launched without the attribute).
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // barrier of the first kThreads threads of the CTA
 template <int kThreads>
 __device__ __forceinline__ void consumers_sync() {
@@ -727,6 +734,7 @@ __global__ void __launch_bounds__(kInitThreads, kInitCtas) k_init(Params P) {
     }
     __shared__ BandSlots bands;
     if (threadIdx.x == 0) bands.taken = 0;
+    chain_next();
     __syncthreads();
     if (warp == kInitConsumers) {               // producer warp
         if (lane == 0) init_produce<kBatched, kGen>(P, st, full, empty, bands);
@@ -852,6 +860,8 @@ constexpr int kParkCap = 32 * kAnaChunks + 32;       // < 32 left + one group's 
 template <bool kBatched, bool kPark>
 __global__ void __launch_bounds__(512, 4) k_analysis(Params P) {
     extern __shared__ int s_park[];                  // kPark: site and label of kParkCap chains per warp
+    chain_next();
+    chain_wait();
     const int lane = threadIdx.x & 31;
     int *s_site = s_park + (threadIdx.x >> 5) * (2 * kParkCap), *s_x = s_site + kParkCap;
     const unsigned lt = (1u << lane) - 1u;
@@ -1332,6 +1342,8 @@ __global__ void __launch_bounds__(kRedThreads, kBatched ? 6 : 8) k_reduce_park(P
     __shared__ long long s_warp[kRedThreads / 32];
     __shared__ int2 s_pair[kRedThreads / 32][kParkList];
     __shared__ int s_k[kBatched ? kRedThreads / 32 : 1][kBatched ? kParkList : 1];
+    chain_next();
+    chain_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
     const long long nwarps = (long long)gridDim.x * (kRedThreads / 32);
