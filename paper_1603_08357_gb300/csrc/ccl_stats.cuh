@@ -18,19 +18,26 @@ constexpr int kRelThreads = 256;
 constexpr int kRelPerThread = 32;
 constexpr int kRelBlock = kRelThreads * kRelPerThread;   // sites per relabel block
 
-// number of roots (label[i] == i) in each block of kRelBlock sites
+// number of roots (label[i] == i) in each block of kRelBlock sites, and a bit
+// per site, set for roots. A warp takes 1024 consecutive sites and keeps the 32
+// ballots one per lane.
 __global__ void __launch_bounds__(kRelThreads) k_root_counts(int32_t n, const int32_t *__restrict__ lab,
-                                                             int32_t *__restrict__ block_cnt) {
+                                                             int32_t *__restrict__ block_cnt,
+                                                             uint32_t *__restrict__ roots) {
     __shared__ int s_w[kRelThreads / 32];
-    const int64_t base = (int64_t)blockIdx.x * kRelBlock;
-    int c = 0;
-#pragma unroll 4
+    static_assert(kRelPerThread == 32, "one ballot per lane");
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t base = (int64_t)blockIdx.x * kRelBlock + warp * (32 * kRelPerThread) + lane;
+    unsigned mine = 0;                  // lane u: the roots among the warp's u-th 32 sites
+#pragma unroll 8
     for (int u = 0; u < kRelPerThread; ++u) {
-        const int64_t i = base + (int64_t)u * kRelThreads + threadIdx.x;
-        if (i < n) c += __ldg(lab + i) == (int32_t)i;
+        const int64_t i = base + 32 * u;
+        const unsigned b = __ballot_sync(kFull, i < n && __ldg(lab + i) == (int32_t)i);
+        if (lane == u) mine = b;
     }
-    c = __reduce_add_sync(kFull, c);
-    if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5] = c;
+    roots[(int64_t)blockIdx.x * kRelThreads + threadIdx.x] = mine;
+    const int c = __reduce_add_sync(kFull, __popc(mine));
+    if (lane == 0) s_w[warp] = c;
     __syncthreads();
     if (threadIdx.x == 0) {
         int t = 0;
@@ -65,24 +72,17 @@ __global__ void __launch_bounds__(1024) k_scan_counts(int32_t nb, int32_t *__res
 }
 
 // sequential id of every root: its block's offset plus the roots before it in
-// the block, in site order; zeroes the size counter of each id. A warp takes
-// 1024 consecutive sites, keeps the 32 root ballots one per lane and needs the
-// other warps' totals once, so the block meets at one barrier (stepping the
+// the block, in site order; zeroes the size counter of each id. The roots come
+// from the bits of k_root_counts, not from the labels again, and a warp needs
+// the other warps' totals once, so the block meets at one barrier (stepping the
 // whole block through 256 sites at a time took 96 barriers).
-__global__ void __launch_bounds__(kRelThreads) k_root_ids(int32_t n, const int32_t *__restrict__ lab,
+__global__ void __launch_bounds__(kRelThreads) k_root_ids(const uint32_t *__restrict__ roots,
                                                           const int32_t *__restrict__ block_off,
                                                           int32_t *__restrict__ out, int32_t *__restrict__ sizes) {
     __shared__ int32_t s_w[kRelThreads / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t base = (int64_t)blockIdx.x * kRelBlock + warp * (32 * kRelPerThread) + lane;
-    static_assert(kRelPerThread == 32, "one ballot per lane");
-    unsigned mine = 0;                  // lane u: the roots among the warp's u-th 32 sites
-#pragma unroll 8
-    for (int u = 0; u < kRelPerThread; ++u) {
-        const int64_t i = base + 32 * u;
-        const unsigned b = __ballot_sync(kFull, i < n && __ldg(lab + i) == (int32_t)i);
-        if (lane == u) mine = b;
-    }
+    const unsigned mine = roots[(int64_t)blockIdx.x * kRelThreads + threadIdx.x];
     int incl = __popc(mine);
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(kRelThreads) k_root_ids(int32_t n, const int32
 // every warp of the GPU adds to the giant cluster's counter, one address:
 // a realisation of honeycomb 2896^2 at 1.25 p_c (labelling, spanning, largest
 // cluster) took 845 us that way and 448 this way; relabelling triangle 4096^2
-// at 0.9 p_c, whose ids and sizes are one pass now, 205 and 118.
+// at 0.9 p_c, whose ids and sizes are one pass now, 205 and 110.
 // Tracks the largest (count, smallest value) key seen after an add.
 struct WarpCounter {
     int32_t *cnt;
