@@ -507,8 +507,10 @@ struct RowsRes {
 // smallest neighbour and its place with one minimum. Warp instructions per 64
 // sites on triangle 3000^2: 537 -> 308. Times of step (i), before -> after:
 // triangle 4096^2 160 -> 118 us (4.6 TB/s; streaming alone takes 88),
-// triangle 16384^2 2.44 -> 1.83 ms, honeycomb 2048^2 71 -> 55 us, Bethe
-// lattice of 24 shells 390 -> 364 us, 1024 mixed instances 4.98 -> 4.80 ms.
+// triangle 16384^2 2.44 -> 1.80 ms, honeycomb 2048^2 71 -> 55 us, Bethe
+// lattice of 24 shells 390 -> 364 us, and 325 with the mixed rows' entries past
+// a row's end read and masked instead of branched around (1024 mixed instances
+// 3.39 -> 3.15 ms by that alone).
 // (Two rows a lane and sixteen warps with the same scan: 140 us on triangle
 // 4096^2; two stages and three CTAs per SM: 124 us there, 347 us on the Bethe
 // lattice.) A call of few tiles pays for the longer lanes: honeycomb 64^2
@@ -532,7 +534,10 @@ __device__ __forceinline__ void scan_rows(const Params &P, const Stage &S, const
             const int32_t rel = tc.rb0 + a[k];
             const uint32_t *bw = S.bw + (rel >> 5);
             // (an empty row's may lie past the copied words)
-            if (kD > 0 || d[k] > 0) w[k] = __funnelshift_r(bw[0], bw[1], (uint32_t)rel & 31u) & 0xffu;
+            if (kD > 0 || d[k] > 0) w[k] = __funnelshift_r(bw[0], bw[1], (uint32_t)rel & 31u);
+            w[k] &= kD > 0 ? 0xffu : 0xffu >> (kRowRegs - d[k]);        // the row's own bits
+        } else {
+            w[k] = kD > 0 ? 0xffu : 0xffu >> (kRowRegs - d[k]);
         }
     }
     // Open entries as keys 8 j + t (closed ones above every site's): the
@@ -540,11 +545,13 @@ __device__ __forceinline__ void scan_rows(const Params &P, const Stage &S, const
     // is an open lower one iff its key is below 8 i. The signs of the keys'
     // differences to 8 i collect in `low`, entry t of T at bit T - 1 - t.
     // Keys need sites below 2^28; kWide keeps the neighbour and its place apart.
-    auto entry = [&](int k, int t, int32_t j) {
+    // (entries past a row's end, closed by w, are read all the same: the scan of
+    // mixed rows does not branch)
+    auto entry = [&](int k, int t, int32_t j, bool in_row) {
         const int32_t i = s00 + kChunk * k + lane;
-        jmax = max(jmax, (uint32_t)j);
-        bool open = kGen || ((w[k] >> t) & 1u);
-        if (kGen) open = (uint32_t)j < (uint32_t)i && gen_bond_open(P.gen_seed, P.gen_thr, (uint32_t)j, (uint32_t)i);
+        jmax = max(jmax, in_row ? (uint32_t)j : 0u);
+        bool open = (w[k] >> t) & 1u;
+        if (kGen) open = open && (uint32_t)j < (uint32_t)i && gen_bond_open(P.gen_seed, P.gen_thr, (uint32_t)j, (uint32_t)i);
         if (kWide) {
             const bool lower = open && (uint32_t)j < (uint32_t)i;
             low[k] = 2u * low[k] + (lower ? 1u : 0u);
@@ -562,22 +569,20 @@ __device__ __forceinline__ void scan_rows(const Params &P, const Stage &S, const
 #pragma unroll
             for (int k = 0; k < kRows; ++k) {
                 const int2 jj = *reinterpret_cast<const int2 *>(col[k] + t);
-                entry(k, t, jj.x);
-                entry(k, t + 1, jj.y);
+                entry(k, t, jj.x, true);
+                entry(k, t + 1, jj.y, true);
             }
     } else if (kD > 0) {
 #pragma unroll
         for (int t = 0; t < kD; ++t)
 #pragma unroll
-            for (int k = 0; k < kRows; ++k) entry(k, t, col[k][t]);
+            for (int k = 0; k < kRows; ++k) entry(k, t, col[k][t], true);
     } else {
 #pragma unroll
         for (int t = 0; t < kRowRegs; ++t) {
             if (t >= dmax) break;
 #pragma unroll
-            for (int k = 0; k < kRows; ++k)
-                if (t < d[k]) entry(k, t, col[k][t]);
-                else low[k] <<= 1;
+            for (int k = 0; k < kRows; ++k) entry(k, t, col[k][t], t < d[k]);
         }
     }
     bad = jmax >= (uint32_t)n;
