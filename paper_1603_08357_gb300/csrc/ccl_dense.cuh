@@ -426,13 +426,14 @@ __device__ __forceinline__ void dense_emit_rows(const Params &P, const DenseStag
     uint32_t mm = q.res;
     int2 *qp = P.q + slot;
     for (int it = 0; it < iters; ++it) {
-        if (mm) {
-            const int t = __ffs(mm) - 1;
-            mm &= mm - 1;
-            const int k = last - (t & 7);
-            const int32_t up = t & 8 ? q.lab[1] : q.lab[0], up2 = t & 8 ? q.lab[3] : q.lab[2];
-            *qp++ = make_int2(t & 16 ? up2 : up, S.nn[k][S.h.off[k].x + loc0 + kChunk * (t >> 3)]);
-        }
+        const bool put = mm != 0;
+        const int t = put ? __ffs(mm) - 1 : 0;
+        mm &= mm - 1;
+        const int k = last - (t & 7);
+        const int32_t up = t & 8 ? q.lab[1] : q.lab[0], up2 = t & 8 ? q.lab[3] : q.lab[2];
+        const int2 pr = make_int2(t & 16 ? up2 : up, S.nn[k][S.h.off[k].x + loc0 + kChunk * (t >> 3)]);
+        if (put) *qp = pr;
+        ++qp;
     }
 }
 

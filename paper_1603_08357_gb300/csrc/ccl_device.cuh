@@ -700,8 +700,11 @@ __device__ __forceinline__ void init_emit_chunk(const Params &P, const Stage &S,
 }
 
 // The residual pairs of a lane's four rows on the register path, in one loop
-// with a warp-uniform trip count, so the warp neither diverges nor loops four
-// times. The warp's queue slots have been checked against the queue's end.
+// with a warp-uniform trip count and without branches, so the warp neither
+// diverges nor loops four times (with a branch around lanes that have no pair
+// left: step (i) of 1024 mixed instances 3.15 ms instead of 3.08, of the Bethe
+// lattice 325 us instead of 318). The warp's queue slots have been checked
+// against the queue's end.
 template <bool kBatched>
 __device__ __forceinline__ void init_emit_rows(const Params &P, const Stage &S, const TileHdr &h, const RowsRes &q,
                                                int64_t slot, int rr) {
@@ -710,15 +713,20 @@ __device__ __forceinline__ void init_emit_rows(const Params &P, const Stage &S, 
     int2 *qp = P.q + slot;
     int32_t *kp = kBatched ? P.qk + slot : nullptr;
     for (int it = 0; it < iters; ++it) {
-        if (mm) {
-            const int t = __ffs(mm) - 1;
-            mm &= mm - 1;
-            int32_t off = t & 8 ? q.off[1] : q.off[0], up = t & 8 ? q.lab[1] : q.lab[0];
-            const int32_t off2 = t & 8 ? q.off[3] : q.off[2], up2 = t & 8 ? q.lab[3] : q.lab[2];
-            if (t & 16) { off = off2; up = up2; }
-            *qp++ = make_int2(up, S.ci[off + q.last - (t & 7)]);
-            if (kBatched) *kp++ = h.k;
+        // (a lane without a pair left reads some column and stores nothing)
+        const bool put = mm != 0;
+        const int t = put ? __ffs(mm) - 1 : 0;
+        mm &= mm - 1;
+        int32_t off = t & 8 ? q.off[1] : q.off[0], up = t & 8 ? q.lab[1] : q.lab[0];
+        const int32_t off2 = t & 8 ? q.off[3] : q.off[2], up2 = t & 8 ? q.lab[3] : q.lab[2];
+        if (t & 16) { off = off2; up = up2; }
+        const int2 pr = make_int2(up, S.ci[off + q.last - (t & 7)]);
+        if (put) {
+            *qp = pr;
+            if (kBatched) *kp = h.k;
         }
+        ++qp;
+        if (kBatched) ++kp;
     }
 }
 
