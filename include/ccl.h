@@ -99,7 +99,9 @@ typedef enum {
     CCL_OPT_CTAS_PER_SM = 4,   /* persistent CTAs per SM of the analysis kernel; 0 (default) = occupancy maximum */
     CCL_OPT_LINK_MODE = 5,     /* step (iii): 0 (default) a root is linked under the other tree's
                                   root, as in Algorithm 1; 1 under the node the other chain has
-                                  reached (same atomicMin loop, shorter walks on trees) */
+                                  reached (same atomicMin loop, shorter walks on trees). With 0
+                                  a large instance of few residual pairs (a quarter of the sites
+                                  at most) uses 1 where the ends of its pairs lie far apart */
     CCL_OPT_REFILL = 6,        /* step (iii): 1 (default) each thread serves a fixed stride of the
                                   residual pairs (and, when the call's labels take at most three
                                   eighths of L2, pairs with long chains are set aside and finished

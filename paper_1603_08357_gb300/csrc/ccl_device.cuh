@@ -1079,9 +1079,10 @@ __device__ __forceinline__ long long block_excl_scan(long long v, long long *s_w
 }
 
 // Cuts the call's pairs into windows: fills s_win[0 .. n_bands], stores the
-// statistics and returns the number of windows. The whole CTA calls.
+// statistics and returns the number of windows; total = all pairs. The whole
+// CTA calls.
 __device__ __forceinline__ uint32_t red_windows(const Params &P, uint32_t *s_win, long long *s_warp, int lane,
-                                                long long nwarps) {
+                                                long long nwarps, long long &total) {
     // Every warp takes as many windows as every other, the fewest that keeps
     // them below the limit: a last round of a few windows leaves the chip idle
     // (Bethe lattice of 24 shells, 5.5M pairs: 254 us with windows of 1024 pairs,
@@ -1093,7 +1094,6 @@ __device__ __forceinline__ uint32_t red_windows(const Params &P, uint32_t *s_win
         const long long waves = max((total + room * wmax - 1) / (room * wmax), 1ll);
         return min(max((total + room * waves - 1) / (room * waves), 64ll), wmax);
     };
-    long long total;
     if (P.n_bands <= 32) {
         // a small call: every warp by itself, without barriers (all write the
         // same values)
@@ -1183,7 +1183,10 @@ __global__ void __launch_bounds__(kRedThreads, !kBatched ? 5 : kFar ? 4 : 3) k_r
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
     const long long nwarps = (long long)gridDim.x * (kRedThreads / 32);
-    const long long nwin = red_windows(P, s_win, s_warp, lane, nwarps);
+    long long total;
+    const long long nwin = red_windows(P, s_win, s_warp, lane, nwarps, total);
+    // Few pairs: the clusters are small or tree-like (see `far` below).
+    const bool few = !kBatched && kStatic && total <= P.one.n / 4;
 #ifdef CCL_DEVICE_STATS
     unsigned long long st_hops = 0, st_atom = 0, st_iter = 0;
 #endif
@@ -1214,116 +1217,130 @@ __global__ void __launch_bounds__(kRedThreads, !kBatched ? 5 : kFar ? 4 : 3) k_r
             pnext += 32;
         };
         if (kStatic && pnext < wlen) fetch();
-        int32_t *L[kRedSlots];
-        uint32_t off[kRedSlots];
-        int32_t a[kRedSlots], b[kRedSlots], st[kRedSlots];
+        // Link mode 1 (a root goes under the other chain's node, whose own root
+        // need not be found) where it cannot build deep trees: an instance of
+        // few pairs whose ends lie far apart in the numbering, a sixteenth of
+        // the sites or more in half of the window's first 32 pairs. On randomly
+        // numbered trees it saves a quarter of the loads (Bethe lattice of 24
+        // shells at 0.5 / 1 / 1.5 p_c 71 / 235 / 498 -> 49 / 173 / 391 us); on
+        // lattices it builds chains along the rows (triangle 4096^2 94 -> 613),
+        // and on a random graph of 1.07 pairs per site 956 -> 1655.
+        const bool far = few && __popc(__ballot_sync(kFull, pf_ok && abs(pf.x - pf.y) > P.one.n / 16)) >= 16;
+        // (one copy of the loop per link choice: with the choice in a register
+        // the common copy was 6 % slower)
+        const auto drain = [&](const uint32_t table) {
+            int32_t *L[kRedSlots];
+            uint32_t off[kRedSlots];
+            int32_t a[kRedSlots], b[kRedSlots], st[kRedSlots];
 #pragma unroll
-        for (int u = 0; u < kRedSlots; ++u) {
-            st[u] = kTaskDone;
-            L[u] = nullptr;
-            off[u] = 0;
-            a[u] = b[u] = 0;
-        }
-        for (;;) {
-            if (kStatic) {
-                // at most one empty slot per lane and round takes the prefetched pair
-                int take = -1;
+            for (int u = 0; u < kRedSlots; ++u) {
+                st[u] = kTaskDone;
+                L[u] = nullptr;
+                off[u] = 0;
+                a[u] = b[u] = 0;
+            }
+            for (;;) {
+                if (kStatic) {
+                    // at most one empty slot per lane and round takes the prefetched pair
+                    int take = -1;
 #pragma unroll
-                for (int u = kRedSlots - 1; u >= 0; --u)
-                    if (st[u] == kTaskDone) take = u;
-                if (take >= 0 && pf_ok) {
-                    const int32_t na = max(pf.x, pf.y), nb = min(pf.x, pf.y);
-                    if (kBatched && pfk != lk) {
-                        lk = pfk;
-                        int32_t *l = P.insts[pfk].labels;
-                        if (kFar) llab = l; else loff = (uint32_t)(l - base);
-                    }
-#pragma unroll
-                    for (int u = 0; u < kRedSlots; ++u)
-                        if (u == take) {
-                            a[u] = na;
-                            b[u] = nb;
-                            st[u] = kTaskChase;
-                            if (kFar) L[u] = llab;
-                            if (kOff) off[u] = loff;
+                    for (int u = kRedSlots - 1; u >= 0; --u)
+                        if (st[u] == kTaskDone) take = u;
+                    if (take >= 0 && pf_ok) {
+                        const int32_t na = max(pf.x, pf.y), nb = min(pf.x, pf.y);
+                        if (kBatched && pfk != lk) {
+                            lk = pfk;
+                            int32_t *l = P.insts[pfk].labels;
+                            if (kFar) llab = l; else loff = (uint32_t)(l - base);
                         }
-                    pf_ok = false;
-                    if (pnext < wlen) fetch();
-                }
-            } else {
-                // refill empty slots with the window's next pairs, in order (the
-                // tests are warp-uniform: nothing runs once the window is handed out)
-                if (nxt < wlen) {
 #pragma unroll
-                    for (int u = 0; u < kRedSlots; ++u) {
-                        const unsigned need = __ballot_sync(kFull, st[u] == kTaskDone);
-                        if (need == 0) continue;
-                        const int pos = nxt + __popc(need & lt);
-                        if (st[u] == kTaskDone && pos < wlen) {
-                            const int2 pr = wq[pos];
-                            if (kBatched) {
-                                const int k = wqk[pos];
-                                if (k != lk) {
-                                    lk = k;
-                                    int32_t *l = P.insts[k].labels;
-                                    if (kFar) llab = l; else loff = (uint32_t)(l - base);
-                                }
+                        for (int u = 0; u < kRedSlots; ++u)
+                            if (u == take) {
+                                a[u] = na;
+                                b[u] = nb;
+                                st[u] = kTaskChase;
                                 if (kFar) L[u] = llab;
                                 if (kOff) off[u] = loff;
                             }
-                            a[u] = max(pr.x, pr.y);
-                            b[u] = min(pr.x, pr.y);
-                            st[u] = kTaskChase;
+                        pf_ok = false;
+                        if (pnext < wlen) fetch();
+                    }
+                } else {
+                    // refill empty slots with the window's next pairs, in order (the
+                    // tests are warp-uniform: nothing runs once the window is handed out)
+                    if (nxt < wlen) {
+#pragma unroll
+                        for (int u = 0; u < kRedSlots; ++u) {
+                            const unsigned need = __ballot_sync(kFull, st[u] == kTaskDone);
+                            if (need == 0) continue;
+                            const int pos = nxt + __popc(need & lt);
+                            if (st[u] == kTaskDone && pos < wlen) {
+                                const int2 pr = wq[pos];
+                                if (kBatched) {
+                                    const int k = wqk[pos];
+                                    if (k != lk) {
+                                        lk = k;
+                                        int32_t *l = P.insts[k].labels;
+                                        if (kFar) llab = l; else loff = (uint32_t)(l - base);
+                                    }
+                                    if (kFar) L[u] = llab;
+                                    if (kOff) off[u] = loff;
+                                }
+                                a[u] = max(pr.x, pr.y);
+                                b[u] = min(pr.x, pr.y);
+                                st[u] = kTaskChase;
+                            }
+                            nxt = min(nxt + __popc(need), wlen);
+                            if (nxt >= wlen) break;
                         }
-                        nxt = min(nxt + __popc(need), wlen);
-                        if (nxt >= wlen) break;
                     }
                 }
-            }
 #ifdef CCL_DEVICE_STATS
-            st_iter++;
+                st_iter++;
 #endif
-            // issue: one load or one atomicMin per live slot
-            int32_t v[kRedSlots];
+                // issue: one load or one atomicMin per live slot
+                int32_t v[kRedSlots];
 #pragma unroll
-            for (int u = 0; u < kRedSlots; ++u) {
-                const int32_t x = st[u] == kTaskRoot ? b[u] : a[u];
-                int32_t *ptr = kFar ? L[u] + x : base + (uint32_t)((kOff ? off[u] : 0u) + (uint32_t)x);
-                v[u] = 0;
-                if (st[u] == kTaskMerge) v[u] = atomicMin(ptr, b[u]);
-                else if (st[u] != kTaskDone) v[u] = red_load(ptr);
-            }
-            // use: the next state of every slot (no divergent paths). With
-            // mx = max(y, b) and mn = min(y, b) every transition sets b = mn
-            // and a = mx, except Root, which keeps a:
-            //   Chase (y = label[a]): y == a means a root, so mx = a, mn = b;
-            //     otherwise the walk goes on from the larger node;
-            //   Root (y = label[b] <= b): b = y;
-            //   Merge (y = old label[a]): Algorithm 1 continues with (old, b)
-            //     when old > b and with (b, old) when old < b.
-            // The next state is looked up by (state, y == a, y == b).
-            const uint32_t table = P.link_mode ? kRedNextLink1 : kRedNextLink0;
-            bool any = false;
+                for (int u = 0; u < kRedSlots; ++u) {
+                    const int32_t x = st[u] == kTaskRoot ? b[u] : a[u];
+                    int32_t *ptr = kFar ? L[u] + x : base + (uint32_t)((kOff ? off[u] : 0u) + (uint32_t)x);
+                    v[u] = 0;
+                    if (st[u] == kTaskMerge) v[u] = atomicMin(ptr, b[u]);
+                    else if (st[u] != kTaskDone) v[u] = red_load(ptr);
+                }
+                // use: the next state of every slot (no divergent paths). With
+                // mx = max(y, b) and mn = min(y, b) every transition sets b = mn
+                // and a = mx, except Root, which keeps a:
+                //   Chase (y = label[a]): y == a means a root, so mx = a, mn = b;
+                //     otherwise the walk goes on from the larger node;
+                //   Root (y = label[b] <= b): b = y;
+                //   Merge (y = old label[a]): Algorithm 1 continues with (old, b)
+                //     when old > b and with (b, old) when old < b.
+                // The next state is looked up by (state, y == a, y == b).
+                bool any = false;
 #pragma unroll
-            for (int u = 0; u < kRedSlots; ++u) {
-                const int32_t y = v[u], A = a[u], Bv = b[u];
-                const int s = st[u];
+                for (int u = 0; u < kRedSlots; ++u) {
+                    const int32_t y = v[u], A = a[u], Bv = b[u];
+                    const int s = st[u];
 #ifdef CCL_DEVICE_STATS
-                st_hops += (s == kTaskChase || s == kTaskRoot);
-                st_atom += (s == kTaskMerge);
+                    st_hops += (s == kTaskChase || s == kTaskRoot);
+                    st_atom += (s == kTaskMerge);
 #endif
-                const uint32_t idx = ((uint32_t)s << 2) | ((y == A) ? 2u : 0u) | ((y == Bv) ? 1u : 0u);
-                a[u] = s == kTaskRoot ? A : max(y, Bv);
-                b[u] = min(y, Bv);
-                st[u] = (int32_t)((table >> (2u * idx)) & 3u);
-                any |= st[u] != kTaskDone;
+                    const uint32_t idx = ((uint32_t)s << 2) | ((y == A) ? 2u : 0u) | ((y == Bv) ? 1u : 0u);
+                    a[u] = s == kTaskRoot ? A : max(y, Bv);
+                    b[u] = min(y, Bv);
+                    st[u] = (int32_t)((table >> (2u * idx)) & 3u);
+                    any |= st[u] != kTaskDone;
+                }
+                if (!__any_sync(kFull, any || pf_ok) && (kStatic || nxt >= wlen)) break;
+                if (++rounds > round_cap) {
+                    raise_err(P.err, kErrNonconv);
+                    break;
+                }
             }
-            if (!__any_sync(kFull, any || pf_ok) && (kStatic || nxt >= wlen)) break;
-            if (++rounds > round_cap) {
-                raise_err(P.err, kErrNonconv);
-                break;
-            }
-        }
+        };
+        if (far) drain(kRedNextLink1);
+        else drain(P.link_mode ? kRedNextLink1 : kRedNextLink0);
     }
 #ifdef CCL_DEVICE_STATS
     if (st_hops) atomicAdd(P.counters + 1, st_hops);
@@ -1360,7 +1377,8 @@ __global__ void __launch_bounds__(kRedThreads, kBatched ? 6 : 8) k_reduce_park(P
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
     const long long nwarps = (long long)gridDim.x * (kRedThreads / 32);
-    const long long nwin = red_windows(P, s_win, s_warp, lane, nwarps);
+    long long total;
+    const long long nwin = red_windows(P, s_win, s_warp, lane, nwarps, total);
     const bool eager = P.link_mode != 0;            // link a root to the other end's node, not its root
     // the labels of the lane's last instance
     int lk = -1;

@@ -112,3 +112,17 @@ def test_long_chains(rungs, link):
             assert np.array_equal(gpu_label(c, lat), oracle.uf_label(lat))
     finally:
         ccl.ccl_context_destroy(c)
+
+
+def test_far_pairs_beyond_l2(ctx):
+    """Windows that take link mode 1 by themselves (few pairs, far ends) next to
+    windows that do not: a randomly numbered tree, and the same sites with a
+    lattice in the second half, both beyond L2."""
+    tree = L.cayley(3, 23, 0.6, 3, perm_seed=7)
+    sq = L.square(4000, 0.55, 5)
+    both = L.Lattice("random", tree.n + sq.n, tree.nnz + sq.nnz,
+                     np.concatenate([tree.row_ptr, sq.row_ptr[1:] + tree.nnz]).astype(np.int32),
+                     np.concatenate([tree.col_idx, sq.col_idx + tree.n]).astype(np.int32),
+                     L.pack_bits(np.concatenate([L.unpack_bits(tree.open_bits, tree.nnz), L.unpack_bits(sq.open_bits, sq.nnz)])), 0.5, 1)
+    for lat in (tree, both):
+        assert np.array_equal(gpu_label(ctx, lat), oracle.uf_label(lat))
