@@ -30,7 +30,7 @@ namespace {
 
 constexpr int64_t kNoAllocMaxEntries = int64_t(1) << 21;   // CSR entries (residual-pair slots)
 constexpr size_t kOffErr = 0;                               // unsigned error word
-constexpr size_t kOffCounters = 256;                        // 4 x u64 counters
+constexpr size_t kOffCounters = 256;                        // kCounters x u64 counters
 constexpr size_t kOffBand = 512;                            // kMaxBands BandRec
 constexpr size_t kOffQueue = kOffBand + sizeof(BandRec) * kMaxBands;
 constexpr size_t kScratchBytes = kOffQueue + sizeof(int2) * (size_t)kNoAllocMaxEntries;

@@ -126,3 +126,27 @@ def test_far_pairs_beyond_l2(ctx):
                      L.pack_bits(np.concatenate([L.unpack_bits(tree.open_bits, tree.nnz), L.unpack_bits(sq.open_bits, sq.nnz)])), 0.5, 1)
     for lat in (tree, both):
         assert np.array_equal(gpu_label(ctx, lat), oracle.uf_label(lat))
+
+
+@pytest.mark.parametrize("L_cells", [16, 200, 400])
+def test_small_call_in_a_users_graph(ctx, L_cells):
+    """A call captured into a user's graph: the programmatic chain of small
+    calls (16 and 200 cells) and the ordinary launches (400), replayed on inputs
+    rewritten in place."""
+    a, b = (L.honeycomb(L_cells, p, seed) for p, seed in ((0.6527, 3), (0.75, 4)))
+    rp, ci, bits = (torch.from_numpy(x).to(DEV) for x in (a.row_ptr, a.col_idx, a.open_bits.view(np.int32)))
+    out = torch.full((a.n,), -7, dtype=torch.int32, device=DEV)
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    assert ccl.ccl_label(ctx, a.n, a.nnz, rp, ci, bits, out, s) == ccl.CCL_OK    # sizes the workspace
+    assert ccl.ccl_sync(ctx, s) == ccl.CCL_OK
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        assert ccl.ccl_label(ctx, a.n, a.nnz, rp, ci, bits, out, s) == ccl.CCL_OK
+    for x in (a, b, a):
+        out.fill_(-7)
+        bits.copy_(torch.from_numpy(x.open_bits.view(np.int32)))
+        for _ in range(3):
+            g.replay()
+        torch.cuda.synchronize()
+        assert np.array_equal(out.cpu().numpy(), oracle.uf_label(x))
