@@ -418,15 +418,18 @@ bool resolve_park(const TuneChoice &tc, const Params &P) {
     return tc.ana_seq && P.iter_cap == 0 && tc.ana_park > 0;    // (the iteration-cap test option takes the plain walk)
 }
 
-// Whether step (ii) runs as a pass of its own: as set, else not. Steps (i) and
-// (iii) do without it (the band shortcut and the in-window jump of step (i)
+// Whether step (ii) runs over all sites: as set, else not. Near p_c steps (i)
+// and (iii) do without it (the band shortcut and the in-window jump of step (i)
 // leave short chains, and step (iii)'s search is bounded by the window's
 // slowest pair, not by the mean chain), and step (iv) repeats its work: on one
 // GB300 a call with / without it took 356 / 313 us (triangle 4096^2 at p_c),
 // 1105 / 910 us (Bethe lattice, 24 shells, random numbering), 5.73 / 5.05 ms
 // (triangle 16384^2), 11.3 / 9.9 ms (1024 mixed instances) and 30.2 / 30.6 us
 // (honeycomb 64^2).
+// Left to the library, the pass samples the labels of each instance and walks
+// only where chains are long (k_analysis), which the data alone can tell.
 bool resolve_pre(const TuneChoice &tc) { return tc.pre_analysis > 0; }
+constexpr int kSampleGroup = 64;     // groups per run of the sampling pass beyond L2
 
 // Records in the context's statistics the settings a call runs with.
 void note_settings(ccl_context *ctx, const TuneChoice &tc, const Params &P) {
@@ -490,17 +493,21 @@ ccl_status enqueue_tail(ccl_context *ctx, const Params &P0, bool batched, const 
     }
     if (profile) CCL_CUDA(cudaEventRecord(ctx->ev[1], s));
     const bool park = resolve_park(tc, P);
-    auto analysis = [&]() {
+    auto analysis = [&](bool sample) {
         Params A = P;
         if (!tc.ana_seq) A.ana_group = 1;       // groups interleaved over the warps
+        if (sample && A.ana_group > 0) A.ana_group = kSampleGroup;
         const int64_t groups = (P.n_chunks + kAnaChunks - 1) / kAnaChunks;
         const unsigned g = (unsigned)grid_for(ctx, (park ? 11 : 2) + (batched ? 1 : 0), tc, groups);
+        if (sample)
+            return launch_tail(batched ? k_analysis<true, false, true> : k_analysis<false, false, true>, g, (unsigned)T,
+                               0, s, chain, A);
         const size_t smem = park ? park_smem(T) : 0;
         return launch_tail(batched ? (park ? k_analysis<true, true> : k_analysis<true, false>)
                                    : (park ? k_analysis<false, true> : k_analysis<false, false>),
                            g, (unsigned)T, smem, s, chain, A);
     };
-    if (resolve_pre(tc)) CCL_CUDA(analysis());
+    if (tc.pre_analysis != 0) CCL_CUDA(analysis(!resolve_pre(tc)));
     if (profile) CCL_CUDA(cudaEventRecord(ctx->ev[2], s));
     auto reduce = k_reduce<false, true, false>;
     if (short_walk) reduce = batched ? k_reduce_park<true> : k_reduce_park<false>;
@@ -509,7 +516,7 @@ ccl_status enqueue_tail(ccl_context *ctx, const Params &P0, bool batched, const 
     else if (!tc.refill) reduce = k_reduce<false, false, false>;
     CCL_CUDA(launch_tail(reduce, (unsigned)g_red, kRedThreads, red_smem(P), s, chain, P));
     if (profile) CCL_CUDA(cudaEventRecord(ctx->ev[3], s));
-    CCL_CUDA(analysis());
+    CCL_CUDA(analysis(false));
     if (profile) CCL_CUDA(cudaEventRecord(ctx->ev[4], s));
     return CCL_OK;
 }

@@ -870,7 +870,22 @@ constexpr int kParkCap = 32 * kAnaChunks + 32;       // < 32 left + one group's 
 // few long chains do not hold up the lanes of a whole group. (Slower than
 // waiting on every input measured: triangle 4096^2 55 us, 1024 mixed instances
 // 1.53 ms.)
-template <bool kBatched, bool kPark>
+//
+// kSample = true (step (ii) when the library chooses): an instance is left alone
+// unless fewer than one in kSampleRoots of kSampleChunks chunks spread over it
+// are roots (which sites are roots does not change here, so every warp decides
+// alike). A chain ends at each hop with about that probability: where roots
+// are common chains are a few hops long and step (iii) does better alone, where
+// they are rare each of its pairs would walk a long chain. Calls without / with
+// the pass, and by sample: honeycomb 362^2 at 1.5 p_c 109 / 45 / 44 us, 1448^2
+// there 233 / 140 / 143, 2896^2 581 / 308 / 302, square 2048^2 200 / 131 / 134,
+// triangle 2048^2 156 / 124 / 126; at p_c, left alone, it costs its launch and
+// one read: triangle 4096^2 250 / 279 / 254, honeycomb 256^2 33 / 36 / 36. The
+// line lies at 0.125: triangles at 1.5 p_c (0.11) and honeycomb lattices at 1.2
+// p_c (0.13) are about even. Deciding per stretch of 96 sites instead costs
+// more than either at the line (triangle 2048^2 at 1.5 p_c 173).
+constexpr int kSampleRoots = 8, kSampleChunks = 12;
+template <bool kBatched, bool kPark, bool kSample = false>
 __global__ void __launch_bounds__(512, 4) k_analysis(Params P) {
     extern __shared__ int s_park[];                  // kPark: site and label of kParkCap chains per warp
     chain_next();
@@ -911,6 +926,19 @@ __global__ void __launch_bounds__(512, 4) k_analysis(Params P) {
         cnt = base;
         __syncwarp();
     };
+    const auto sample = [&]() {
+        const int32_t step = n / kSampleChunks;
+        int roots = 0, sites = 0;
+#pragma unroll
+        for (int u = 0; u < kSampleChunks; ++u) {
+            const int32_t i = u * step + step / 2 + lane;
+            roots += __popc(__ballot_sync(kFull, i < n && lab[min(i, n - 1)] == i));
+            sites += __popc(__ballot_sync(kFull, i < n));
+        }
+        return roots * kSampleRoots < sites;
+    };
+    bool walk = kSample && !kBatched && sample();
+    if (kSample && !kBatched && !walk) return;
     for (int64_t run = wid * G; run < ngroups; run += nwarps * G) {
         int64_t c = run * kAnaChunks;
         const int64_t c_end = min((run + G) * kAnaChunks, P.n_chunks);
@@ -921,6 +949,7 @@ __global__ void __launch_bounds__(512, 4) k_analysis(Params P) {
                 kc_hi = kc + 1 < P.K ? P.insts[kc + 1].chunk_begin : P.n_chunks;
                 lab = P.insts[kc].labels;
                 n = P.insts[kc].n;
+                if (kSample) walk = sample();
             }
             // the stretch of this run inside the instance: the lane's sites s
             // + 32 u below s_end
@@ -928,6 +957,7 @@ __global__ void __launch_bounds__(512, 4) k_analysis(Params P) {
             int32_t s = (int32_t)((c - kc_lo) * kChunk) + lane;
             const int32_t s_end = (int32_t)min((ce - kc_lo) * kChunk, (int64_t)n);
             c = ce;
+            if (kSample && !walk) continue;
             for (; s - lane < s_end; s += kChunk * kAnaChunks) {
                 int32_t x[kAnaChunks], first[kAnaChunks];
                 bool act[kAnaChunks];

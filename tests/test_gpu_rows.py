@@ -150,3 +150,25 @@ def test_small_call_in_a_users_graph(ctx, L_cells):
             g.replay()
         torch.cuda.synchronize()
         assert np.array_equal(out.cpu().numpy(), oracle.uf_label(x))
+
+
+@pytest.mark.parametrize("n_cells", [1, 3, 13, 14, 100, 300])
+def test_sampled_analysis(n_cells):
+    """Step (ii) left to the library: inputs it walks (few roots), leaves alone
+    (many) and batches of both, from fewer sites than it samples."""
+    c = ccl.ccl_context_create(0)
+    lats = [L.honeycomb(n_cells, p, 5) for p in (0.0, 0.5, 0.8, 0.95, 1.0)] if n_cells > 2 else \
+        [_graph(k, np.full(k, 2), 0.9, k) for k in (1, 2, 31, 33, 384)]
+    for x in lats:
+        assert np.array_equal(gpu_label(c, x), oracle.uf_label(x))
+    so = np.concatenate([[0], np.cumsum([x.n for x in lats])])
+    eo = np.concatenate([[0], np.cumsum([x.nnz for x in lats])])
+    bits = L.pack_bits(np.concatenate([L.unpack_bits(x.open_bits, x.nnz) for x in lats]))
+    dev = [torch.from_numpy(np.concatenate(a)).to(DEV) for a in ([x.row_ptr for x in lats], [x.col_idx for x in lats])]
+    out = torch.full((int(so[-1]),), -1, dtype=torch.int32, device=DEV)
+    assert ccl.ccl_label_batched(c, len(lats), so, eo, *dev, torch.from_numpy(bits.view(np.int32)).to(DEV), out) == ccl.CCL_OK
+    assert ccl.ccl_sync(c) == ccl.CCL_OK
+    got = out.cpu().numpy()
+    for k, x in enumerate(lats):
+        assert np.array_equal(got[so[k]:so[k + 1]], oracle.uf_label(x)), k
+    ccl.ccl_context_destroy(c)
