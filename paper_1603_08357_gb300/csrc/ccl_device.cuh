@@ -620,6 +620,16 @@ __device__ __forceinline__ void jump_and_shortcut(const int32_t *labels, int32_t
         if ((uint32_t)lab[k] - vis_lo < vis_n) lab[k] = __ldcg(labels + lab[k]);
 }
 
+// Whether rows lie in the tile's entries [e0, e1], given the first row's start
+// and the last one's end and that every row is between 0 and kRowRegs long modulo
+// 2^32: row pointers that pass 2^31 on the way come out below where they began.
+__host__ __device__ constexpr bool rows_inside(int32_t first, int32_t last, int32_t e0, int32_t e1) {
+    return first >= e0 && last >= first && last <= e1;
+}
+static_assert(rows_inside(0, 384, 0, 3072) && rows_inside(2688, 3072, 0, 3072) && rows_inside(5, 5, 5, 5), "valid rows");
+static_assert(!rows_inside(INT32_MAX - 60, INT32_MIN + 323, 0, 3072), "wrapped row pointers");
+static_assert(!rows_inside(-1, 383, 0, 3072) && !rows_inside(2689, 3073, 0, 3072), "outside the tile");
+
 // The four chunks of a consumer warp at once, when all their rows exist, are
 // short and staged (the common case). Returns false (having done nothing)
 // otherwise.
@@ -640,7 +650,8 @@ __device__ __forceinline__ bool init_scan_rows(const Params &P, const Stage &S, 
 #pragma unroll
     for (int k = 1; k < kRows; ++k) x |= (uint32_t)a[k] - (uint32_t)a[k - 1] - kChunk * D;
     x |= (uint32_t)last - (uint32_t)first - kRows * kChunk * D;
-    const bool one_degree = __all_sync(kFull, x == 0) && first >= h.e0 && last <= h.e1;
+    const bool inside = rows_inside(first, last, h.e0, h.e1);
+    const bool one_degree = __all_sync(kFull, x == 0) && inside;
     const bool wide = n > (1 << 28);
     bool bad = false;
     if (one_degree && !wide && D == 3) {
@@ -657,7 +668,7 @@ __device__ __forceinline__ bool init_scan_rows(const Params &P, const Stage &S, 
             dm = max(dm, (uint32_t)d[k]);       // (a row running backwards counts as long)
         }
         const int32_t dmax = (int32_t)__reduce_max_sync(kFull, dm);
-        if ((uint32_t)dmax > (uint32_t)kRowRegs || first < h.e0 || last > h.e1) return false;
+        if ((uint32_t)dmax > (uint32_t)kRowRegs || !inside) return false;
         if (wide) scan_rows<kGen, 0, true>(P, S, tc, h, n, s00, lane, a, d, dmax, q, bad);
         else scan_rows<kGen, 0>(P, S, tc, h, n, s00, lane, a, d, dmax, q, bad);
     }
