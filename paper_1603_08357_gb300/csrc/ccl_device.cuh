@@ -1200,6 +1200,25 @@ __device__ __forceinline__ RedWindow red_window(const Params &P, const uint32_t 
     return r;
 }
 
+// A batch with corrupt row pointers may emit more pairs than its rows have
+// entries, and then a band's pairs and their instances are overwritten by
+// another's, each by two stores. When an error is latched, every pair of a window
+// is compared with its instance's size before it is followed, and one that does
+// not fit becomes the pair (0, 0) of the first instance with sites. (A pair of
+// one instance always fits.)
+__device__ __forceinline__ void check_window(const Params &P, const RedWindow &w, int lane) {
+    const int32_t first = find_inst_tile(P, 0);
+    for (int e = lane; e < w.len; e += 32) {
+        const int2 q = w.q[e];
+        const int32_t k = w.qk[e];
+        const uint32_t n = (uint32_t)k < (uint32_t)P.K ? (uint32_t)P.insts[k].n : 0u;
+        if ((uint32_t)q.x < n && (uint32_t)q.y < n) continue;
+        const_cast<int2 *>(w.q)[e] = make_int2(0, 0);
+        const_cast<int32_t *>(w.qk)[e] = first;
+    }
+    __syncwarp();
+}
+
 // A pair needs at most 4n + 8 rounds (its chains and Algorithm 1's loop are
 // bounded by the instance's n <= 32 n_chunks); a lane serves at most len pairs.
 // Past this many rounds a window is abandoned with an error.
@@ -1226,6 +1245,7 @@ __global__ void __launch_bounds__(kRedThreads, !kBatched ? 5 : kFar ? 4 : 3) k_r
     const long long nwarps = (long long)gridDim.x * (kRedThreads / 32);
     long long total;
     const long long nwin = red_windows(P, s_win, s_warp, lane, nwarps, total);
+    const unsigned latched = kBatched ? __ldcg(P.err) : 0u;
     // Few pairs: the clusters are small or tree-like (see `far` below).
     const bool few = !kBatched && kStatic && total <= P.one.n / 4;
 #ifdef CCL_DEVICE_STATS
@@ -1233,6 +1253,7 @@ __global__ void __launch_bounds__(kRedThreads, !kBatched ? 5 : kFar ? 4 : 3) k_r
 #endif
     for (long long w = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w < nwin; w += nwarps) {
         const RedWindow win = red_window<kBatched>(P, s_win, (uint32_t)w);
+        if (kBatched && latched) check_window(P, win, lane);
         const int wlen = win.len;
         const int2 *wq = win.q;
         const int32_t *wqk = win.qk;
@@ -1420,6 +1441,7 @@ __global__ void __launch_bounds__(kRedThreads, kBatched ? 6 : 8) k_reduce_park(P
     const long long nwarps = (long long)gridDim.x * (kRedThreads / 32);
     long long total;
     const long long nwin = red_windows(P, s_win, s_warp, lane, nwarps, total);
+    const unsigned latched = kBatched ? __ldcg(P.err) : 0u;
     const bool eager = P.link_mode != 0;            // link a root to the other end's node, not its root
     // the labels of the lane's last instance
     int lk = -1;
@@ -1461,6 +1483,7 @@ __global__ void __launch_bounds__(kRedThreads, kBatched ? 6 : 8) k_reduce_park(P
     };
     for (long long w = (long long)blockIdx.x * (kRedThreads / 32) + warp; w < nwin; w += nwarps) {
         const RedWindow win = red_window<kBatched>(P, s_win, (uint32_t)w);
+        if (kBatched && latched) check_window(P, win, lane);
         const int round_cap = (int)min(red_round_cap(P, win.len), (long long)INT32_MAX - 3);
         int rounds = 0;
         int cnt = 0;                // pairs set aside; below 32 whenever pairs are added
