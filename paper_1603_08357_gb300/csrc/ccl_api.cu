@@ -718,14 +718,15 @@ void set_bounds(Inst &I, const int32_t *rp, int64_t rp_len, const int32_t *ci, i
     I.bits_hi = bits ? bits + bits_len : bits;
 }
 
-Params base_params(ccl_context *ctx, const TuneChoice &tc) {
+// Parameters of a call of `slots` queue slots (its CSR entries).
+Params base_params(ccl_context *ctx, const TuneChoice &tc, int64_t slots) {
     Params P;
     memset(&P, 0, sizeof(P));
     P.link_mode = tc.link_mode;
     P.band = ctx->d_band;
     P.q = ctx->d_q;
     P.qk = ctx->d_qk;
-    P.q_cap = ctx->q_cap;
+    P.q_cap = slots;            // (the workspace may be larger, q and qk unlike)
     P.gen_thr = kNoGen;
     P.err = ctx->d_err;
     P.counters = ctx->d_counters;
@@ -754,7 +755,7 @@ ccl_status label_single(ccl_context *ctx, int32_t n, int64_t nnz, const int32_t 
     const int64_t chunks = ((int64_t)n + kChunk - 1) / kChunk;
     ccl_status st = ensure_workspace(ctx, nnz, false);
     if (st != CCL_OK) return st;
-    Params P = base_params(ctx, tc);
+    Params P = base_params(ctx, tc, nnz);
     P.K = 1;
     P.n_chunks = chunks;
     P.n_tiles = ((int64_t)n + kTileSites - 1) / kTileSites;
@@ -790,7 +791,7 @@ ccl_status label_dense(ccl_context *ctx, int32_t n, int32_t width, const int32_t
     const int64_t slots = (int64_t)n * width;
     ccl_status st = ensure_workspace(ctx, slots, false);
     if (st != CCL_OK) return st;
-    Params P = base_params(ctx, tc);
+    Params P = base_params(ctx, tc, slots);
     P.K = 1;
     P.n_chunks = ((int64_t)n + kChunk - 1) / kChunk;
     P.n_tiles = ((int64_t)n + kTileSites - 1) / kTileSites;
@@ -838,7 +839,7 @@ ccl_status label_instances(ccl_context *ctx, std::vector<Inst> &table, cudaStrea
     ccl_status st = ensure_workspace(ctx, q, table.size() > 1);
     if (st != CCL_OK) return st;
     const TuneChoice tc = ctx->opt;
-    Params P = base_params(ctx, tc);
+    Params P = base_params(ctx, tc, q);
     P.K = (int32_t)table.size();
     P.n_chunks = chunks;
     P.n_tiles = tiles;
@@ -1143,7 +1144,7 @@ ccl_status label_batched(ccl_context *ctx, int32_t K, const int64_t *site_off, c
     ccl_status st = ensure_workspace(ctx, nnz_tot, K > 1);
     if (st != CCL_OK) return st;
     const TuneChoice tc = force_tc ? *force_tc : choice_for_class(ctx, batch_class(n_tot, nnz_tot, K));
-    Params P = base_params(ctx, tc);
+    Params P = base_params(ctx, tc, nnz_tot);
     P.K = K;
     P.n_chunks = chunks;
     P.n_tiles = tiles;
@@ -1391,7 +1392,7 @@ ccl_status label_host_parts(ccl_context *ctx, int32_t n, int64_t nnz, const int3
     }
     ccl_status st = ensure_workspace(ctx, nnz, false);
     if (st != CCL_OK) return st;
-    Params P = base_params(ctx, tc);
+    Params P = base_params(ctx, tc, nnz);
     P.K = 1;
     P.n_chunks = ((int64_t)n + kChunk - 1) / kChunk;
     P.one.row_ptr = d_rp;
@@ -1602,7 +1603,7 @@ ccl_status ccl_label_batched_host(ccl_context *ctx, int32_t K, const int64_t *si
             I.q_off -= ent_off[k0];
         }
         const bool bat = k1 - k0 > 1;
-        Params P = base_params(ctx, tc);
+        Params P = base_params(ctx, tc, ent_off[k1] - ent_off[k0]);
         P.K = k1 - k0;
         P.n_chunks = c1 - c0;
         if (bat) {

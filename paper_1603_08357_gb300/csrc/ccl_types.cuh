@@ -75,7 +75,7 @@ struct Params {
     BandRec *band;             // [n_bands]
     int2 *q;                   // residual pairs (i, j); slots indexed by global CSR entry
     int32_t *qk;               // instance of each pair (K > 1 only)
-    int64_t q_cap;             // slots of q (and qk)
+    int64_t q_cap;             // slots of q (and qk) this call may use
     uint64_t gen_seed;         // bonds drawn on the device: SplitMix64 state ...
     uint64_t gen_thr;          // ... and threshold (bond open iff output >> 11 < gen_thr)
     const int32_t *nn;         // dense neighbour list (slot k of site i at nn[i + k*n]), or null

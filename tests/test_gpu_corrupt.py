@@ -81,3 +81,21 @@ def test_overfull_rows_in_a_batch(sites, far):
             assert np.array_equal(got[ok.site_off[k]:ok.site_off[k + 1]], oracle.uf_label(x))
     finally:
         ccl.ccl_context_destroy(c)
+
+
+def test_overfull_batch_after_a_larger_single_call():
+    """The workspace's pairs grown by a single instance, the pairs' instance numbers
+    (only batches have them) not: a corrupt batch stays inside both."""
+    c = ccl.ccl_context_create(0)
+    try:
+        big = L.triangle(1200, 0.4, 3)
+        assert np.array_equal(gpu_label(c, big), oracle.uf_label(big))
+        good = _rows(300, np.full(300, 3), 2)
+        b = _batch([_overfull(1024, 4000), good, _overfull(3000, 4000)])
+        dev = [torch.from_numpy(a).to(DEV) for a in (b.row_ptr, b.col_idx, b.open_bits.view(np.int32))]
+        out = torch.zeros(b.n_total, dtype=torch.int32, device=DEV)
+        assert ccl.ccl_label_batched(c, b.k, b.site_off, b.ent_off, *dev, out) == ccl.CCL_OK
+        assert ccl.ccl_sync(c) == ccl.CCL_ERR_INDEX_OUT_OF_RANGE
+        assert np.array_equal(gpu_label(c, big), oracle.uf_label(big))
+    finally:
+        ccl.ccl_context_destroy(c)
