@@ -66,7 +66,7 @@ struct ccl_context {
     int64_t q_cap = 0;
     int32_t *d_qk = nullptr;     // instance of each pair (batched calls)
     int64_t qk_cap = 0;
-    BandRec *d_band = nullptr;   // [kMaxBands]
+    BandRec *d_band = nullptr;   // [1 + kMaxBands]; the first is step (i)'s band ticket
     unsigned *d_err = nullptr;
     unsigned long long *d_counters = nullptr;
     // batched descriptor table (non-graph path)
@@ -117,7 +117,7 @@ struct ccl_context {
 namespace {
 
 constexpr size_t kMaxGraphs = 16;
-constexpr int kCounters = 5;           // statistics (4) and step (i)'s band ticket
+constexpr int kCounters = 4;           // statistics
 constexpr uint64_t kNoGen = ~0ull;     // Params::gen_thr of calls that read open_bits
 constexpr int64_t kProfRing = 4096;
 
@@ -374,7 +374,10 @@ void split_bands(Params &P, int64_t g, bool batched) {
 
 ccl_status launch_init(const Params &P, bool batched, int64_t g, cudaStream_t s) {
     const bool gen = P.gen_thr != kNoGen;
-    if (P.init_bands > g) CCL_CUDA(cudaMemsetAsync(P.ticket, 0, sizeof(unsigned), s));
+    // rounds of bands: the ticket starts at zero, and so do the band records behind
+    // it: a CTA whose wait expires leaves, and a band it had taken but not begun must
+    // not count the pairs of an earlier call
+    if (P.init_bands > g) CCL_CUDA(cudaMemsetAsync(P.ticket, 0, sizeof(BandRec) * (size_t)(1 + P.init_bands), s));
     if (P.dense && P.nn_width <= kRowRegs) {
         if (gen) k_init_dense_tma<true><<<(unsigned)g, kInitThreads, kDenseSmem, s>>>(P);
         else k_init_dense_tma<false><<<(unsigned)g, kInitThreads, kDenseSmem, s>>>(P);
@@ -723,14 +726,14 @@ Params base_params(ccl_context *ctx, const TuneChoice &tc, int64_t slots) {
     Params P;
     memset(&P, 0, sizeof(P));
     P.link_mode = tc.link_mode;
-    P.band = ctx->d_band;
+    P.band = ctx->d_band + 1;
+    P.ticket = (unsigned *)ctx->d_band;
     P.q = ctx->d_q;
     P.qk = ctx->d_qk;
     P.q_cap = slots;            // (the workspace may be larger, q and qk unlike)
     P.gen_thr = kNoGen;
     P.err = ctx->d_err;
     P.counters = ctx->d_counters;
-    P.ticket = (unsigned *)(ctx->d_counters + 4);
     P.iter_cap = ctx->iter_cap;
     return P;
 }
@@ -914,7 +917,7 @@ ccl_status ccl_context_create(ccl_context **out, int device) {
     ctx->l2_bytes = l2;
     if (e == cudaSuccess) e = cudaMalloc(&ctx->d_err, sizeof(unsigned));
     if (e == cudaSuccess) e = cudaMemset(ctx->d_err, 0, sizeof(unsigned));
-    if (e == cudaSuccess) e = cudaMalloc(&ctx->d_band, kMaxBands * sizeof(BandRec));
+    if (e == cudaSuccess) e = cudaMalloc(&ctx->d_band, (1 + kMaxBands) * sizeof(BandRec));
     if (e == cudaSuccess) e = cudaMalloc(&ctx->d_counters, kCounters * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMemset(ctx->d_counters, 0, kCounters * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&ctx->cap_stream, cudaStreamNonBlocking);

@@ -82,7 +82,8 @@ struct Params {
     int64_t nn_width;          // slots per site of the dense list
     int32_t init_bands;        // bands of a step (i) launch: rounds of one per CTA (the last may be short) ...
     int32_t round_per[kRounds];    // ... and the tiles of a band of each round
-    unsigned *ticket;          // bands taken beyond the first of every CTA (cleared before a launch in rounds)
+    unsigned *ticket;          // bands taken beyond the first of every CTA, just before band[0] (both cleared
+                               // before a launch in rounds)
     int64_t tile_off;          // step (i) on part of the tiles: its first tile ...
     int32_t band_off;          // ... and its first band record
     int32_t more_pairs;        // 1: the pairs of this step (iii) add to counters[0], 0: they replace it

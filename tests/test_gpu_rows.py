@@ -2,6 +2,8 @@
 degree (3, 4 and 6 have their own code), mixed rows, rows past the register
 path, chunk groups that end at 128 sites, and every alignment of an instance's
 entries inside a batch. Labels are integers: equality, no tolerance."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -172,3 +174,42 @@ def test_sampled_analysis(n_cells):
     for k, x in enumerate(lats):
         assert np.array_equal(got[so[k]:so[k + 1]], oracle.uf_label(x)), k
     ccl.ccl_context_destroy(c)
+
+
+def test_rounds_start_from_empty_band_records():
+    """A launch in rounds clears the ticket and every band's record with it: a band
+    that a CTA took but never began (it gave up waiting) counts no pairs. Read off
+    the captured call, whose graph is not run."""
+    class Memset(ctypes.Structure):
+        _fields_ = [("dst", ctypes.c_uint64), ("pitch", ctypes.c_size_t), ("value", ctypes.c_uint),
+                    ("element", ctypes.c_uint), ("width", ctypes.c_size_t), ("height", ctypes.c_size_t)]
+
+    ctx = ccl.ccl_context_create(0)
+    n = 12_000_000                              # isolated sites, enough tiles for the rounds
+    so, eo = np.array([0, n, 2 * n], np.int64), np.zeros(3, np.int64)
+    rp = torch.zeros(2 * n + 2, dtype=torch.int32, device=DEV)
+    out = torch.empty(2 * n, dtype=torch.int32, device=DEV)
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    assert ccl.ccl_label_batched(ctx, 2, so, eo, rp, None, None, out, s) == ccl.CCL_OK
+    assert ccl.ccl_sync(ctx, s) == ccl.CCL_OK
+    drv = ctypes.CDLL("libcuda.so.1")
+    h, graph, count = ctypes.c_void_p(s.cuda_stream), ctypes.c_void_p(), ctypes.c_size_t()
+    assert drv.cuStreamBeginCapture_v2(h, 2) == 0
+    assert ccl.ccl_label_batched(ctx, 2, so, eo, rp, None, None, out, s) == ccl.CCL_OK
+    assert drv.cuStreamEndCapture(h, ctypes.byref(graph)) == 0
+    assert drv.cuGraphGetNodes(graph, None, ctypes.byref(count)) == 0
+    nodes, kind, cleared = (ctypes.c_void_p * count.value)(), ctypes.c_int(), []
+    assert drv.cuGraphGetNodes(graph, nodes, ctypes.byref(count)) == 0
+    for node in nodes:
+        assert drv.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
+        if kind.value == 2:                     # a memset
+            m = Memset()
+            assert drv.cuGraphMemsetNodeGetParams(ctypes.c_void_p(node), ctypes.byref(m)) == 0
+            assert m.value == 0
+            cleared.append(m.element * m.width * m.height)
+    assert drv.cuGraphDestroy(graph) == 0
+    # a ticket and at least eleven rounds of a 16-byte record per SM
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert len(cleared) == 1 and cleared[0] >= 16 * (1 + 11 * sms)
+    ccl.ccl_context_destroy(ctx)
