@@ -137,10 +137,12 @@ static_assert(offsetof(StageHdr, t_rb0) % 16 == 0 && offsetof(StageHdr, t_nbits)
 struct __align__(16) Stage {
     StageHdr h;
     int32_t rp[kRpBuf];
-    int32_t ci[kColBuf];
+    int32_t ci[kColBuf + kRowRegs];     // (mixed rows read up to kRowRegs - 1 entries past a row's end, masked)
     uint32_t bw[kBitBuf];
 };
 
+static_assert(offsetof(Stage, rp) % 16 == 0 && offsetof(Stage, ci) % 16 == 0 && offsetof(Stage, bw) % 16 == 0,
+              "destinations of bulk copies");
 constexpr size_t kInitSmem = 64 + sizeof(Stage) * kStages;
 
 }  // namespace ccl

@@ -213,3 +213,28 @@ def test_rounds_start_from_empty_band_records():
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     assert len(cleared) == 1 and cleared[0] >= 16 * (1 + 11 * sms)
     ccl.ccl_context_destroy(ctx)
+
+
+@pytest.mark.parametrize("shift", [0, 1, 2, 3])
+@pytest.mark.parametrize("mixed", [False, True])
+def test_full_stage(shift, mixed):
+    """Tiles whose 7168 entries fill a stage: rows of seven, or mixed rows whose last
+    ones are empty (a row's scan reads past the last entry there), with the
+    columns `shift` entries off their alignment (an instance of that many before)."""
+    n = 3 * 1024
+    deg = np.full(n, 7)
+    if mixed:
+        rng = np.random.default_rng(shift)
+        deg = np.concatenate([np.concatenate([rng.permutation([6, 8] * 448), np.full(112, 8), np.zeros(16, np.int64)])
+                              for _ in range(3)])
+        assert deg.size == n and deg[:1024].sum() == 7168
+    lats = [_graph(shift + 1, np.r_[0, np.ones(shift, np.int64)], 0.5, 1), _graph(n, deg, 0.4, 9 + shift)]
+    so, eo = (np.concatenate([[0], np.cumsum([getattr(x, f) for x in lats])]) for f in ("n", "nnz"))
+    bits = L.pack_bits(np.concatenate([L.unpack_bits(x.open_bits, x.nnz) for x in lats]))
+    rp, ci = (np.concatenate(a).astype(np.int32) for a in ([x.row_ptr for x in lats], [x.col_idx for x in lats]))
+    c = ccl.ccl_context_create(0)
+    got = gpu_label_batched(c, L.Batch(so, eo, rp, ci, bits, [{"kind": "random"}] * 2))
+    for k, x in enumerate(lats):
+        assert np.array_equal(got[so[k]:so[k + 1]], oracle.uf_label(x)), k
+    assert np.array_equal(gpu_label(c, lats[1]), oracle.uf_label(lats[1]))
+    ccl.ccl_context_destroy(c)
