@@ -27,7 +27,7 @@ namespace {
 struct TuneChoice {
     int threads = 256;
     int ctas_per_sm = 0;
-    int pre_analysis = -1;  // step (ii): 1 run, 0 skip; -1 (never set) the library's choice: skip
+    int pre_analysis = -1;  // step (ii): 1 run, 0 skip; -1 by sample on the device (k_analysis)
     int link_mode = 0;
     int refill = 1;         // step (iii): 1 static per-lane pairs, 0 in-order hand-out
     int ana_seq = 1;        // steps (ii)/(iv): 1 contiguous ranges per warp, 0 interleaved
@@ -1003,7 +1003,7 @@ void ccl_context_destroy(ccl_context *ctx) {
 ccl_status ccl_set_option(ccl_context *ctx, int option, int64_t value) {
     if (!ctx) return CCL_ERR_INVALID_ARGUMENT;
     switch (option) {
-        case CCL_OPT_PRE_ANALYSIS: ctx->opt.pre_analysis = value ? 1 : 0; break;
+        case CCL_OPT_PRE_ANALYSIS: ctx->opt.pre_analysis = value == -1 ? -1 : value ? 1 : 0; break;
         case CCL_OPT_BLOCK_THREADS:
             if (value < 64 || value > 512 || value % 32) return CCL_ERR_INVALID_ARGUMENT;
             ctx->opt.threads = (int)value;
@@ -1051,7 +1051,7 @@ ccl_status ccl_set_option(ccl_context *ctx, int option, int64_t value) {
 ccl_status ccl_get_option(ccl_context *ctx, int option, int64_t *value) {
     if (!ctx || !value) return CCL_ERR_INVALID_ARGUMENT;
     switch (option) {
-        case CCL_OPT_PRE_ANALYSIS: *value = ctx->opt.pre_analysis != 0; break;
+        case CCL_OPT_PRE_ANALYSIS: *value = ctx->opt.pre_analysis; break;
         case CCL_OPT_BLOCK_THREADS: *value = ctx->opt.threads; break;
         case CCL_OPT_USE_GRAPHS: *value = ctx->use_graphs; break;
         case CCL_OPT_PROFILE: *value = ctx->profile; break;

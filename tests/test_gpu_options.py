@@ -1,0 +1,38 @@
+"""Options and tuning where the library has a choice of its own: it can be read,
+written back and had again, and tuning on one input does not take it away."""
+import numpy as np
+import pytest
+import torch
+
+import lattices as L
+import oracle
+import paper_1603_08357_gb300 as ccl
+from ccl_testutil import DEV, gpu_label, to_dev
+
+pytestmark = pytest.mark.gpu
+
+OPTIONS = [getattr(ccl, f"CCL_OPT_{n}") for n in (
+    "PRE_ANALYSIS", "BLOCK_THREADS", "CTAS_PER_SM", "LINK_MODE", "REFILL", "ANALYSIS_ORDER", "ITER_CAP",
+    "REDUCE_WINDOW", "ANALYSIS_GROUP", "ANALYSIS_PARK")]
+
+
+@pytest.fixture
+def fresh():
+    c = ccl.ccl_context_create(0)
+    yield c
+    ccl.ccl_context_destroy(c)
+
+
+def test_step_ii_by_sample_can_be_read_and_set(fresh):
+    opt = ccl.CCL_OPT_PRE_ANALYSIS
+    assert ccl.ccl_get_option(fresh, opt) == -1
+    for v, reads in ((1, 1), (0, 0), (-1, -1), (5, 1), (-1, -1)):
+        assert ccl.ccl_set_option(fresh, opt, v) == ccl.CCL_OK
+        assert ccl.ccl_get_option(fresh, opt) == reads
+
+
+@pytest.mark.parametrize("opt", OPTIONS)
+def test_writing_back_what_was_read_changes_nothing(fresh, opt):
+    v = ccl.ccl_get_option(fresh, opt)
+    assert ccl.ccl_set_option(fresh, opt, v) == ccl.CCL_OK
+    assert ccl.ccl_get_option(fresh, opt) == v
