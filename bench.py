@@ -497,7 +497,7 @@ def run_ours(args, rank, world, local):
                     "h2d_bytes_per_step": h2d,
                     "d2h_bytes_per_step": 4 * lat.n, "ms_per_step": e_ms,
                     "entry": entry},
-            "gpu_launches": args.steps * (4 if opts["pre_analysis"] else 3),
+            "gpu_launches": args.steps * launches_per_step(opts),
             "clocks": clk,
             "parity_last_step": ok_sample,      # from the CPU-baseline leg (None without it)
         }
@@ -511,6 +511,12 @@ def _phases(st) -> dict:
     """The request loop's latency by phase (p50 / p99 in ms)."""
     names = ("admit", "upload", "wait_launch", "gpu_and_return")
     return {n: [round(st.phase_p50_ms[k], 3), round(st.phase_p99_ms[k], 3)] for k, n in enumerate(names)}
+
+
+def launches_per_step(settings: dict) -> int:
+    """Labelling kernels of a call: steps (i), (iii), (iv), and (ii) when it ran or
+    was decided by sample (-1, a launch too)."""
+    return 3 if settings["pre_analysis"] == 0 else 4
 
 
 def _settings(stats) -> dict:
@@ -730,7 +736,7 @@ def run_batched(args, rank, world, local):
                     "step_ms": [round(x, 2) for x in e_step_ms],
                     "entry": "ccl_label_batched_host (pinned host allocations)",
                     "labels_identical": e2e_same},
-            "gpu_launches": args.steps * (4 if opts["pre_analysis"] else 3),
+            "gpu_launches": args.steps * launches_per_step(opts),
             "clocks": clk,
             "parity_all_instances": ok,       # every label of the last timed step vs the oracle
         }

@@ -354,7 +354,8 @@ typedef struct {
        operations of the merge loops, warp iterations of the reduction */
     int64_t chase_loads, merge_atomics, reduce_iterations;
     /* the settings the last call ran with (tuned, set, or chosen by size):
-       step (ii) on, step (iii) link mode and hand-out, step (ii)/(iv) order,
+       step (ii) (1 ran, 0 not, -1 by sample: a launch in which the instances
+       that call for it are walked), step (iii) link mode and hand-out, step (ii)/(iv) order,
        step (iii) window, step (ii)/(iv) super-chunk run length (0: one range
        per warp), step (ii)/(iv) parking -- see ccl_option */
     int32_t pre_analysis, link_mode, refill, analysis_order, reduce_window, analysis_group, analysis_park;

@@ -436,7 +436,7 @@ constexpr int kSampleGroup = 64;     // groups per run of the sampling pass beyo
 
 // Records in the context's statistics the settings a call runs with.
 void note_settings(ccl_context *ctx, const TuneChoice &tc, const Params &P) {
-    ctx->last.pre_analysis = resolve_pre(tc) ? 1 : 0;
+    ctx->last.pre_analysis = tc.pre_analysis;
     ctx->last.link_mode = tc.link_mode;
     ctx->last.refill = tc.refill;
     ctx->last.analysis_order = tc.ana_seq;

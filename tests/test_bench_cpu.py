@@ -103,3 +103,7 @@ def test_threaded_batched_oracle_equals_serial():
     b = L.make_batch(L.batched_mix_specs(40, seed=9))
     got, threads = oracle.uf_label_batched_threads(b, 3)
     assert threads == 3 and np.array_equal(got, oracle.uf_label_batched(b))
+
+
+def test_launch_count_follows_the_reported_step_ii():
+    assert [bench.launches_per_step({"pre_analysis": v}) for v in (0, 1, -1)] == [3, 4, 4]

@@ -36,3 +36,13 @@ def test_writing_back_what_was_read_changes_nothing(fresh, opt):
     v = ccl.ccl_get_option(fresh, opt)
     assert ccl.ccl_set_option(fresh, opt, v) == ccl.CCL_OK
     assert ccl.ccl_get_option(fresh, opt) == v
+
+
+def test_statistics_tell_how_step_ii_ran(fresh):
+    """By sample (-1), also where it walks (honeycomb at 1.5 p_c, long chains)."""
+    lats = [L.honeycomb(750, p, 3) for p in (L.PC_HONEYCOMB, 1.5 * L.PC_HONEYCOMB)]
+    for setting in (-1, 0, 1, -1):
+        assert ccl.ccl_set_option(fresh, ccl.CCL_OPT_PRE_ANALYSIS, setting) == ccl.CCL_OK
+        for lat in lats:
+            assert np.array_equal(gpu_label(fresh, lat), oracle.uf_label(lat))
+            assert ccl.ccl_get_stats(fresh).pre_analysis == setting
