@@ -379,7 +379,9 @@ CCL_API ccl_status ccl_get_step_times(ccl_context *ctx, float *ms, int32_t n);
  * refill mode, analysis order)
  * and keeps the fastest for instances of this size class (log2 of the site
  * count, mean degree rounded); the choice also becomes the context's
- * options (ccl_get_option reports it). Every candidate writes the same labels,
+ * options (ccl_get_option reports it), except what follows the size of a call
+ * or its data (CCL_OPT_PRE_ANALYSIS, the window, run length and parking): those
+ * stay as they were for other size classes. Every candidate writes the same labels,
  * so `labels` holds the correct result afterwards. best_ms (optional)
  * receives the best time.
  * If the environment variable CCL_TUNE_CACHE names a file, ccl_autotune
@@ -393,12 +395,12 @@ CCL_API ccl_status ccl_autotune(ccl_context *ctx, int32_t n_sites, int64_t nnz, 
 
 /*
  * ccl_autotune_batched -- ccl_autotune for ccl_label_batched: times one
- * batched call of these K instances under each candidate setting (step (ii)
- * on/off, link mode, refill mode, analysis order) and keeps the fastest for
+ * batched call of these K instances under each candidate setting (step (ii) by
+ * sample, on or off, link mode, refill mode, analysis order) and keeps the fastest for
  * batches of this mean instance size and degree (a class of its own, apart
  * from single instances). Arguments as ccl_label_batched; `labels` holds the
  * correct result afterwards; best_ms (optional) receives the best time.
- * Synchronous; each candidate runs three times, so budget ~50 calls.
+ * Synchronous; each candidate runs three times, so budget ~100 calls.
  */
 CCL_API ccl_status ccl_autotune_batched(ccl_context *ctx, int32_t n_inst, const int64_t *site_off,
                                         const int64_t *ent_off, const int32_t *row_ptr,

@@ -956,7 +956,7 @@ ccl_status ccl_context_create(ccl_context **out, int device) {
                 const int nf = sscanf(line, "%lld %d %d %d %d %d %d %d %d %d", &cls, &a, &b, &c, &d, &r, &q, &w, &g, &k);
                 if (nf != 7 && nf != 10) continue;
                 TuneChoice t;
-                t.threads = a; t.ctas_per_sm = b < 0 ? 0 : b; t.pre_analysis = c > 0 ? 1 : 0;
+                t.threads = a; t.ctas_per_sm = b < 0 ? 0 : b; t.pre_analysis = c == -1 ? -1 : c > 0 ? 1 : 0;
                 t.link_mode = d ? 1 : 0; t.refill = r ? 1 : 0; t.ana_seq = q ? 1 : 0;
                 t.red_window = (w >= 64 && w <= 65536) ? w : 0;
                 t.ana_group = g >= 0 ? g : -1;
@@ -1179,7 +1179,7 @@ ccl_status ccl_autotune_batched(ccl_context *ctx, int32_t K, const int64_t *site
     DeviceGuard guard(ctx->device);
     cudaStream_t s = (cudaStream_t)stream;
     std::vector<TuneChoice> cands;
-    for (int pre = 0; pre < 2; ++pre)
+    for (int pre = -1; pre < 2; ++pre)      // (by sample: the instances of a batch differ)
         for (int lm = 0; lm < 2; ++lm)
             for (int rf = 0; rf < 2; ++rf)
                 for (int sq = 0; sq < 2; ++sq) {
@@ -1728,8 +1728,12 @@ ccl_status ccl_autotune(ccl_context *ctx, int32_t n, int64_t nnz, const int32_t 
     if (st != CCL_OK) return st;
     ctx->tune_table[size_class(n, nnz)] = best;
     // also the default for other size classes, except the settings that
-    // follow the size of the call
+    // follow the size of the call and, for step (ii), the data: a choice made on
+    // an input near p_c leaves the long chains of one far above it to step (iii)
+    // (honeycomb 362^2 at 1.5 p_c 109 us without step (ii), 44 by sample)
+    const int pre = ctx->opt.pre_analysis;
     ctx->opt = best;
+    ctx->opt.pre_analysis = pre;
     ctx->opt.red_window = 0;
     ctx->opt.ana_group = -1;
     ctx->opt.ana_park = -1;

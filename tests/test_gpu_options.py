@@ -46,3 +46,32 @@ def test_statistics_tell_how_step_ii_ran(fresh):
         for lat in lats:
             assert np.array_equal(gpu_label(fresh, lat), oracle.uf_label(lat))
             assert ccl.ccl_get_stats(fresh).pre_analysis == setting
+
+
+def _supercritical():
+    return L.honeycomb(750, 1.5 * L.PC_HONEYCOMB, 3)       # 1,125,000 sites of degree 3: size class 20 * 1024 + 3
+
+
+def test_tuning_at_the_threshold_keeps_the_sample_for_other_sizes(fresh):
+    lat = L.triangle(256, L.PC_TRIANGLE, 3)
+    rp, ci, bits = to_dev(lat)
+    out = torch.empty(lat.n, dtype=torch.int32, device=DEV)
+    st, _ = ccl.ccl_autotune(fresh, lat.n, lat.nnz, rp, ci, bits, out)
+    assert st == ccl.CCL_OK
+    assert ccl.ccl_get_option(fresh, ccl.CCL_OPT_PRE_ANALYSIS) == -1
+    other = _supercritical()
+    assert np.array_equal(gpu_label(fresh, other), oracle.uf_label(other))
+    assert ccl.ccl_get_stats(fresh).pre_analysis == -1
+
+
+def test_tune_cache_keeps_the_sample(tmp_path, monkeypatch):
+    path = tmp_path / "tune.txt"
+    path.write_text(f"{20 * 1024 + 3} 256 0 -1 0 1 1 0 -1 -1\n")
+    monkeypatch.setenv("CCL_TUNE_CACHE", str(path))
+    c = ccl.ccl_context_create(0)
+    try:
+        other = _supercritical()
+        assert np.array_equal(gpu_label(c, other), oracle.uf_label(other))
+        assert ccl.ccl_get_stats(c).pre_analysis == -1
+    finally:
+        ccl.ccl_context_destroy(c)
