@@ -97,11 +97,11 @@ typedef enum {
     CCL_OPT_PROFILE = 3,       /* 1: record CUDA events between the steps (ccl_get_step_times);
                                   setting it restarts the averaging */
     CCL_OPT_CTAS_PER_SM = 4,   /* persistent CTAs per SM of the analysis kernel; 0 (default) = occupancy maximum */
-    CCL_OPT_LINK_MODE = 5,     /* step (iii): 0 (default) a root is linked under the other tree's
-                                  root, as in Algorithm 1; 1 under the node the other chain has
-                                  reached (same atomicMin loop, shorter walks on trees). With 0
-                                  a large instance of few residual pairs (a quarter of the sites
-                                  at most) uses 1 where the ends of its pairs lie far apart */
+    CCL_OPT_LINK_MODE = 5,     /* step (iii): 0 a root is linked under the other tree's root, as in
+                                  Algorithm 1; 1 under the node the other chain has reached
+                                  (same atomicMin loop, shorter walks on trees); -1 (default) as
+                                  0, but a large instance of few residual pairs (a quarter of the
+                                  sites at most) uses 1 where the ends of its pairs lie far apart */
     CCL_OPT_REFILL = 6,        /* step (iii): 1 (default) each thread serves a fixed stride of the
                                   residual pairs (and, when the call's labels take at most three
                                   eighths of L2, pairs with long chains are set aside and finished
@@ -355,9 +355,10 @@ typedef struct {
     int64_t chase_loads, merge_atomics, reduce_iterations;
     /* the settings the last call ran with (tuned, set, or chosen by size):
        step (ii) (1 ran, 0 not, -1 by sample: a launch in which the instances
-       that call for it are walked), step (iii) link mode and hand-out, step (ii)/(iv) order,
-       step (iii) window, step (ii)/(iv) super-chunk run length (0: one range
-       per warp), step (ii)/(iv) parking -- see ccl_option */
+       that call for it are walked), step (iii) link mode (-1 where it went by
+       window) and hand-out, step (ii)/(iv) order, step (iii) window, step
+       (ii)/(iv) super-chunk run length (0: one range per warp), step (ii)/(iv)
+       parking -- see ccl_option */
     int32_t pre_analysis, link_mode, refill, analysis_order, reduce_window, analysis_group, analysis_park;
 } ccl_run_stats;
 

@@ -28,7 +28,7 @@ struct TuneChoice {
     int threads = 256;
     int ctas_per_sm = 0;
     int pre_analysis = -1;  // step (ii): 1 run, 0 skip; -1 by sample on the device (k_analysis)
-    int link_mode = 0;
+    int link_mode = -1;     // step (iii): 0 root to root, 1 root to the other chain's node; -1 by window (k_reduce)
     int refill = 1;         // step (iii): 1 static per-lane pairs, 0 in-order hand-out
     int ana_seq = 1;        // steps (ii)/(iv): 1 contiguous ranges per warp, 0 interleaved
     int red_window = 0;     // step (iii): most pairs per warp window; 0 by size (see resolve_tail)
@@ -434,10 +434,17 @@ bool resolve_park(const TuneChoice &tc, const Params &P) {
 bool resolve_pre(const TuneChoice &tc) { return tc.pre_analysis > 0; }
 constexpr int kSampleGroup = 64;     // groups per run of the sampling pass beyond L2
 
+// Step (iii) by short walks (k_reduce_park) for labels of at most three eighths of
+// L2, else (and where the hand-out or the iteration cap is asked for) the slots.
+bool walks_short(const ccl_context *ctx, const TuneChoice &tc, const Params &P) {
+    return tc.refill && P.iter_cap == 0 && 4 * kChunk * P.n_chunks <= ctx->l2_bytes * 3 / 8;
+}
+
 // Records in the context's statistics the settings a call runs with.
 void note_settings(ccl_context *ctx, const TuneChoice &tc, const Params &P) {
     ctx->last.pre_analysis = tc.pre_analysis;
-    ctx->last.link_mode = tc.link_mode;
+    // (by window only in the slots of a single instance, k_reduce<false, true, ..>)
+    ctx->last.link_mode = tc.link_mode >= 0 ? tc.link_mode : P.K == 1 && tc.refill && !walks_short(ctx, tc, P) ? -1 : 0;
     ctx->last.refill = tc.refill;
     ctx->last.analysis_order = tc.ana_seq;
     ctx->last.reduce_window = P.red_window;
@@ -474,9 +481,7 @@ ccl_status enqueue_tail(ccl_context *ctx, const Params &P0, bool batched, const 
     resolve_tail(ctx, tc, P);
     note_settings(ctx, tc, P);
     const int T = tc.threads;
-    // short walks for labels of at most three eighths of L2, else (and where
-    // the hand-out or the iteration cap is asked for) the slots
-    const bool short_walk = tc.refill && P.iter_cap == 0 && 4 * kChunk * P.n_chunks <= ctx->l2_bytes * 3 / 8;
+    const bool short_walk = walks_short(ctx, tc, P);
     // Programmatic launches for calls of at most one step (i) CTA per SM: the
     // launch latencies between the steps overlap. Not for larger ones: the next
     // kernel would start on SMs still set to step (i)'s shared memory and run
@@ -957,7 +962,7 @@ ccl_status ccl_context_create(ccl_context **out, int device) {
                 if (nf != 7 && nf != 10) continue;
                 TuneChoice t;
                 t.threads = a; t.ctas_per_sm = b < 0 ? 0 : b; t.pre_analysis = c == -1 ? -1 : c > 0 ? 1 : 0;
-                t.link_mode = d ? 1 : 0; t.refill = r ? 1 : 0; t.ana_seq = q ? 1 : 0;
+                t.link_mode = d > 0 ? 1 : -1; t.refill = r ? 1 : 0; t.ana_seq = q ? 1 : 0;
                 t.red_window = (w >= 64 && w <= 65536) ? w : 0;
                 t.ana_group = g >= 0 ? g : -1;
                 t.ana_park = k >= 0 ? (k ? 1 : 0) : -1;
@@ -1018,7 +1023,7 @@ ccl_status ccl_set_option(ccl_context *ctx, int option, int64_t value) {
             if (value < 0 || value > 64) return CCL_ERR_INVALID_ARGUMENT;
             ctx->opt.ctas_per_sm = (int)value;
             break;
-        case CCL_OPT_LINK_MODE: ctx->opt.link_mode = value ? 1 : 0; break;
+        case CCL_OPT_LINK_MODE: ctx->opt.link_mode = value == -1 ? -1 : value ? 1 : 0; break;
         case CCL_OPT_REFILL: ctx->opt.refill = value ? 1 : 0; break;
         case CCL_OPT_ANALYSIS_ORDER: ctx->opt.ana_seq = value ? 1 : 0; break;
         case CCL_OPT_REDUCE_WINDOW:
@@ -1180,7 +1185,7 @@ ccl_status ccl_autotune_batched(ccl_context *ctx, int32_t K, const int64_t *site
     cudaStream_t s = (cudaStream_t)stream;
     std::vector<TuneChoice> cands;
     for (int pre = -1; pre < 2; ++pre)      // (by sample: the instances of a batch differ)
-        for (int lm = 0; lm < 2; ++lm)
+        for (int lm : {-1, 1})
             for (int rf = 0; rf < 2; ++rf)
                 for (int sq = 0; sq < 2; ++sq) {
                     TuneChoice tc;
@@ -1712,7 +1717,7 @@ ccl_status ccl_autotune(ccl_context *ctx, int32_t n, int64_t nnz, const int32_t 
     std::vector<TuneChoice> cands;
     for (int T : {128, 256, 512})
         for (int pre = 0; pre < 2; ++pre)
-            for (int lm = 0; lm < 2; ++lm)
+            for (int lm : {-1, 1})
                 for (int rf = 0; rf < 2; ++rf)
                     for (int sq = 0; sq < 2; ++sq) {
                         TuneChoice tc;
@@ -1741,7 +1746,7 @@ ccl_status ccl_autotune(ccl_context *ctx, int32_t n, int64_t nnz, const int32_t 
         if (FILE *f = fopen(env, "w")) {
             for (auto &kv : ctx->tune_table)
                 fprintf(f, "%lld %d %d %d %d %d %d %d %d %d\n", (long long)kv.first, kv.second.threads,
-                        kv.second.ctas_per_sm, kv.second.pre_analysis, kv.second.link_mode, kv.second.refill,
+                        kv.second.ctas_per_sm, kv.second.pre_analysis, kv.second.link_mode > 0 ? 1 : 0, kv.second.refill,
                         kv.second.ana_seq, kv.second.red_window, kv.second.ana_group, kv.second.ana_park);
             fclose(f);
         }

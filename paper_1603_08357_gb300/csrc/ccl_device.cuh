@@ -1247,7 +1247,7 @@ __global__ void __launch_bounds__(kRedThreads, !kBatched ? 5 : kFar ? 4 : 3) k_r
     const long long nwin = red_windows(P, s_win, s_warp, lane, nwarps, total);
     const unsigned latched = kBatched ? __ldcg(P.err) : 0u;
     // Few pairs: the clusters are small or tree-like (see `far` below).
-    const bool few = !kBatched && kStatic && total <= P.one.n / 4;
+    const bool few = !kBatched && kStatic && P.link_mode < 0 && total <= P.one.n / 4;
 #ifdef CCL_DEVICE_STATS
     unsigned long long st_hops = 0, st_atom = 0, st_iter = 0;
 #endif
@@ -1402,7 +1402,7 @@ __global__ void __launch_bounds__(kRedThreads, !kBatched ? 5 : kFar ? 4 : 3) k_r
             }
         };
         if (far) drain(kRedNextLink1);
-        else drain(P.link_mode ? kRedNextLink1 : kRedNextLink0);
+        else drain(P.link_mode > 0 ? kRedNextLink1 : kRedNextLink0);
     }
 #ifdef CCL_DEVICE_STATS
     if (st_hops) atomicAdd(P.counters + 1, st_hops);
@@ -1442,7 +1442,7 @@ __global__ void __launch_bounds__(kRedThreads, kBatched ? 6 : 8) k_reduce_park(P
     long long total;
     const long long nwin = red_windows(P, s_win, s_warp, lane, nwarps, total);
     const unsigned latched = kBatched ? __ldcg(P.err) : 0u;
-    const bool eager = P.link_mode != 0;            // link a root to the other end's node, not its root
+    const bool eager = P.link_mode > 0;            // link a root to the other end's node, not its root
     // the labels of the lane's last instance
     int lk = -1;
     int32_t *llab = P.one.labels;

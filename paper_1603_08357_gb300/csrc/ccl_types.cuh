@@ -67,7 +67,7 @@ struct Params {
     int32_t *lab_base;         // K > 1: the lowest labels, when all lie within 2^32 labels of them; else null
     Inst one;                  // the instance when K == 1
     int32_t K;
-    int32_t link_mode;         // step (iii): 0 root to root, 1 root to the other chain's node
+    int32_t link_mode;         // step (iii): 0 root to root, 1 root to the other chain's node, -1 by window
     int64_t n_chunks;          // over all instances
     int64_t n_tiles;           // over all instances
     int32_t n_bands;           // CTAs of step (i)

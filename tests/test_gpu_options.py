@@ -75,3 +75,17 @@ def test_tune_cache_keeps_the_sample(tmp_path, monkeypatch):
         assert ccl.ccl_get_stats(c).pre_analysis == -1
     finally:
         ccl.ccl_context_destroy(c)
+
+
+def test_link_mode_as_set_or_by_window(fresh):
+    """0 and 1 as set; -1 (the default) by window in the slots of one large instance,
+    0 elsewhere."""
+    small, large = L.square(200, 0.5, 4), L.square(3700, 0.5, 4)
+    opt = ccl.CCL_OPT_LINK_MODE
+    assert ccl.ccl_get_option(fresh, opt) == -1
+    for setting in (-1, 0, 1, -1):
+        assert ccl.ccl_set_option(fresh, opt, setting) == ccl.CCL_OK
+        assert ccl.ccl_get_option(fresh, opt) == setting
+        for lat, by_window in ((small, 0), (large, -1)):
+            assert np.array_equal(gpu_label(fresh, lat), oracle.uf_label(lat))
+            assert ccl.ccl_get_stats(fresh).link_mode == (setting if setting >= 0 else by_window)
