@@ -310,7 +310,8 @@ CCL_API ccl_status ccl_validate(ccl_context *ctx, int32_t n_sites, int64_t nnz, 
  *   seq         DEVICE int32[n], output; must not alias labels
  *   n_clusters  DEVICE int32, output: C
  *   sizes       DEVICE int32[n] or NULL: sizes[c] = sites of cluster c (c < C)
- * Asynchronous on `stream`; labels that are not canonical give undefined ids.
+ * Uses 4 bytes of context scratch per 8192 sites (grown with cudaMalloc when
+ * needed). Asynchronous on `stream`; labels that are not canonical give undefined ids.
  */
 CCL_API ccl_status ccl_relabel(ccl_context *ctx, int32_t n, const int32_t *labels, int32_t *seq,
                                int32_t *n_clusters, int32_t *sizes, void *stream);

@@ -1284,14 +1284,12 @@ ccl_status ccl_relabel(ccl_context *ctx, int32_t n, const int32_t *labels, int32
     }
     if (!labels || !seq || labels == seq) return CCL_ERR_INVALID_ARGUMENT;
     const int64_t nb = ((int64_t)n + kRelBlock - 1) / kRelBlock;
-    // scratch: a count per block, then a bit per site
-    ccl_status st = ensure_aux(ctx, nb * (int64_t)sizeof(int32_t) * (1 + kRelThreads));
+    ccl_status st = ensure_aux(ctx, nb * (int64_t)sizeof(int32_t));       // a count per block
     if (st != CCL_OK) return st;
     int32_t *cnt = (int32_t *)ctx->d_aux;
-    uint32_t *roots = (uint32_t *)(cnt + nb);
-    k_root_counts<<<(unsigned)nb, kRelThreads, 0, s>>>(n, labels, cnt, roots);
+    k_root_counts<<<(unsigned)nb, kRelThreads, 0, s>>>(n, labels, cnt, seq);
     k_scan_counts<<<1, 1024, 0, s>>>((int32_t)nb, cnt, n_clusters);
-    k_root_ids<<<(unsigned)nb, kRelThreads, 0, s>>>(roots, cnt, seq, sizes);
+    k_root_ids<<<(unsigned)nb, kRelThreads, 0, s>>>(n, cnt, seq, sizes);
     k_site_ids<<<(unsigned)run_grid(ctx, n), 256, 0, s>>>(n, labels, seq, sizes);
     CCL_CUDA(cudaGetLastError());
     return CCL_OK;

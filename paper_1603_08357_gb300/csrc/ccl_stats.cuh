@@ -20,10 +20,12 @@ constexpr int kRelBlock = kRelThreads * kRelPerThread;   // sites per relabel bl
 
 // number of roots (label[i] == i) in each block of kRelBlock sites, and a bit
 // per site, set for roots. A warp takes 1024 consecutive sites and keeps the 32
-// ballots one per lane.
+// ballots one per lane. The block's words wait in the first places of its own
+// part of `out`, which k_root_ids and k_site_ids write afterwards (word t belongs
+// to sites from 32 t on, so a short block's words fit too): no scratch for them.
 __global__ void __launch_bounds__(kRelThreads) k_root_counts(int32_t n, const int32_t *__restrict__ lab,
                                                              int32_t *__restrict__ block_cnt,
-                                                             uint32_t *__restrict__ roots) {
+                                                             int32_t *__restrict__ out) {
     __shared__ int s_w[kRelThreads / 32];
     static_assert(kRelPerThread == 32, "one ballot per lane");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -35,7 +37,8 @@ __global__ void __launch_bounds__(kRelThreads) k_root_counts(int32_t n, const in
         const unsigned b = __ballot_sync(kFull, i < n && __ldg(lab + i) == (int32_t)i);
         if (lane == u) mine = b;
     }
-    roots[(int64_t)blockIdx.x * kRelThreads + threadIdx.x] = mine;
+    const int64_t first = (int64_t)blockIdx.x * kRelBlock;
+    if (first + 32 * (int)threadIdx.x < n) out[first + threadIdx.x] = (int32_t)mine;
     const int c = __reduce_add_sync(kFull, __popc(mine));
     if (lane == 0) s_w[warp] = c;
     __syncthreads();
@@ -76,13 +79,14 @@ __global__ void __launch_bounds__(1024) k_scan_counts(int32_t nb, int32_t *__res
 // from the bits of k_root_counts, not from the labels again, and a warp needs
 // the other warps' totals once, so the block meets at one barrier (stepping the
 // whole block through 256 sites at a time took 96 barriers).
-__global__ void __launch_bounds__(kRelThreads) k_root_ids(const uint32_t *__restrict__ roots,
-                                                          const int32_t *__restrict__ block_off,
+__global__ void __launch_bounds__(kRelThreads) k_root_ids(int32_t n, const int32_t *__restrict__ block_off,
                                                           int32_t *__restrict__ out, int32_t *__restrict__ sizes) {
     __shared__ int32_t s_w[kRelThreads / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t base = (int64_t)blockIdx.x * kRelBlock + warp * (32 * kRelPerThread) + lane;
-    const unsigned mine = roots[(int64_t)blockIdx.x * kRelThreads + threadIdx.x];
+    // (every thread has its word before the barrier below, none writes before it)
+    const int64_t first = (int64_t)blockIdx.x * kRelBlock;
+    const unsigned mine = first + 32 * (int)threadIdx.x < n ? (unsigned)out[first + threadIdx.x] : 0u;
     int incl = __popc(mine);
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {

@@ -58,3 +58,33 @@ def test_spanning_set_limit(ctx, n_top, spans):
     assert ccl.ccl_spanning(ctx, n, args[0], args[1], n_top, args[2], bottom.size, res) == ccl.CCL_OK
     assert ccl.ccl_sync(ctx) == ccl.CCL_OK
     assert int(res) == (int(min(top[-1], top[n_top // 2])) if spans else -1)
+
+
+def test_relabel_needs_a_count_per_block_only():
+    """Scratch of 4 bytes per 8192 sites: a context whose scratch is that large (from
+    the largest cluster of 100 sites, 416 bytes) relabels 104 blocks under capture,
+    where nothing can be allocated."""
+    n = 104 * 8192 - 5
+    lab = _labels(n, "pairs", 3)
+    c = ccl.ccl_context_create(0)
+    s = torch.cuda.Stream()
+    d = torch.from_numpy(lab).to(DEV)
+    seq, sizes = (torch.full((n,), -1, dtype=torch.int32, device=DEV) for _ in range(2))
+    count, big = (torch.zeros(k, dtype=torch.int32, device=DEV) for k in (1, 2))
+    torch.cuda.synchronize()
+    assert ccl.ccl_largest_cluster(c, 100, d, big, s) == ccl.CCL_OK
+    assert ccl.ccl_relabel(c, 100, d, seq, count, sizes, s) == ccl.CCL_OK        # (loads the kernels)
+    assert ccl.ccl_sync(c, s) == ccl.CCL_OK
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        assert ccl.ccl_relabel(c, n, d, seq, count, sizes, s) == ccl.CCL_OK
+    want_seq, want_sizes = stats.sequential(lab)
+    for _ in range(2):
+        seq.fill_(-1)
+        sizes.fill_(-1)
+        g.replay()
+        torch.cuda.synchronize()
+        assert int(count) == want_sizes.size
+        assert np.array_equal(seq.cpu().numpy(), want_seq)
+        assert np.array_equal(sizes.cpu().numpy()[:want_sizes.size], want_sizes)
+    ccl.ccl_context_destroy(c)
