@@ -946,7 +946,7 @@ ccl_status ccl_context_create(ccl_context **out, int device) {
                                  (int)kDenseSmem);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_span_few, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 2 * kSpanTop * (int)sizeof(int32_t));
+                                 kSpanSpread * kSpanTop * (int)sizeof(int32_t));
     if (e != cudaSuccess) {
         (void)cudaGetLastError();
         ccl_context_destroy(ctx);
@@ -1303,11 +1303,11 @@ ccl_status ccl_spanning(ccl_context *ctx, int32_t n, const int32_t *labels, cons
     if ((n_top > 0 && !top) || (n_bottom > 0 && !bottom)) return CCL_ERR_INVALID_ARGUMENT;
     DeviceGuard guard(ctx->device);
     cudaStream_t s = (cudaStream_t)stream;
-    if (n_top <= kSpanTop && n_bottom <= 16 * kSpanTop) {
+    if (n_top <= kSpanTop && n_bottom <= kSpanBottom) {
         int32_t slots = 64;
-        while (slots < 2 * n_top) slots *= 2;
-        k_span_few<<<1, kSpanThreads, (size_t)slots * sizeof(int32_t), s>>>(n, labels, top, n_top, bottom, n_bottom,
-                                                                          slots, result, ctx->d_err);
+        while (slots < kSpanSpread * n_top) slots *= 2;
+        k_span_few<<<kSpanCtas, kSpanThreads, (size_t)slots * sizeof(int32_t), s>>>(
+            n, labels, top, n_top, bottom, n_bottom, slots, result, ctx->d_err);
         CCL_CUDA(cudaGetLastError());
         return CCL_OK;
     }

@@ -8,6 +8,7 @@
 //  * the largest cluster (its size and label).
 #pragma once
 #include <stdint.h>
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include "ccl_types.cuh"
@@ -226,47 +227,68 @@ __global__ void k_span_check(int32_t n, const int32_t *__restrict__ lab, const i
     }
 }
 
-// The spanning test of few top sites in one launch: the top labels go into a
-// hash set in shared memory (open addressing, at most half full), the bottom
-// labels are looked up in it. Clearing a bit per site, marking, checking and
-// finishing took four launches.
+// The spanning test of few sites in one launch of one cluster: every CTA keeps all
+// top labels in a hash set in its shared memory (open addressing, at most a
+// quarter full: the slowest lane of a warp decides) and looks its share of the
+// bottom labels up. Clearing a bit per site, marking, checking and finishing took
+// four launches. An SM loads scattered labels at 1 ns a site, so the loads are split
+// over the CTAs, and the top labels are then read from each other's shared memory.
+// Four launches / this, 4096 + 4096 and 8192 + 12,288 scattered sites of 16.8M: 17 / 13
+// and 17 / 17 us, 2 x 5792 in rows 17 / 11 (one CTA: 17, 35 and 11). The line lies
+// at 16,384 bottom sites: 8192 + 65,536 scattered ones 17 / 21.
 constexpr int kSpanTop = 8192;              // most top sites of this path
+constexpr int kSpanBottom = 16384;          // most bottom sites
+constexpr int kSpanSpread = 4;              // slots per top site, at least
 constexpr int kSpanThreads = 1024;
-__global__ void __launch_bounds__(kSpanThreads) k_span_few(int32_t n, const int32_t *__restrict__ lab,
-                                                           const int32_t *__restrict__ top, int32_t n_top,
-                                                           const int32_t *__restrict__ bottom, int32_t n_bottom,
-                                                           int32_t slots, int32_t *__restrict__ best, unsigned *err) {
-    extern __shared__ int32_t s_set[];      // `slots`, a power of two, -1 where empty
-    __shared__ unsigned s_best;
-    for (int t = threadIdx.x; t < slots; t += kSpanThreads) s_set[t] = -1;
-    if (threadIdx.x == 0) s_best = 0xffffffffu;         // -1: no cluster spans
-    __syncthreads();
-    const unsigned mask = (unsigned)slots - 1u;
-    for (int t = threadIdx.x; t < n_top; t += kSpanThreads) {
-        const int32_t s = top[t];
+constexpr int kSpanCtas = kSpanTop / kSpanThreads;      // (a top site per thread)
+__global__ void __cluster_dims__(kSpanCtas, 1, 1) __launch_bounds__(kSpanThreads)
+    k_span_few(int32_t n, const int32_t *__restrict__ lab, const int32_t *__restrict__ top, int32_t n_top,
+               const int32_t *__restrict__ bottom, int32_t n_bottom, int32_t slots, int32_t *__restrict__ best,
+               unsigned *err) {
+    extern __shared__ __align__(16) int32_t s_set[];    // `slots`, a power of two, -1 where empty
+    __shared__ int32_t s_top[kSpanThreads]; // the labels of the CTA's top sites
+    __shared__ unsigned s_best;             // (the first CTA's is used)
+    const auto cluster = cooperative_groups::this_cluster();
+    const int first = (int)cluster.block_rank() * kSpanThreads + (int)threadIdx.x;
+    const auto label = [&](const int32_t *__restrict__ sites, int t) {
+        const int32_t s = sites[t];
         const int32_t l = (uint32_t)s < (uint32_t)n ? lab[s] : -1;
-        if ((uint32_t)l >= (uint32_t)n) { atomicOr(err, kErrIndex); continue; }
-        unsigned h = ((unsigned)l * 2654435761u >> 16) & mask;
+        if ((uint32_t)l < (uint32_t)n) return l;
+        atomicOr(err, kErrIndex);
+        return -1;
+    };
+    s_top[threadIdx.x] = first < n_top ? label(top, first) : -1;
+    for (int t = threadIdx.x; t < slots / 4; t += kSpanThreads)
+        reinterpret_cast<int4 *>(s_set)[t] = make_int4(-1, -1, -1, -1);
+    if (threadIdx.x == 0) s_best = 0xffffffffu;         // -1: no cluster spans
+    cluster.sync();
+    const unsigned mask = (unsigned)slots - 1u;
+    int32_t l[kSpanCtas];
+#pragma unroll
+    for (int c = 0; c < kSpanCtas; ++c)
+        l[c] = c * kSpanThreads < n_top ? cluster.map_shared_rank(s_top, c)[threadIdx.x] : -1;
+#pragma unroll
+    for (int c = 0; c < kSpanCtas; ++c) {
+        if (l[c] < 0) continue;
+        unsigned h = ((unsigned)l[c] * 2654435761u >> 16) & mask;
         for (int probe = 0; probe < slots; ++probe, h = (h + 1u) & mask) {
-            const int32_t was = atomicCAS(&s_set[h], -1, l);
-            if (was == -1 || was == l) break;
+            const int32_t was = atomicCAS(&s_set[h], -1, l[c]);
+            if (was == -1 || was == l[c]) break;
         }
     }
     __syncthreads();
     unsigned mine = 0xffffffffu;
-    for (int t = threadIdx.x; t < n_bottom; t += kSpanThreads) {
-        const int32_t s = bottom[t];
-        const int32_t l = (uint32_t)s < (uint32_t)n ? lab[s] : -1;
-        if ((uint32_t)l >= (uint32_t)n) { atomicOr(err, kErrIndex); continue; }
-        if ((unsigned)l >= mine) continue;
-        unsigned h = ((unsigned)l * 2654435761u >> 16) & mask;
+    for (int t = first; t < n_bottom; t += kSpanCtas * kSpanThreads) {
+        const int32_t b = label(bottom, t);
+        if (b < 0 || (unsigned)b >= mine) continue;
+        unsigned h = ((unsigned)b * 2654435761u >> 16) & mask;
         for (int probe = 0; probe < slots && s_set[h] != -1; ++probe, h = (h + 1u) & mask)
-            if (s_set[h] == l) { mine = (unsigned)l; break; }
+            if (s_set[h] == b) { mine = (unsigned)b; break; }
     }
     mine = __reduce_min_sync(kFull, mine);
-    if ((threadIdx.x & 31) == 0) atomicMin(&s_best, mine);
-    __syncthreads();
-    if (threadIdx.x == 0) *best = (int32_t)s_best;
+    if ((threadIdx.x & 31) == 0 && mine != 0xffffffffu) atomicMin(cluster.map_shared_rank(&s_best, 0), mine);
+    cluster.sync();                         // (also: no CTA leaves while another reads its labels)
+    if (first == 0) *best = (int32_t)s_best;
 }
 
 // Largest cluster (Section 4's largest-cluster statistic): cnt[l] = sites

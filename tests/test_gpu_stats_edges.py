@@ -88,3 +88,29 @@ def test_relabel_needs_a_count_per_block_only():
         assert np.array_equal(seq.cpu().numpy(), want_seq)
         assert np.array_equal(sizes.cpu().numpy()[:want_sizes.size], want_sizes)
     ccl.ccl_context_destroy(c)
+
+
+@pytest.mark.parametrize("n_top", [1, 1023, 1025, 8192])
+@pytest.mark.parametrize("n_bottom", [1, 8193, 16384, 16385, 70_000])
+def test_spanning_scattered_sites(ctx, n_top, n_bottom):
+    """Sites anywhere, some twice, some out of range (skipped and latched), on both
+    sides of the one-launch path's limits and of a CTA's share of them."""
+    n = 300_000
+    rng = np.random.default_rng(n_top + n_bottom)
+    for spans in (False, True):
+        lab = np.arange(n, dtype=np.int32)
+        top, bottom = rng.integers(0, n // 2, n_top), rng.integers(n // 2, n, n_bottom)
+        if spans:
+            lab[bottom[-1]] = top[-1]
+            lab[bottom[n_bottom // 2]] = top[n_top // 3]
+        for bad in (False, True):
+            t, b = top, bottom
+            if bad:
+                t, b = np.append(t[2:], [n, -1]), np.append(b[1:], n + 7)
+            t_in, b_in = t[(t >= 0) & (t < n)], b[b < n]
+            common = set(lab[t_in].tolist()) & set(lab[b_in].tolist())
+            res = torch.zeros(1, dtype=torch.int32, device=DEV)
+            args = [torch.from_numpy(a.astype(np.int32)).to(DEV) for a in (lab, t, b)]
+            assert ccl.ccl_spanning(ctx, n, args[0], args[1], t.size, args[2], b.size, res) == ccl.CCL_OK
+            assert ccl.ccl_sync(ctx) == (ccl.CCL_ERR_INDEX_OUT_OF_RANGE if bad else ccl.CCL_OK)
+            assert int(res) == (min(common) if common else -1)
