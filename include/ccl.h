@@ -89,9 +89,9 @@ CCL_API void ccl_context_destroy(ccl_context *ctx);
 /* Tunable options (ccl_set_option / ccl_get_option). */
 typedef enum {
     CCL_OPT_PRE_ANALYSIS = 0,  /* 1: run step (ii) as a pass of its own before (iii); 0: skip it;
-                                  -1 (default): the labels of each instance
-                                  are sampled on the device and the pass runs only where few
-                                  sites are roots (long chains) */
+                                  -1 (default): calls of at most 2^18 sites run it; in larger
+                                  ones the labels of each instance are sampled on the device
+                                  and the pass runs only where few sites are roots (long chains) */
     CCL_OPT_BLOCK_THREADS = 1, /* threads per CTA of the analysis kernel (64..512, multiple of 32) */
     CCL_OPT_USE_GRAPHS = 2,    /* 1 (default): replay captured CUDA graphs for repeated shapes */
     CCL_OPT_PROFILE = 3,       /* 1: record CUDA events between the steps (ccl_get_step_times);

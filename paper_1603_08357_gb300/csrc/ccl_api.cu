@@ -27,7 +27,7 @@ namespace {
 struct TuneChoice {
     int threads = 256;
     int ctas_per_sm = 0;
-    int pre_analysis = -1;  // step (ii): 1 run, 0 skip; -1 by sample on the device (k_analysis)
+    int pre_analysis = -1;  // step (ii): 1 run, 0 skip; -1 the library's choice (resolve_pre)
     int link_mode = -1;     // step (iii): 0 root to root, 1 root to the other chain's node; -1 by window (k_reduce)
     int refill = 1;         // step (iii): 1 static per-lane pairs, 0 in-order hand-out
     int ana_seq = 1;        // steps (ii)/(iv): 1 contiguous ranges per warp, 0 interleaved
@@ -421,17 +421,11 @@ bool resolve_park(const TuneChoice &tc, const Params &P) {
     return tc.ana_seq && P.iter_cap == 0 && tc.ana_park > 0;    // (the iteration-cap test option takes the plain walk)
 }
 
-// Whether step (ii) runs over all sites: as set, else not. Near p_c steps (i)
-// and (iii) do without it (the band shortcut and the in-window jump of step (i)
-// leave short chains, and step (iii)'s search is bounded by the window's
-// slowest pair, not by the mean chain), and step (iv) repeats its work: on one
-// GB300 a call with / without it took 356 / 313 us (triangle 4096^2 at p_c),
-// 1105 / 910 us (Bethe lattice, 24 shells, random numbering), 5.73 / 5.05 ms
-// (triangle 16384^2), 11.3 / 9.9 ms (1024 mixed instances) and 30.2 / 30.6 us
-// (honeycomb 64^2).
-// Left to the library, the pass samples the labels of each instance and walks
-// only where chains are long (k_analysis), which the data alone can tell.
-bool resolve_pre(const TuneChoice &tc) { return tc.pre_analysis > 0; }
+// Step (ii): 1 walk all sites, 0 leave it out, -1 walk the instances whose sampled
+// labels are long chains (k_analysis, kSample). As set, else by size (kWalkSites).
+int resolve_pre(const TuneChoice &tc, const Params &P) {
+    return tc.pre_analysis < 0 && kChunk * P.n_chunks <= kWalkSites ? 1 : tc.pre_analysis;
+}
 constexpr int kSampleGroup = 64;     // groups per run of the sampling pass beyond L2
 
 // Step (iii) by short walks (k_reduce_park) for labels of at most three eighths of
@@ -442,7 +436,7 @@ bool walks_short(const ccl_context *ctx, const TuneChoice &tc, const Params &P) 
 
 // Records in the context's statistics the settings a call runs with.
 void note_settings(ccl_context *ctx, const TuneChoice &tc, const Params &P) {
-    ctx->last.pre_analysis = tc.pre_analysis;
+    ctx->last.pre_analysis = resolve_pre(tc, P);
     // (by window only in the slots of a single instance, k_reduce<false, true, ..>)
     ctx->last.link_mode = tc.link_mode >= 0 ? tc.link_mode : P.K == 1 && tc.refill && !walks_short(ctx, tc, P) ? -1 : 0;
     ctx->last.refill = tc.refill;
@@ -515,7 +509,8 @@ ccl_status enqueue_tail(ccl_context *ctx, const Params &P0, bool batched, const 
                                    : (park ? k_analysis<false, true> : k_analysis<false, false>),
                            g, (unsigned)T, smem, s, chain, A);
     };
-    if (tc.pre_analysis != 0) CCL_CUDA(analysis(!resolve_pre(tc)));
+    const int pre = resolve_pre(tc, P);
+    if (pre != 0) CCL_CUDA(analysis(pre < 0));
     if (profile) CCL_CUDA(cudaEventRecord(ctx->ev[2], s));
     auto reduce = k_reduce<false, true, false>;
     if (short_walk) reduce = batched ? k_reduce_park<true> : k_reduce_park<false>;

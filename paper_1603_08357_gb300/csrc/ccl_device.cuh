@@ -896,6 +896,13 @@ constexpr int kParkCap = 32 * kAnaChunks + 32;       // < 32 left + one group's 
 // p_c (0.13) are about even. Deciding per stretch of 96 sites instead costs
 // more than either at the line (triangle 2048^2 at 1.5 p_c 173).
 constexpr int kSampleRoots = 8, kSampleChunks = 12;
+// Calls of at most this many sites are walked without a sample. They are launches
+// and latency: the walk costs them what the sample does, and mends the inputs the
+// sample leaves alone although step (iii) has long chains to follow (square 256^2 at
+// 1.3 p_c 41 us sampled, 36 walked; triangle 256^2 at 1.5 p_c 46 and 38; at p_c
+// honeycomb 64^2 27 and 26, triangle 512^2 38 and 39). From a million sites on the
+// walk costs more at p_c than it gives (triangle 1024^2 52 and 55).
+constexpr int64_t kWalkSites = 1 << 18;
 template <bool kBatched, bool kPark, bool kSample = false>
 __global__ void __launch_bounds__(512, 4) k_analysis(Params P) {
     extern __shared__ int s_park[];                  // kPark: site and label of kParkCap chains per warp

@@ -149,7 +149,8 @@ extern "C" ccl_status ccl_label_noalloc(int32_t n, int64_t nnz, const int32_t *r
     cudaError_t e = cudaMemsetAsync(d->scratch + kOffErr, 0, sizeof(unsigned), s);
     if (e == cudaSuccess) {
         k_init<false><<<(unsigned)g_init, kInitThreads, kInitSmem, s>>>(P);
-        k_analysis<false, false, true><<<(unsigned)g_ana, 256, 0, s>>>(P);
+        if (n <= kWalkSites) k_analysis<false, false><<<(unsigned)g_ana, 256, 0, s>>>(P);
+        else k_analysis<false, false, true><<<(unsigned)g_ana, 256, 0, s>>>(P);
         k_reduce_park<false><<<(unsigned)g_red, kRedThreads, sizeof(uint32_t) * (size_t)(g_init + 1), s>>>(P);
         k_analysis<false, false><<<(unsigned)g_ana, 256, 0, s>>>(P);
         e = cudaGetLastError();

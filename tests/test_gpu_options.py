@@ -7,7 +7,7 @@ import torch
 import lattices as L
 import oracle
 import paper_1603_08357_gb300 as ccl
-from ccl_testutil import DEV, gpu_label, to_dev
+from ccl_testutil import DEV, gpu_label, gpu_label_batched, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -89,3 +89,14 @@ def test_link_mode_as_set_or_by_window(fresh):
         for lat, by_window in ((small, 0), (large, -1)):
             assert np.array_equal(gpu_label(fresh, lat), oracle.uf_label(lat))
             assert ccl.ccl_get_stats(fresh).link_mode == (setting if setting >= 0 else by_window)
+
+
+def test_small_calls_walk_step_ii(fresh):
+    """Up to 2^18 sites, single and batched, step (ii) left to the library runs."""
+    for side, ran in ((512, 1), (513, -1)):
+        lat = L.square(side, 0.65, 2)
+        assert np.array_equal(gpu_label(fresh, lat), oracle.uf_label(lat))
+        assert ccl.ccl_get_stats(fresh).pre_analysis == ran
+        b = L.make_batch([dict(kind="square", L=side // 2, p=0.65, seed=k) for k in range(4 if ran == 1 else 5)])
+        assert np.array_equal(gpu_label_batched(fresh, b), oracle.uf_label_batched(b))
+        assert ccl.ccl_get_stats(fresh).pre_analysis == ran
