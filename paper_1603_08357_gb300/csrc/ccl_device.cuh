@@ -336,35 +336,6 @@ __device__ __forceinline__ void init_produce(const Params &P, Stage *st, uint64_
     drain_armed(full, t_local, P.err);
 }
 
-// General scan of one lane's row (rows longer than kRowRegs, or parts of the
-// input outside the shared-memory copy): per-entry bounds-checked reads.
-// the open bit of local entry e of instance I (row i, column j < i)
-template <bool kGen>
-__device__ __forceinline__ bool entry_open(const Params &P, const Stage &S, const Inst &I, int32_t e,
-                                           int32_t i, int32_t j) {
-    if (kGen) return gen_bond_open(P.gen_seed, P.gen_thr, (uint32_t)j, (uint32_t)i);
-    const StageHdr &h = S.h;
-    const int64_t ge = I.bit_off + e;
-    const int64_t we = ge >> 5;
-    const uint32_t w = (we >= h.w_lo && we < h.w_hi) ? S.bw[we - h.w_lo] : __ldg(I.bits + we);
-    return (w >> (ge & 31)) & 1u;
-}
-
-template <bool kGen>
-__device__ __forceinline__ void scan_row_general(const Params &P, const Stage &S, const Inst &I, int32_t a,
-                                                 int32_t a_next, int32_t i, int32_t &m, int32_t &mk,
-                                                 int32_t &cnt, bool &bad) {
-    const StageHdr &h = S.h;
-    for (int32_t e = a; e < a_next; ++e) {
-        const int32_t j = (e >= h.ci_lo && e < h.ci_hi) ? S.ci[e - h.ci_lo] : __ldg(I.col_idx + e);
-        bad |= (uint32_t)j >= (uint32_t)I.n;
-        if ((uint32_t)j < (uint32_t)i && entry_open<kGen>(P, S, I, e, i, j)) {
-            ++cnt;
-            if (j < m) { m = j; mk = e; }
-        }
-    }
-}
-
 // Per-tile values a consumer warp computes once: the stage-relative bit
 // offset of entry 0 and the number of copied bits (32-bit), and the range of
 // the instance's tiles whose labels are final and visible here.
@@ -392,21 +363,61 @@ __device__ __forceinline__ void load_tile_hdr(const StageHdr &h, TileHdr &th, Ti
     tc.vis_hi = h.t_vis_hi;
 }
 
-// One chunk of 32 sites. The tiles of this CTA's band that were finished at
-// least kStages tiles ago are visible (their labels were released through the
-// stage barriers): a site whose smallest open lower neighbour m lies in such
-// a tile takes label[m] (the root of m's tree after steps (i)/(ii)) instead of
-// m, which shortcuts the chain step (ii) would walk.
-// What the emission of a scanned chunk needs (per lane).
-struct ChunkRes {
-    int32_t i, a, a_next, mk;
-    int32_t lab;        // label[i] to store (may be a load still in flight)
-    uint32_t resmask;
-    int32_t r;          // residual pairs of the lane's site
-    bool fast;          // warp-uniform: the register path scanned the chunk
+// The open lower entries among the `cnt` (at most kRowRegs) entries from e on of
+// row i, as a mask, and their columns. A tile's entries are in the stage or, when
+// it has more than the stage holds, all read from global memory; either way a
+// lane's loads of a block do not depend on one another.
+template <bool kGen>
+__device__ __forceinline__ uint32_t lower_block(const Params &P, const Stage &S, const Inst &I, const TileCtx &tc,
+                                                int32_t e, int32_t cnt, int32_t i, int32_t (&j)[kRowRegs], bool &bad) {
+    uint32_t win = 0;
+    if (tc.staged) {
+        const int32_t *col = S.ci + (e - S.h.ci_lo);
+#pragma unroll
+        for (int u = 0; u < kRowRegs; ++u) j[u] = u < cnt ? col[u] : -1;
+        if (!kGen && cnt > 0) {
+            const int32_t rel = tc.rb0 + e;
+            win = __funnelshift_r(S.bw[rel >> 5], S.bw[(rel + cnt - 1) >> 5], (uint32_t)rel & 31u);
+        }
+    } else {
+        const int32_t *col = I.col_idx + e;
+#pragma unroll
+        for (int u = 0; u < kRowRegs; ++u) j[u] = u < cnt ? __ldg(col + u) : -1;
+        if (!kGen && cnt > 0) {
+            const int64_t ge = I.bit_off + e;
+            win = __funnelshift_r(__ldg(I.bits + (ge >> 5)), __ldg(I.bits + ((ge + cnt - 1) >> 5)), (uint32_t)ge & 31u);
+        }
+    }
+    uint32_t low = 0;
+#pragma unroll
+    for (int u = 0; u < kRowRegs; ++u) {
+        const bool lower = (uint32_t)j[u] < (uint32_t)i;            // (none past cnt)
+        const bool open = kGen ? lower && gen_bond_open(P.gen_seed, P.gen_thr, (uint32_t)j[u], (uint32_t)i)
+                               : lower && ((win >> u) & 1u);
+        bad |= u < cnt && (uint32_t)j[u] >= (uint32_t)I.n;
+        low |= open ? 1u << u : 0u;
+    }
+    return low;
+}
+
+// One chunk of 32 sites, whatever its rows: in blocks of kRowRegs entries. The tiles
+// of this CTA's band that were finished at least kStages tiles ago are visible
+// (their labels were released through the stage barriers): a site whose smallest
+// open lower neighbour m lies in such a tile takes label[m] (the root of m's tree
+// after steps (i)/(ii)) instead of m, which shortcuts the chain step (ii) would walk.
+// What bounds it is the latency of the columns when the stage does not hold them:
+// the blocks' loads overlap. Step (i) of 4M sites with 12 random near entries each
+// took 550 us entry by entry with four rows a lane (349 with two, twice the warps),
+// 150 so; of a tree of 23,437 sites, whose last tile the stage holds short of its last
+// entries, 18 (13) and 14.
+struct ChunkRes {           // what the emission needs (per lane)
+    int32_t i, a, deg, mk;
+    int32_t lab;            // label[i] to store (may be a load still in flight)
+    uint32_t resmask;       // residual entries among the row's first 32
+    int32_t r;              // residual pairs of the lane's site
 };
 
-template <bool kBatched, bool kGen = false>
+template <bool kGen>
 __device__ __forceinline__ void init_scan_chunk(const Params &P, const Stage &S, const Inst &I,
                                                 int cc, int lane, const TileCtx &tc, ChunkRes &cr) {
     const StageHdr &h = S.h;
@@ -432,43 +443,22 @@ __device__ __forceinline__ void init_scan_chunk(const Params &P, const Stage &S,
     // all of that range (columns and bits)
     const int32_t deg = a_next - a;
     const int32_t dmax = __reduce_max_sync(kFull, (uint32_t)deg);
-    const bool all_fast = dmax <= kRowRegs && tc.staged;
-    int32_t m = INT32_MAX, cnt = 0;
-    int32_t mk = -1;
+    int32_t m = INT32_MAX, cnt = 0, mk = -1;
     uint32_t resmask = 0;
     bool bad = false;
-    if (all_fast) {
-        const int32_t *col = S.ci + (a - h.ci_lo);
-        uint32_t win = 0;
-        if (!kGen && deg > 0) {
-            const int32_t rel = tc.rb0 + a;
-            win = __funnelshift_r(S.bw[rel >> 5], S.bw[(rel + deg - 1) >> 5], (uint32_t)rel & 31u);
-        }
-        uint32_t lowmask = 0, jmax = 0;
+    for (int32_t t = 0; t < dmax; t += kRowRegs) {
+        int32_t j[kRowRegs];
+        const uint32_t low = lower_block<kGen>(P, S, I, tc, a + t, min(max(deg - t, 0), kRowRegs), i, j, bad);
 #pragma unroll
-        for (int t = 0; t < kRowRegs; ++t) {
-            if (t >= dmax) break;
-            if (t < deg) {
-                const int32_t j = col[t];
-                jmax = max(jmax, (uint32_t)j);
-                const bool open = kGen ? ((uint32_t)j < (uint32_t)i &&
-                                          gen_bond_open(P.gen_seed, P.gen_thr, (uint32_t)j, (uint32_t)i))
-                                       : ((win >> t) & 1u) != 0;
-                if (open && (uint32_t)j < (uint32_t)i) {
-                    lowmask |= 1u << t;
-                    if (j < m) { m = j; mk = t; }
-                }
-            }
-        }
-        bad = jmax >= (uint32_t)n;
-        cnt = __popc(lowmask);
-        resmask = cnt ? (lowmask & ~(1u << mk)) : 0u;
-    } else {
-        scan_row_general<kGen>(P, S, I, a, a_next, i, m, mk, cnt, bad);
+        for (int u = 0; u < kRowRegs; ++u)
+            if (((low >> u) & 1u) && j[u] < m) { m = j[u]; mk = t + u; }
+        cnt += __popc(low);
+        if (t < 32) resmask |= low << t;
     }
+    if (cnt && mk < 32) resmask &= ~(1u << mk);
     if (bad) raise_err(P.err, kErrIndex);
-    // the label; the caller stores it after scanning its other chunks, so the
-    // shortcut's load below has their scans' time to arrive
+    // the label; the caller stores it after the prefix sum over the pairs, so the
+    // shortcut's load below has that time to arrive
     int32_t lab = cnt ? m : i;
     if (cnt) {
         const int32_t mt = (int32_t)((uint32_t)m / kTileSites);
@@ -477,10 +467,9 @@ __device__ __forceinline__ void init_scan_chunk(const Params &P, const Stage &S,
     cr.lab = lab;
     cr.i = i;
     cr.a = a;
-    cr.a_next = a_next;
+    cr.deg = deg;
     cr.mk = mk;
     cr.resmask = resmask;
-    cr.fast = all_fast;
     cr.r = cnt > 1 ? cnt - 1 : 0;
 }
 
@@ -677,36 +666,28 @@ __device__ __forceinline__ bool init_scan_rows(const Params &P, const Stage &S, 
     return true;
 }
 
-// Writes the residual pairs of one scanned chunk from queue slot `slot` on.
+// Writes the residual pairs of one scanned chunk from queue slot `slot` on (the
+// warp's slots have been checked against the queue's end).
 // A pair {i, j} is stored as (label[i], j): label[i] is i's parent in the
 // label forest and, i not being a root, step (iii) never rewrites it, so the
 // pair joins the same two trees and its root search starts one hop higher.
 template <bool kBatched, bool kGen = false>
-__device__ __forceinline__ void init_emit_chunk(const Params &P, const Stage &S, const Inst &I,
+__device__ __forceinline__ void init_emit_chunk(const Params &P, const Stage &S, const Inst &I, const TileCtx &tc,
                                                 const ChunkRes &cr, int64_t slot) {
-    const StageHdr &h = S.h;
-    const int32_t i = cr.i;
-    const int32_t up = cr.lab;
-    if (slot + cr.r > P.q_cap) { raise_err(P.err, kErrIndex); return; }   // corrupt rows only
-    if (cr.fast) {
-        const int32_t *col = S.ci + (cr.a - h.ci_lo);
-        uint32_t resmask = cr.resmask;
-        while (resmask) {
-            const int t = __ffs(resmask) - 1;
-            resmask &= resmask - 1;
-            P.q[slot] = make_int2(up, col[t]);
-            if (kBatched) P.qk[slot] = h.k;
-            ++slot;
-        }
-    } else {
-        for (int32_t e = cr.a; e < cr.a_next; ++e) {
-            const int32_t j = (e >= h.ci_lo && e < h.ci_hi) ? S.ci[e - h.ci_lo] : __ldg(I.col_idx + e);
-            if ((uint32_t)j < (uint32_t)i && e != cr.mk && entry_open<kGen>(P, S, I, e, i, j)) {
-                P.q[slot] = make_int2(up, j);
-                if (kBatched) P.qk[slot] = h.k;
-                ++slot;
-            }
-        }
+    const auto put = [&](int32_t j) {
+        P.q[slot] = make_int2(cr.lab, j);
+        if (kBatched) P.qk[slot] = S.h.k;
+        ++slot;
+    };
+    const int32_t *col = tc.staged ? S.ci + (cr.a - S.h.ci_lo) : I.col_idx + cr.a;
+    for (uint32_t res = cr.resmask; res; res &= res - 1) put(col[__ffs(res) - 1]);
+    for (int32_t t = 32; t < cr.deg; t += kRowRegs) {           // past the mask: scanned again
+        int32_t j[kRowRegs];
+        bool bad = false;
+        const uint32_t low = lower_block<kGen>(P, S, I, tc, cr.a + t, min(cr.deg - t, kRowRegs), cr.i, j, bad);
+#pragma unroll
+        for (int u = 0; u < kRowRegs; ++u)
+            if (((low >> u) & 1u) && t + u != cr.mk) put(j[u]);
     }
 }
 
@@ -739,6 +720,33 @@ __device__ __forceinline__ void init_emit_rows(const Params &P, const Stage &S, 
         ++qp;
         if (kBatched) ++kp;
     }
+}
+
+// Queue slots for the residual pairs of a warp's sites, r of the lane's: sets the
+// first slot and the warp's total, returns the pairs of the lanes before.
+__device__ __forceinline__ int take_slots(const Stage &S, BandSlots &bands, int lane, int r, int64_t &slot, int &total) {
+    const int incl = warp_incl_scan(r, lane);
+    total = __shfl_sync(kFull, incl, 31);
+    unsigned long long base = 0;
+    if (total > 0) {
+        if (lane == 0) base = atomicAdd(&bands.cnt[S.h.slot], (unsigned long long)total);
+        base = __shfl_sync(kFull, base, 0);
+    }
+    slot = S.h.qband + (int64_t)base;
+    return incl - r;
+}
+
+// Whether the slots end inside the queue (always, but for corrupt rows: then what is
+// left of it becomes pairs (0, 0), as step (iii) reads every slot up to the end).
+template <bool kBatched>
+__device__ __forceinline__ bool slots_fit(const Params &P, int32_t k, int64_t slot, int total, int lane) {
+    if (slot + total <= P.q_cap) return true;
+    if (lane == 0) raise_err(P.err, kErrIndex);
+    for (int64_t e = slot + lane; e < P.q_cap; e += 32) {
+        P.q[e] = make_int2(0, 0);
+        if (kBatched) P.qk[e] = k;
+    }
+    return false;
 }
 
 template <bool kBatched, bool kGen = false>
@@ -779,7 +787,7 @@ __global__ void __launch_bounds__(kInitThreads, kInitCtas) k_init(Params P) {
         TileCtx tc;
         TileHdr th;
         load_tile_hdr(S.h, th, tc);
-        // The chunks are scanned first; their pairs then take one range of
+        // The warp's rows are scanned first; their pairs then take one range of
         // queue slots (one prefix sum and one band counter update per tile),
         // taken before the labels are stored: the shortcut's label loads land
         // meanwhile.
@@ -787,54 +795,30 @@ __global__ void __launch_bounds__(kInitThreads, kInitCtas) k_init(Params P) {
         if (loc < th.ts) {
             const int32_t s00 = th.s0 + loc;
             RowsRes q;
-            ChunkRes c[kRows];
-            const bool fast = init_scan_rows<kGen>(P, S, I, s00, lane, tc, th, q);
-            int rr;
-            if (fast) {
-                rr = __popc(q.res);
-            } else {
-                rr = 0;
-#pragma unroll
-                for (int k = 0; k < kRows; ++k) {
-                    c[k].r = 0;
-                    if (loc + k * kChunk < th.ts) init_scan_chunk<kBatched, kGen>(P, S, I, warp * kRows + k, lane, tc, c[k]);
-                    rr += c[k].r;
-                }
-            }
-            const int incl = warp_incl_scan(rr, lane);
-            const int total = __shfl_sync(kFull, incl, 31);
-            unsigned long long base = 0;
-            if (total > 0) {
-                if (lane == 0) base = atomicAdd(&bands.cnt[S.h.slot], (unsigned long long)total);
-                base = __shfl_sync(kFull, base, 0);
-            }
-            if (fast) {
+            if (init_scan_rows<kGen>(P, S, I, s00, lane, tc, th, q)) {
+                const int rr = __popc(q.res);
+                int64_t slot;
+                int total;
+                const int before = take_slots(S, bands, lane, rr, slot, total);
                 int32_t *out = I.labels + s00 + lane;
 #pragma unroll
                 for (int k = 0; k < kRows; ++k) out[kChunk * k] = q.lab[k];
+                if (total > 0 && slots_fit<kBatched>(P, th.k, slot, total, lane))
+                    init_emit_rows<kBatched>(P, S, th, q, slot + before, rr);
             } else {
-#pragma unroll
-                for (int k = 0; k < kRows; ++k)
-                    if (loc + k * kChunk < th.ts && c[k].i < I.n) I.labels[c[k].i] = c[k].lab;
-            }
-            if (total > 0) {
-                int64_t slot = S.h.qband + (int64_t)base;
-                if (slot + total > P.q_cap) {           // corrupt rows only
-                    if (lane == 0) raise_err(P.err, kErrIndex);
-                    // step (iii) reads every slot up to the queue's end
-                    for (int64_t e = slot + lane; e < P.q_cap; e += 32) {
-                        P.q[e] = make_int2(0, 0);
-                        if (kBatched) P.qk[e] = th.k;
-                    }
-                } else if (fast) {
-                    init_emit_rows<kBatched>(P, S, th, q, slot + (incl - rr), rr);
-                } else {
-                    slot += incl - rr;
-#pragma unroll
-                    for (int k = 0; k < kRows; ++k) {
-                        if (c[k].r > 0) init_emit_chunk<kBatched, kGen>(P, S, I, c[k], slot);
-                        slot += c[k].r;
-                    }
+                // chunk by chunk, in one copy of the code: a call of few tiles runs it
+                // from a cold instruction cache (a whole call of honeycomb 256^2 at
+                // 1.2 p_c with four copies 41 us, 38 so; registers 90, 61 so)
+#pragma unroll 1
+                for (int k = 0; k < kRows && loc + k * kChunk < th.ts; ++k) {
+                    ChunkRes c;
+                    init_scan_chunk<kGen>(P, S, I, warp * kRows + k, lane, tc, c);
+                    int64_t slot;
+                    int total;
+                    const int before = take_slots(S, bands, lane, c.r, slot, total);
+                    if (c.i < I.n) I.labels[c.i] = c.lab;
+                    if (total > 0 && slots_fit<kBatched>(P, th.k, slot, total, lane) && c.r > 0)
+                        init_emit_chunk<kBatched, kGen>(P, S, I, tc, c, slot + before);
                 }
             }
         }

@@ -238,3 +238,23 @@ def test_full_stage(shift, mixed):
         assert np.array_equal(got[so[k]:so[k + 1]], oracle.uf_label(x)), k
     assert np.array_equal(gpu_label(c, lats[1]), oracle.uf_label(lats[1]))
     ccl.ccl_context_destroy(c)
+
+
+@pytest.mark.parametrize("degree", [7, 9, 15, 16, 17, 31, 32, 33, 40, 41, 65])
+def test_long_rows_in_blocks(ctx, degree):
+    """Rows scanned in blocks of eight, around the blocks' ends and the 32 entries of
+    the residual mask: in a stage (few rows) and too many for it, alone and mixed
+    with short rows, with bits from memory and drawn."""
+    for n, mixed in ((70, False), (1300, False), (1300, True)):
+        rng = np.random.default_rng(degree + n)
+        deg = np.where(rng.random(n) < 0.7, rng.integers(0, 4, n), degree) if mixed else np.full(n, degree)
+        for p in (0.05, 0.5, 1.0):
+            lat = _graph(n, deg, p, degree + n)
+            assert np.array_equal(gpu_label(ctx, lat), oracle.uf_label(lat))
+            assert ccl.ccl_get_stats(ctx).residual_pairs == oracle.steps_label(lat)["n_residual"]
+        rp, ci = torch.from_numpy(lat.row_ptr).to(DEV), torch.from_numpy(lat.col_idx).to(DEV)
+        out = torch.full((n,), -1, dtype=torch.int32, device=DEV)
+        assert ccl.ccl_label_random(ctx, n, lat.nnz, rp, ci, 99, 0.2, out) == ccl.CCL_OK
+        assert ccl.ccl_sync(ctx) == ccl.CCL_OK
+        drawn = L.Lattice("random", n, lat.nnz, lat.row_ptr, lat.col_idx, oracle.keyed_bits(lat, 99, 0.2), 0.2, 0)
+        assert np.array_equal(out.cpu().numpy(), oracle.uf_label(drawn))
