@@ -117,7 +117,7 @@ struct ccl_context {
 namespace {
 
 constexpr size_t kMaxGraphs = 16;
-constexpr int kCounters = 4;           // statistics
+constexpr int kCounters = 5;           // statistics (4), whether the sample found long chains
 constexpr uint64_t kNoGen = ~0ull;     // Params::gen_thr of calls that read open_bits
 constexpr int64_t kProfRing = 4096;
 
@@ -510,6 +510,7 @@ ccl_status enqueue_tail(ccl_context *ctx, const Params &P0, bool batched, const 
                            g, (unsigned)T, smem, s, chain, A);
     };
     const int pre = resolve_pre(tc, P);
+    if (pre < 0 && !batched && short_walk && kChunk * P.n_chunks > kDeepSites) P.deep = (int32_t *)(ctx->d_counters + 4);
     if (pre != 0) CCL_CUDA(analysis(pre < 0));
     if (profile) CCL_CUDA(cudaEventRecord(ctx->ev[2], s));
     auto reduce = k_reduce<false, true, false>;

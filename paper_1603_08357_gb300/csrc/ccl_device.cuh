@@ -887,6 +887,10 @@ constexpr int kSampleRoots = 8, kSampleChunks = 12;
 // honeycomb 64^2 27 and 26, triangle 512^2 38 and 39). From a million sites on the
 // walk costs more at p_c than it gives (triangle 1024^2 52 and 55).
 constexpr int64_t kWalkSites = 1 << 18;
+// Instances of more than kDeepSites sites of whose sample fewer than one in
+// kDeepRoots is a root: see drain_deep.
+constexpr int64_t kDeepSites = 1 << 21;
+constexpr int kDeepRoots = 18;
 template <bool kBatched, bool kPark, bool kSample = false>
 __global__ void __launch_bounds__(512, 4) k_analysis(Params P) {
     extern __shared__ int s_park[];                  // kPark: site and label of kParkCap chains per warp
@@ -937,6 +941,7 @@ __global__ void __launch_bounds__(512, 4) k_analysis(Params P) {
             roots += __popc(__ballot_sync(kFull, i < n && lab[min(i, n - 1)] == i));
             sites += __popc(__ballot_sync(kFull, i < n));
         }
+        if (!kBatched && P.deep && wid == 0 && lane == 0) *P.deep = roots * kDeepRoots < sites;
         return roots * kSampleRoots < sites;
     };
     bool walk = kSample && !kBatched && sample();
@@ -1402,6 +1407,88 @@ __global__ void __launch_bounds__(kRedThreads, !kBatched ? 5 : kFar ? 4 : 3) k_r
 #endif
 }
 
+// A window of k_reduce_park where the sample found chains so long that most pairs
+// would be set aside: k_reduce's slots, three a lane, which walk only the larger
+// node of a pair and so load half as much. Two walks at once / three slots (slots in
+// k_reduce, as before there were short walks): honeycomb 1448^2 at 1.42 and 1.5 p_c
+// 133 / 116 (124) and 140 / 111 (122) us a call, 2048^2 at 1.5 p_c 231 / 192 (205).
+// The line: honeycomb 2400^2 at 1.36 p_c, one root in 16, takes 228 / 244, at 1.42,
+// one in 26, 243 / 250 and 1750^2 there 157 / 148. Below 2M sites (1024^2 at 1.5 p_c
+// 96) the caches hide the loads.
+struct DeepCount {
+    unsigned long long hops, atom, iter;        // (CCL_DEVICE_STATS)
+};
+__device__ __forceinline__ void drain_deep(const Params &P, const RedWindow &win, int lane, int32_t *labels,
+                                           DeepCount &n) {
+    constexpr int kSlots = 3;
+    const uint32_t table = P.link_mode > 0 ? kRedNextLink1 : kRedNextLink0;
+    const long long cap = red_round_cap(P, win.len);
+    long long rounds = 0;
+    int pnext = lane;
+    int2 pf = make_int2(0, 0);
+    bool pf_ok = false;
+    const auto fetch = [&]() {
+        pf = win.q[pnext];
+        pf_ok = true;
+        pnext += 32;
+    };
+    if (pnext < win.len) fetch();
+    int32_t a[kSlots], b[kSlots], st[kSlots];
+#pragma unroll
+    for (int u = 0; u < kSlots; ++u) {
+        st[u] = kTaskDone;
+        a[u] = b[u] = 0;
+    }
+    for (;;) {
+        int take = -1;          // at most one empty slot per lane and round takes the prefetched pair
+#pragma unroll
+        for (int u = kSlots - 1; u >= 0; --u)
+            if (st[u] == kTaskDone) take = u;
+        if (take >= 0 && pf_ok) {
+            const int32_t na = max(pf.x, pf.y), nb = min(pf.x, pf.y);
+#pragma unroll
+            for (int u = 0; u < kSlots; ++u)
+                if (u == take) {
+                    a[u] = na;
+                    b[u] = nb;
+                    st[u] = kTaskChase;
+                }
+            pf_ok = false;
+            if (pnext < win.len) fetch();
+        }
+        int32_t v[kSlots];
+#pragma unroll
+        for (int u = 0; u < kSlots; ++u) {
+            int32_t *at = labels + (st[u] == kTaskRoot ? b[u] : a[u]);
+            v[u] = 0;
+            if (st[u] == kTaskMerge) v[u] = atomicMin(at, b[u]);
+            else if (st[u] != kTaskDone) v[u] = red_load(at);
+        }
+        bool any = false;       // the transitions of k_reduce
+#pragma unroll
+        for (int u = 0; u < kSlots; ++u) {
+            const int32_t y = v[u], A = a[u], B = b[u], s = st[u];
+#ifdef CCL_DEVICE_STATS
+            n.hops += (s == kTaskChase || s == kTaskRoot);
+            n.atom += (s == kTaskMerge);
+#endif
+            const uint32_t idx = ((uint32_t)s << 2) | ((y == A) ? 2u : 0u) | ((y == B) ? 1u : 0u);
+            a[u] = s == kTaskRoot ? A : max(y, B);
+            b[u] = min(y, B);
+            st[u] = (int32_t)((table >> (2u * idx)) & 3u);
+            any |= st[u] != kTaskDone;
+        }
+#ifdef CCL_DEVICE_STATS
+        n.iter++;
+#endif
+        if (!__any_sync(kFull, any || pf_ok)) break;
+        if (++rounds > cap) {
+            raise_err(P.err, kErrNonconv);
+            break;
+        }
+    }
+}
+
 // Step (iii) for calls whose labels take at most three eighths of L2: two pairs
 // a lane start together
 // with their warp and run a fixed number of steps, both ends of a pair walking
@@ -1433,6 +1520,7 @@ __global__ void __launch_bounds__(kRedThreads, kBatched ? 6 : 8) k_reduce_park(P
     long long total;
     const long long nwin = red_windows(P, s_win, s_warp, lane, nwarps, total);
     const unsigned latched = kBatched ? __ldcg(P.err) : 0u;
+    const bool deep = !kBatched && P.deep && __ldcg(P.deep);
     const bool eager = P.link_mode > 0;            // link a root to the other end's node, not its root
     // the labels of the lane's last instance
     int lk = -1;
@@ -1475,6 +1563,16 @@ __global__ void __launch_bounds__(kRedThreads, kBatched ? 6 : 8) k_reduce_park(P
     for (long long w = (long long)blockIdx.x * (kRedThreads / 32) + warp; w < nwin; w += nwarps) {
         const RedWindow win = red_window<kBatched>(P, s_win, (uint32_t)w);
         if (kBatched && latched) check_window(P, win, lane);
+        if (!kBatched && deep) {
+            DeepCount n{0, 0, 0};
+            drain_deep(P, win, lane, P.one.labels, n);
+#ifdef CCL_DEVICE_STATS
+            st_hops += n.hops;
+            st_atom += n.atom;
+            st_iter += n.iter;
+#endif
+            continue;
+        }
         const int round_cap = (int)min(red_round_cap(P, win.len), (long long)INT32_MAX - 3);
         int rounds = 0;
         int cnt = 0;                // pairs set aside; below 32 whenever pairs are added

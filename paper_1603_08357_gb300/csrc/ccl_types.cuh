@@ -86,6 +86,7 @@ struct Params {
                                // before a launch in rounds)
     int64_t tile_off;          // step (i) on part of the tiles: its first tile ...
     int32_t band_off;          // ... and its first band record
+    int32_t *deep;             // large single instances: set by the sample where chains are long, read by step (iii)
     int32_t more_pairs;        // 1: the pairs of this step (iii) add to counters[0], 0: they replace it
     int32_t iter_cap;          // > 0: steps (ii)-(iv) give up after this many iterations (test option)
     int32_t red_window;        // step (iii): most pairs per warp window (0: kRedWindowMax)

@@ -258,3 +258,20 @@ def test_long_rows_in_blocks(ctx, degree):
         assert ccl.ccl_sync(ctx) == ccl.CCL_OK
         drawn = L.Lattice("random", n, lat.nnz, lat.row_ptr, lat.col_idx, oracle.keyed_bits(lat, 99, 0.2), 0.2, 0)
         assert np.array_equal(out.cpu().numpy(), oracle.uf_label(drawn))
+
+
+@pytest.mark.parametrize("link", [-1, 0, 1])
+def test_deep_windows(link):
+    """Calls of more than 2^21 sites whose sample finds long chains (honeycomb from
+    1.4 p_c on) drain their windows in slots; the choice is made anew by each call."""
+    c = ccl.ccl_context_create(0)
+    try:
+        assert ccl.ccl_set_option(c, ccl.CCL_OPT_LINK_MODE, link) == ccl.CCL_OK
+        lats = [L.honeycomb(1030, r * L.PC_HONEYCOMB, 5) for r in (1.5, 1.0, 1.42)]
+        assert lats[0].n > 1 << 21
+        for graphs in (1, 0):
+            assert ccl.ccl_set_option(c, ccl.CCL_OPT_USE_GRAPHS, graphs) == ccl.CCL_OK
+            for lat in lats:
+                assert np.array_equal(gpu_label(c, lat), oracle.uf_label(lat))
+    finally:
+        ccl.ccl_context_destroy(c)
