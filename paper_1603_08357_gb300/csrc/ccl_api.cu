@@ -1263,9 +1263,9 @@ ccl_status ensure_aux(ccl_context *ctx, int64_t bytes) {
 
 namespace {
 // CTAs of 256 threads of the kernels that give every warp one run of 128-site
-// groups (warp_run): all the SM's warps, fewer for short inputs.
-int64_t run_grid(const ccl_context *ctx, int64_t n) {
-    return std::max<int64_t>(1, std::min<int64_t>((int64_t)ctx->num_sms * 8, (n + 1023) / 1024));
+// groups (warp_run): as many as an SM holds, fewer for short inputs.
+int64_t run_grid(const ccl_context *ctx, int64_t n, int per_sm) {
+    return std::max<int64_t>(1, std::min<int64_t>((int64_t)ctx->num_sms * per_sm, (n + 1023) / 1024));
 }
 }  // namespace
 
@@ -1286,7 +1286,7 @@ ccl_status ccl_relabel(ccl_context *ctx, int32_t n, const int32_t *labels, int32
     k_root_counts<<<(unsigned)nb, kRelThreads, 0, s>>>(n, labels, cnt, seq);
     k_scan_counts<<<1, 1024, 0, s>>>((int32_t)nb, cnt, n_clusters);
     k_root_ids<<<(unsigned)nb, kRelThreads, 0, s>>>(n, cnt, seq, sizes);
-    k_site_ids<<<(unsigned)run_grid(ctx, n), 256, 0, s>>>(n, labels, seq, sizes);
+    k_site_ids<<<(unsigned)run_grid(ctx, n, 8), 256, 0, s>>>(n, labels, seq, sizes);
     CCL_CUDA(cudaGetLastError());
     return CCL_OK;
 }
@@ -1332,7 +1332,7 @@ ccl_status ccl_largest_cluster(ccl_context *ctx, int32_t n, const int32_t *label
     LargestScratch *scratch = (LargestScratch *)ctx->d_aux;
     int32_t *cnt = (int32_t *)(scratch + 1);
     CCL_CUDA(cudaMemsetAsync(ctx->d_aux, 0, sizeof(LargestScratch) + (size_t)n * sizeof(int32_t), s));
-    k_largest<<<(unsigned)run_grid(ctx, n), 256, 0, s>>>(n, labels, cnt, scratch, result, ctx->d_err);
+    k_largest<<<(unsigned)run_grid(ctx, n, kLargestCtas), 256, 0, s>>>(n, labels, cnt, scratch, result, ctx->d_err);
     CCL_CUDA(cudaGetLastError());
     return CCL_OK;
 }
