@@ -13,9 +13,10 @@
 // pairs from the start of that range and records their count in band[b], so
 // steps (ii)-(iv) run unchanged.
 //
-// Layout: for one k the 32 lanes of a warp (32 consecutive sites) read 32
-// consecutive ints of nn and at most two bit words, so every load is a
-// coalesced 128-byte line; no shared-memory staging is needed.
+// Two kernels: lists of at most kRowRegs slots go through shared memory
+// (k_init_dense_tma below), wider ones are read in place (k_init_dense): for one k
+// the 32 lanes of a warp (32 consecutive sites) read 32 consecutive ints of nn and
+// at most two bit words, so every load is a coalesced 128-byte line.
 #pragma once
 #include <stdint.h>
 #include <cuda_runtime.h>
@@ -72,7 +73,6 @@ __global__ void __launch_bounds__(kDenseThreads) k_init_dense(Params P) {
     cta_band(P, band_lo, band_hi);
     const int64_t n = P.one.n;
     const int W = (int)P.nn_width;
-    const int64_t n_words = ((int64_t)W * n + 31) >> 5;
     const int64_t s_lo = min(band_lo * kTileSites, n), s_hi = min(band_hi * kTileSites, n);
     const int64_t qband = s_lo * W;
     if (threadIdx.x == 0) {
@@ -84,93 +84,32 @@ __global__ void __launch_bounds__(kDenseThreads) k_init_dense(Params P) {
     const int warp = threadIdx.x >> 5;
     bool bad = false;
     for (int64_t t0 = s_lo; t0 < s_hi; t0 += kDenseSpan) {
-        if (W <= kRowRegs) {
-            // Every load of the step is issued before any is used: lane i's
-            // slots, and the chunk's bit words. Chunk c0 (a multiple of 32)
-            // has the bits of slot k in the 64 bits from word (c0 + k*n) >> 5
-            // on: lane k holds that word, lane 8 + k the next one.
-            int32_t jr[kDenseChunks][kRowRegs];
-            uint32_t wl[kDenseChunks];
-#pragma unroll
-            for (int c = 0; c < kDenseChunks; ++c) {
-                const int64_t c0 = t0 + (int64_t)(warp * kDenseChunks + c) * kChunk;
-                const int64_t i64 = c0 + lane;
-                const bool live = i64 < s_hi;
-#pragma unroll
-                for (int k = 0; k < kRowRegs; ++k)
-                    jr[c][k] = (live && k < W) ? __ldcs(P.nn + i64 + k * n) : -1;
-                wl[c] = 0;
-                if (!kGen) {
-                    const int kk = lane & 7;
-                    const int64_t w = ((c0 + (int64_t)kk * n) >> 5) + (lane >> 3);
-                    if (lane < 16 && kk < W && c0 < s_hi && w < n_words) wl[c] = __ldg(P.one.bits + w);
-                }
-            }
-#pragma unroll
-            for (int c = 0; c < kDenseChunks; ++c) {
-                const int64_t c0 = t0 + (int64_t)(warp * kDenseChunks + c) * kChunk;
-                if (c0 >= s_hi) break;
-                const int64_t i64 = c0 + lane;
-                const int32_t i = (int32_t)i64;
-                int32_t m = INT32_MAX, mk = 0;
-                uint32_t lowmask = 0;
-#pragma unroll
-                for (int k = 0; k < kRowRegs; ++k) {
-                    bool open;
-                    const int32_t j = jr[c][k];
-                    if (kGen) {
-                        open = j >= 0 && j < i && gen_bond_open(P.gen_seed, P.gen_thr, (uint32_t)j, (uint32_t)i);
-                    } else {
-                        const uint32_t lo = __shfl_sync(kFull, wl[c], k);
-                        const uint32_t hi = __shfl_sync(kFull, wl[c], 8 + k);
-                        const uint32_t win = __funnelshift_r(lo, hi, (uint32_t)((c0 + (int64_t)k * n) & 31));
-                        open = j >= 0 && j < i && ((win >> lane) & 1u);
-                    }
+        for (int c = 0; c < kDenseChunks; ++c) {
+            const int64_t c0 = t0 + (int64_t)(warp * kDenseChunks + c) * kChunk;
+            if (c0 >= s_hi) break;
+            const int64_t i64 = c0 + lane;
+            const bool live = i64 < s_hi;
+            const int32_t i = (int32_t)i64;
+            int32_t m = INT32_MAX, mk = -1, cnt = 0;
+            if (live) {
+                for (int k = 0; k < W; ++k) {
+                    const int64_t e = i64 + (int64_t)k * n;
+                    const int32_t j = __ldg(P.nn + e);
                     bad |= j < -1 || (int64_t)j >= n;
-                    if (open) {
-                        lowmask |= 1u << k;
+                    if (j >= 0 && j < i && dense_open<kGen>(P, e, i, j)) {
+                        ++cnt;
                         if (j < m) { m = j; mk = k; }
                     }
                 }
-                const int cnt = __popc(lowmask);
-                if (i64 < s_hi) P.one.labels[i] = dense_label(P, i, m, cnt, s_lo, t0);
-                const int r = cnt > 1 ? cnt - 1 : 0;
-                int64_t slot = dense_emit_slot(qband, &band_cnt, lane, r);
-                if (r > 0) {
-                    const uint32_t rm = lowmask & ~(1u << mk);
-#pragma unroll
-                    for (int k = 0; k < kRowRegs; ++k)
-                        if ((rm >> k) & 1u) P.q[slot++] = make_int2(i, jr[c][k]);
-                }
+                P.one.labels[i] = dense_label(P, i, m, cnt, s_lo, t0);
             }
-        } else {
-            for (int c = 0; c < kDenseChunks; ++c) {
-                const int64_t c0 = t0 + (int64_t)(warp * kDenseChunks + c) * kChunk;
-                if (c0 >= s_hi) break;
-                const int64_t i64 = c0 + lane;
-                const bool live = i64 < s_hi;
-                const int32_t i = (int32_t)i64;
-                int32_t m = INT32_MAX, mk = -1, cnt = 0;
-                if (live) {
-                    for (int k = 0; k < W; ++k) {
-                        const int64_t e = i64 + (int64_t)k * n;
-                        const int32_t j = __ldg(P.nn + e);
-                        bad |= j < -1 || (int64_t)j >= n;
-                        if (j >= 0 && j < i && dense_open<kGen>(P, e, i, j)) {
-                            ++cnt;
-                            if (j < m) { m = j; mk = k; }
-                        }
-                    }
-                    P.one.labels[i] = dense_label(P, i, m, cnt, s_lo, t0);
-                }
-                const int r = cnt > 1 ? cnt - 1 : 0;
-                int64_t slot = dense_emit_slot(qband, &band_cnt, lane, r);
-                if (r > 0) {
-                    for (int k = 0; k < W; ++k) {
-                        const int64_t e = i64 + (int64_t)k * n;
-                        const int32_t j = __ldg(P.nn + e);
-                        if (k != mk && j >= 0 && j < i && dense_open<kGen>(P, e, i, j)) P.q[slot++] = make_int2(i, j);
-                    }
+            const int r = cnt > 1 ? cnt - 1 : 0;
+            int64_t slot = dense_emit_slot(qband, &band_cnt, lane, r);
+            if (r > 0) {
+                for (int k = 0; k < W; ++k) {
+                    const int64_t e = i64 + (int64_t)k * n;
+                    const int32_t j = __ldg(P.nn + e);
+                    if (k != mk && j >= 0 && j < i && dense_open<kGen>(P, e, i, j)) P.q[slot++] = make_int2(i, j);
                 }
             }
         }
