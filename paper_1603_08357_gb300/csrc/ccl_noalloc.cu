@@ -142,7 +142,8 @@ extern "C" ccl_status ccl_label_noalloc(int32_t n, int64_t nnz, const int32_t *r
     P.round_per[0] = (int32_t)per;
     const int64_t ana_warps = (P.n_chunks + kAnaChunks - 1) / kAnaChunks;
     const int64_t g_ana = std::max<int64_t>(1, std::min<int64_t>((int64_t)d->num_sms * d->ana_per_sm, (ana_warps + 7) / 8));
-    const int64_t g_red = (int64_t)d->num_sms * d->red_per_sm;
+    // no more warps than windows of 64 pairs, a pair per entry at most (as in ccl_label)
+    const int64_t g_red = std::min<int64_t>((int64_t)d->num_sms * d->red_per_sm, nnz / (64 * kRedThreads / 32) + 1);
 
     // the array keeps the previous call's contents: clear the error word (step
     // (i) writes every band record, step (iii) the pair count)
