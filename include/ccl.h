@@ -119,8 +119,8 @@ typedef enum {
                                   For testing the failure path; setting it drops cached graphs. */
     CCL_OPT_REDUCE_WINDOW = 9, /* step (iii): most residual pairs a warp drains per window
                                   (64..65536); 0 (default): 2048 when the call's labels fit in
-                                  three quarters of L2, else 1024 (512 for instances whose
-                                  labels lie far apart) */
+                                  three quarters of L2, else 1024 (512 for batches whose
+                                  labels span more than 2^32 sites) */
     CCL_OPT_ANALYSIS_GROUP = 10, /* steps (ii)/(iv) in contiguous order: G > 0 visits the sites in
                                   super-chunks, every warp taking its next G groups of 96 sites
                                   of each, so the labels in use stay in L2; 0 one range per

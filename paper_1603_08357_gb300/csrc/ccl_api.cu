@@ -348,14 +348,12 @@ int64_t init_grid(ccl_context *ctx, const Params &P, bool batched, int64_t max_b
 // for batches of many tiles, kRounds rounds of bands that shrink by 30 % a
 // round. The instances of a batch differ in cost per tile (a randomly numbered
 // tree of coordination 6 against a lattice), and with one band per CTA the SMs
-// were idle for a quarter of step (i); handed out as CTAs become free, 1024
-// mixed instances take 3.38 ms instead of 4.85 (eight rounds shrinking by
-// 40 %: 3.70; twelve equal rounds: 3.50; step (iii) takes 2.53 instead of 2.37
-// ms, the labels reach fewer tiles back). A single instance costs the same
-// everywhere and keeps one band per CTA: with rounds triangle 16384^2 gains
-// 0.07 ms in step (i) and loses 0.2 in step (iii). Below 64 tiles a CTA a
-// round's bands are so short that fetching the ticket shows (256 small
-// instances: 39 us with one band per CTA, 53 with bands of 8 tiles).
+// were idle for a quarter of step (i): handed out as CTAs become free, 1024 mixed
+// instances take 3.38 ms instead of 4.85 (step (iii) 2.53 instead of 2.37, the
+// labels reach fewer tiles back). A single instance costs the same everywhere and
+// keeps one band per CTA (triangle 16384^2 would gain 0.07 ms in step (i) and lose
+// 0.2 in step (iii)). Below 64 tiles a CTA a round's bands are so short that
+// fetching the ticket shows (256 small instances 39 us, 53 in rounds).
 constexpr int64_t kRoundTiles = 64;
 void split_bands(Params &P, int64_t g, bool batched) {
     P.init_bands = (int32_t)g;
@@ -401,8 +399,8 @@ ccl_status launch_init(const Params &P, bool batched, int64_t g, cudaStream_t s)
 // gather hits L2 anyway), else windows of at most 1024 pairs and super-chunks of
 // 16 chunk groups per warp, so the labels the warps touch at once stay in L2.
 // (Windows of 512 / 1024 / 2048 pairs: triangle 16384^2 1.41 / 1.17 / 1.59 ms,
-// 1024 mixed instances 2.76 / 2.24 / 3.0; with instances far apart, six slots,
-// 2.53 / 2.73 / 3.76.)
+// 1024 mixed instances 2.76 / 2.24 / 3.0; in six slots of addresses, the form of
+// batches whose labels span more than 2^32 sites, 2.53 / 2.73 / 3.76.)
 bool batched_far(const Params &P) { return P.K > 1 && !P.lab_base; }
 
 bool labels_fit_l2(const ccl_context *ctx, const Params &P) {

@@ -9,13 +9,16 @@
 //    bulk asynchronous copies (cp.async.bulk, completion on mbarriers, a ring
 //    of kStages stages); kInitConsumers consumer warps scan the rows (four
 //    chunks per warp and tile, one row of each per lane, interleaved), write
-//    the labels and append the residual pairs to their CTA's part of the
-//    queue through one prefix sum per warp and tile. Each CTA owns a contiguous band of tiles; a site whose
-//    smallest lower neighbour lies in a band tile finished kStages tiles
-//    earlier takes that neighbour's label (most of step (ii) on lattices).
+//    the labels and append the residual pairs to their band's part of the
+//    queue through one prefix sum per warp and tile. A CTA works through
+//    contiguous bands of tiles, one or, in large batches, up to kRounds; a
+//    site whose smallest lower neighbour lies in a tile of the band finished
+//    kStages tiles earlier takes that neighbour's label (most of step (ii) on
+//    lattices).
 //  * Step (iii) runs Algorithm 1 over the queue: each warp drains a window of
-//    pairs with six or eight pairs per lane in lockstep rounds (one load
-//    or atomicMin per live pair per round, next state from a small table).
+//    pairs, by short walks of two pairs a lane (labels of at most 3/8 of L2) or
+//    with six or eight pairs per lane in lockstep rounds (one load or atomicMin
+//    per live pair per round, next state from a small table).
 //  * Steps (ii)/(iv) chase every site's chain to its root, three chains per
 //    lane at once, each warp over contiguous runs of sites (or interleaved,
 //    for inputs without locality).
@@ -487,23 +490,16 @@ struct RowsRes {
 // overlap.
 //
 // Step (i) is bound by the instructions of this scan (the integer pipe), not
-// by memory, until rows are cheap. Four rows a lane with eight warps a CTA
-// against two rows with sixteen: the tile's header, the prefix sum and the
-// queue bookkeeping are paid once for 128 sites instead of 64; rows of one
-// degree need no row ends, no per-entry tests of the row's length and half
-// the loads (the rows of a lane lie 32 apart, so 8-byte loads of degree 4 and
-// 6 and 4-byte loads of degree 3 spread over the banks); keys find the
-// smallest neighbour and its place with one minimum. Warp instructions per 64
-// sites on triangle 3000^2: 537 -> 308. Times of step (i), before -> after:
-// triangle 4096^2 160 -> 118 us (4.6 TB/s; streaming alone takes 88),
-// triangle 16384^2 2.44 -> 1.80 ms, honeycomb 2048^2 71 -> 55 us, Bethe
-// lattice of 24 shells 390 -> 364 us, and 325 with the mixed rows' entries past
-// a row's end read and masked instead of branched around (1024 mixed instances
-// 3.39 -> 3.15 ms by that alone).
-// (Two rows a lane and sixteen warps with the same scan: 140 us on triangle
-// 4096^2; two stages and three CTAs per SM: 124 us there, 347 us on the Bethe
-// lattice.) A call of few tiles pays for the longer lanes: honeycomb 64^2
-// 8.4 -> 9.5 us.
+// by memory, until rows are cheap. With four rows a lane the tile's header, the
+// prefix sum and the queue bookkeeping are paid once for 128 sites; rows of one
+// degree need no row ends, no per-entry tests of the row's length and half the
+// loads (the rows of a lane lie 32 apart, so 8-byte loads of degree 4 and 6 and
+// 4-byte loads of degree 3 spread over the banks); keys find the smallest
+// neighbour and its place with one minimum; mixed rows read past their ends and
+// mask instead of branching. Against two rows a lane entry by entry, step (i) of
+// triangle 4096^2 160 -> 116 us (5.0 TB/s; streaming alone takes 88), of the Bethe
+// lattice of 24 shells 390 -> 318; a call of few tiles pays 1 us for the longer
+// lanes (honeycomb 64^2).
 template <bool kGen, int kD, bool kWide = false>
 __device__ __forceinline__ void scan_rows(const Params &P, const Stage &S, const TileCtx &tc, const TileHdr &h,
                                           int32_t n, int32_t s00, int lane, const int32_t (&a)[kRows],
@@ -850,13 +846,11 @@ __global__ void __launch_bounds__(kInitThreads, kInitCtas) k_init(Params P) {
 // latency and the instructions around them, so a run is cut into stretches of
 // one instance with 32-bit site numbers, and a round is a load, a compare and
 // a move per chain. Against the same walk with the instance, 64-bit chunk
-// numbers and caps looked at for every chunk (94 to 108 warp instructions per
-// chunk): 1024 mixed instances 2.54 -> 1.24 ms, triangle 16384^2 1.16 -> 0.67 ms,
-// triangle 4096^2 66 -> 47.5 us (2.8 TB/s of its 8 bytes per site), honeycomb
-// 2048^2 39 -> 28.5 us, 256 small instances 28.6 -> 16.5 us, Bethe lattice of
-// 24 shells 287 -> 282 us (random gathers over 201 MB). Three chunks a group
-// beat two (870 us on triangle 16384^2) and four (790), two rounds between
-// votes beat one (700) and equal three; 256 threads of 32 registers fill the SM.
+// numbers and caps looked at for every chunk: 1024 mixed instances 2.54 -> 1.23 ms,
+// triangle 4096^2 66 -> 47 us (2.8 TB/s of its 8 bytes per site); a Bethe lattice's
+// random gathers over 201 MB hardly gain. Three chunks a group beat two and four
+// (0.67 ms on triangle 16384^2, 0.87, 0.79), two rounds between votes beat one;
+// 256 threads of 32 registers fill the SM.
 constexpr int kAnaRounds = 4;                        // rounds before a chain is set aside (kPark)
 constexpr int kParkCap = 32 * kAnaChunks + 32;       // < 32 left + one group's chains
 
@@ -872,13 +866,11 @@ constexpr int kParkCap = 32 * kAnaChunks + 32;       // < 32 left + one group's 
 // alike). A chain ends at each hop with about that probability: where roots
 // are common chains are a few hops long and step (iii) does better alone, where
 // they are rare each of its pairs would walk a long chain. Calls without / with
-// the pass, and by sample: honeycomb 362^2 at 1.5 p_c 109 / 45 / 44 us, 1448^2
-// there 233 / 140 / 143, 2896^2 581 / 308 / 302, square 2048^2 200 / 131 / 134,
-// triangle 2048^2 156 / 124 / 126; at p_c, left alone, it costs its launch and
-// one read: triangle 4096^2 250 / 279 / 254, honeycomb 256^2 33 / 36 / 36. The
-// line lies at 0.125: triangles at 1.5 p_c (0.11) and honeycomb lattices at 1.2
-// p_c (0.13) are about even. Deciding per stretch of 96 sites instead costs
-// more than either at the line (triangle 2048^2 at 1.5 p_c 173).
+// the pass, and by sample: honeycomb 2896^2 at 1.5 p_c 581 / 308 / 302 us, triangle
+// 2048^2 155 / 122 / 124; at p_c, left alone, it costs its launch and one read:
+// triangle 4096^2 250 / 279 / 254. The line lies at 0.125: triangles at 1.5 p_c
+// (0.11) and honeycomb lattices at 1.2 p_c (0.13) are about even. Deciding per
+// stretch of 96 sites instead costs more than either (triangle 2048^2 173).
 constexpr int kSampleRoots = 8, kSampleChunks = 12;
 // Calls of at most this many sites are walked without a sample. They are launches
 // and latency: the walk costs them what the sample does, and mends the inputs the

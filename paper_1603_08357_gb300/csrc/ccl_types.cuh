@@ -27,7 +27,7 @@ constexpr int kRowRegs = 8;                // rows up to this degree are scanned
 
 constexpr int kAnaChunks = 3;              // steps (ii)/(iv): chunks a warp walks at once
 
-// step (iii): pairs a warp drains per window; most step-(i) CTAs' bands
+// step (iii): pairs a warp drains per window; most bands of a call
 constexpr int kRedWindowMax = 2048;   // default most pairs per warp window (fewer for small queues)
 constexpr int kMaxBands = 4096;
 constexpr int kRounds = 12;           // most bands a CTA of step (i) takes
@@ -55,7 +55,7 @@ struct Inst {
     int32_t nnz;
 };
 
-// Residual pairs of one step-(i) CTA: they are packed from queue slot qbase
+// Residual pairs of one band of step (i): they are packed from queue slot qbase
 // on (inside the slot range of the band's CSR entries, so bands never overlap).
 struct __align__(16) BandRec {
     int64_t qbase;
@@ -70,7 +70,7 @@ struct Params {
     int32_t link_mode;         // step (iii): 0 root to root, 1 root to the other chain's node, -1 by window
     int64_t n_chunks;          // over all instances
     int64_t n_tiles;           // over all instances
-    int32_t n_bands;           // CTAs of step (i)
+    int32_t n_bands;           // bands of step (i), over all its launches
     int32_t dense;             // 1: step (i) reads the dense neighbour list nn
     BandRec *band;             // [n_bands]
     int2 *q;                   // residual pairs (i, j); slots indexed by global CSR entry
