@@ -1708,7 +1708,7 @@ ccl_status ccl_autotune(ccl_context *ctx, int32_t n, int64_t nnz, const int32_t 
     float best_t = 1e30f;
     std::vector<TuneChoice> cands;
     for (int T : {128, 256, 512})
-        for (int pre = 0; pre < 2; ++pre)
+        for (int pre = 0; pre < 2; ++pre)       // (by sample: for one instance one of the two plus a launch)
             for (int lm : {-1, 1})
                 for (int rf = 0; rf < 2; ++rf)
                     for (int sq = 0; sq < 2; ++sq) {
