@@ -791,11 +791,15 @@ __global__ void __launch_bounds__(kInitThreads, kInitCtas) k_init(Params P) {
         if (loc < th.ts) {
             const int32_t s00 = th.s0 + loc;
             RowsRes q;
-            if (init_scan_rows<kGen>(P, S, I, s00, lane, tc, th, q)) {
-                const int rr = __popc(q.res);
-                int64_t slot;
-                int total;
-                const int before = take_slots(S, bands, lane, rr, slot, total);
+            // (both ways meet here before the slots are taken: with a prefix sum of its
+            // own behind the scan the labels' loads were waited for earlier, 3 % of step
+            // (i) beyond L2, triangle 16384^2 1845 us)
+            const bool fast = init_scan_rows<kGen>(P, S, I, s00, lane, tc, th, q);
+            const int rr = fast ? __popc(q.res) : 0;
+            int64_t slot;
+            int total;
+            const int before = take_slots(S, bands, lane, rr, slot, total);
+            if (fast) {
                 int32_t *out = I.labels + s00 + lane;
 #pragma unroll
                 for (int k = 0; k < kRows; ++k) out[kChunk * k] = q.lab[k];
@@ -804,13 +808,11 @@ __global__ void __launch_bounds__(kInitThreads, kInitCtas) k_init(Params P) {
             } else {
                 // chunk by chunk, in one copy of the code: a call of few tiles runs it
                 // from a cold instruction cache (a whole call of honeycomb 256^2 at
-                // 1.2 p_c with four copies 41 us, 38 so; registers 90, 61 so)
+                // 1.2 p_c with four copies 41 us, 38 so; registers 90, 70 so)
 #pragma unroll 1
                 for (int k = 0; k < kRows && loc + k * kChunk < th.ts; ++k) {
                     ChunkRes c;
                     init_scan_chunk<kGen>(P, S, I, warp * kRows + k, lane, tc, c);
-                    int64_t slot;
-                    int total;
                     const int before = take_slots(S, bands, lane, c.r, slot, total);
                     if (c.i < I.n) I.labels[c.i] = c.lab;
                     if (total > 0 && slots_fit<kBatched>(P, th.k, slot, total, lane) && c.r > 0)
