@@ -166,7 +166,9 @@ CCL_API ccl_status ccl_label(ccl_context *ctx, int32_t n_sites, int64_t nnz, con
  *   open_bits  DEVICE uint32: local entry e of instance k is global bit ent_off[k] + e
  *   labels     DEVICE int32[site_off[K]]: labels[site_off[k] + i] = instance-local label
  * Each instance needs n_k <= CCL_MAX_SITES and nnz_k < 2^31. Asynchronous on `stream`.
- * Repeated calls with the same arguments replay a captured CUDA graph.
+ * Repeated calls with the same arguments replay a captured CUDA graph. A call
+ * captured into a user's graph keeps its instance table (120 bytes an instance)
+ * on the device until the context is destroyed.
  */
 CCL_API ccl_status ccl_label_batched(ccl_context *ctx, int32_t n_inst, const int64_t *site_off,
                              const int64_t *ent_off, const int32_t *row_ptr,

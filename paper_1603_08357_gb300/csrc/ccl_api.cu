@@ -75,6 +75,9 @@ struct ccl_context {
     Inst *h_insts = nullptr;     // pinned staging
     int64_t h_insts_cap = 0;
     cudaEvent_t staging_free = nullptr;
+    // the tables of batched calls captured into a user's graph: its replays read
+    // them, so they stay as long as the context
+    std::vector<Inst *> captured_insts;
     // recorded after each labelling call (outside stream capture): statistics
     // reads wait for it instead of the whole device
     cudaEvent_t stats_ev = nullptr;
@@ -624,6 +627,26 @@ ccl_status upload_table(ccl_context *ctx, const std::vector<Inst> &table, cudaSt
     return CCL_OK;
 }
 
+// A device table of its own for a batched call under capture: by the time of a
+// replay the context's table and staging buffer are another call's, or freed to
+// grow, and an event recorded in a capture cannot be waited for outside. It is
+// allocated and filled now, on the context's own stream, not in the graph.
+ccl_status captured_table(ccl_context *ctx, const std::vector<Inst> &table, const Inst **out) {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;      // (of this thread, for these calls)
+    CCL_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
+    Inst *d = nullptr;
+    const size_t bytes = table.size() * sizeof(Inst);
+    cudaError_t e = cudaMalloc(&d, bytes);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(d, table.data(), bytes, cudaMemcpyHostToDevice, ctx->cap_stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->cap_stream);
+    if (e != cudaSuccess && d) cudaFree(d);
+    (void)cudaThreadExchangeStreamCaptureMode(&mode);
+    CCL_CUDA(e);
+    ctx->captured_insts.push_back(d);
+    *out = d;
+    return CCL_OK;
+}
+
 // The lowest labels of the instances if every instance's lie within 2^32 labels
 // of them (whole batches do: their labels are one array), else null.
 int32_t *label_base(const std::vector<Inst> &table) {
@@ -648,9 +671,9 @@ ccl_status run(ccl_context *ctx, Params P, bool batched, const TuneChoice &tc, c
     const bool capturing = stream_capturing(s);
     if (ctx->profile || !ctx->use_graphs || capturing || !allow_graph) {
         if (batched) {
-            ccl_status st = upload_table(ctx, *table, s);
+            ccl_status st = capturing ? captured_table(ctx, *table, &P.insts) : upload_table(ctx, *table, s);
             if (st != CCL_OK) return st;
-            P.insts = ctx->d_insts;
+            if (!capturing) P.insts = ctx->d_insts;
         }
         if (ctx->profile) {
             const size_t slot = (size_t)(ctx->prof_count % kProfRing);
@@ -982,6 +1005,7 @@ void ccl_context_destroy(ccl_context *ctx) {
     if (ctx->d_err) cudaFree(ctx->d_err);
     if (ctx->d_counters) cudaFree(ctx->d_counters);
     if (ctx->d_insts) cudaFree(ctx->d_insts);
+    for (Inst *d : ctx->captured_insts) cudaFree(d);
     if (ctx->h_insts) cudaFreeHost(ctx->h_insts);
     if (ctx->d_host_in) cudaFree(ctx->d_host_in);
     if (ctx->d_aux) cudaFree(ctx->d_aux);

@@ -275,3 +275,37 @@ def test_deep_windows(link):
                 assert np.array_equal(gpu_label(c, lat), oracle.uf_label(lat))
     finally:
         ccl.ccl_context_destroy(c)
+
+
+@pytest.mark.parametrize("before", [False, True])
+def test_batch_in_a_users_graph(before):
+    """A batched call captured into a user's graph, with and without an uncaptured
+    call before it: replays label its own instances after the context has labelled
+    other and larger batches, and those are labelled as ever."""
+    c = ccl.ccl_context_create(0)
+    a = L.make_batch([dict(kind="triangle", L=n, p=0.4, seed=n) for n in (30, 47, 128)])
+    others = [L.make_batch([dict(kind="square", L=5 + k % 9, p=0.5, seed=k) for k in range(K)]) for K in (3, 300)]
+    rp, ci, bits = (torch.from_numpy(x).to(DEV) for x in (a.row_ptr, a.col_idx, a.open_bits.view(np.int32)))
+    out = torch.full((a.n_total,), -7, dtype=torch.int32, device=DEV)
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    assert ccl.ccl_reserve(c, 0, 4 * a.nnz_total, 0) == ccl.CCL_OK
+    if before:
+        assert ccl.ccl_label_batched(c, a.k, a.site_off, a.ent_off, rp, ci, bits, out, s) == ccl.CCL_OK
+        assert ccl.ccl_sync(c, s) == ccl.CCL_OK
+    else:                                       # (loads the kernels)
+        assert np.array_equal(gpu_label_batched(c, others[0]), oracle.uf_label_batched(others[0]))
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        assert ccl.ccl_label_batched(c, a.k, a.site_off, a.ent_off, rp, ci, bits, out, s) == ccl.CCL_OK
+    want = oracle.uf_label_batched(a)
+    for graphs in (0, 1):
+        assert ccl.ccl_set_option(c, ccl.CCL_OPT_USE_GRAPHS, graphs) == ccl.CCL_OK
+        for b in others:
+            assert np.array_equal(gpu_label_batched(c, b), oracle.uf_label_batched(b))
+            out.fill_(-7)
+            g.replay()
+            torch.cuda.synchronize()
+            assert np.array_equal(out.cpu().numpy(), want)
+    del g
+    ccl.ccl_context_destroy(c)
